@@ -27,7 +27,6 @@ struct lamp_ctx {
   lamp_params params{};
   double Hr = 0.0;             // entropy of r
   double log_m = 0.0;
-  int rowblocks = 0;
   int part_width = 3;  // values per point the partial-sum buffers hold (per split)
   std::vector<void*> allocs;
   // owned input copies (lamp_create_owned)
@@ -390,8 +389,6 @@ static int create_impl(lamp_ctx** out, const lamp_problem* prob, const lamp_para
   // workspace
   Work& w = ctx->w;
   const size_t n = (size_t)k.n, m = (size_t)k.m;
-  ctx->rowblocks = (int)fin_blocks(k.n);
-  int colblocks = (int)fin_blocks(k.m);
   // partial-sum width: the sweeps' 2 / 3 values per point, and the gradient's d values;
   // the transport map widens the buffers on first use (ensure_part_width)
   const size_t gradd = k.kind == COST_SQEUCLID ? (size_t)std::min<int64_t>(std::max<int64_t>(k.d, 2), 8) : 2;
@@ -418,11 +415,12 @@ static int create_impl(lamp_ctx** out, const lamp_problem* prob, const lamp_para
   if ((rc = dalloc(ctx, &w.logZ, n))) return bail(rc);
   if ((rc = dalloc(ctx, &w.colA, m))) return bail(rc);
   if ((rc = dalloc(ctx, &w.colz, m))) return bail(rc);
+  if ((rc = dalloc(ctx, &w.gj, m))) return bail(rc);
   if ((rc = dalloc(ctx, &w.rscr, rscr_doubles(k.n, k.m, k.kind == LAMP_COST_SQEUCLID ? (int)k.d : 0)))) return bail(rc);
   if ((rc = dalloc(ctx, &w.nx, n))) return bail(rc);
   if ((rc = dalloc(ctx, &w.ny, m))) return bail(rc);
-  if ((rc = dalloc(ctx, &w.rowred, (size_t)ctx->rowblocks))) return bail(rc);
-  if ((rc = dalloc(ctx, &w.colred, (size_t)colblocks * 3))) return bail(rc);
+  if ((rc = dalloc(ctx, &w.rowred, (size_t)fin_groups(k.n)))) return bail(rc);
+  if ((rc = dalloc(ctx, &w.colred, (size_t)fin_groups(k.m) * 3))) return bail(rc);
   if ((rc = dalloc(ctx, &w.rowmax, (size_t)g.rows_split * 2 * n))) return bail(rc);
   if ((rc = dalloc(ctx, &w.scratch, (size_t)std::max(3 * 4 * g.sms, 3 * 128)))) return bail(rc);
   if ((rc = dalloc(ctx, &w.dev, 1))) return bail(rc);
@@ -601,6 +599,10 @@ static int create_impl(lamp_ctx** out, const lamp_problem* prob, const lamp_para
     k.rnx = k.s * rnx;
   }
 
+  {
+    cudaError_t e = launch_mirror_gain(in, k, w, ctx->stream);
+    if (e != cudaSuccess) return bail(fail(ctx, LAMP_E_CUDA, "mirror gain: %s", cudaGetErrorString(e)));
+  }
   if ((rc = prime(ctx))) return bail(rc);
   {
     cudaError_t e = cudaStreamSynchronize(ctx->stream);
@@ -683,10 +685,10 @@ extern "C" int lamp_solve(lamp_ctx* ctx, lamp_result* out) {
     stop = rule ? LAMP_STOP_INFEAS : LAMP_STOP_MAX_ITER;
   }
   const double rule_res = hd.res;  // the infeasibility the stopping rule saw
-  if (stop != LAMP_STOP_GAP && ctx->k.shared_shift && hd.status == 0) {
-    // the regular iterations of the packed direct-form sweeps leave <C, X^t> out: one
-    // evaluation pass of the final state provides it (its column sums may differ from the
-    // iteration's in the last bits; the result keeps the value the stopping rule used)
+  if (stop != LAMP_STOP_GAP && hd.status == 0) {
+    // the regular iterations leave <C, X^t> and log Z out: one evaluation pass of the final
+    // state provides them (its column sums may differ from the iteration's in the last bits;
+    // the result keeps the value the stopping rule used)
     int rc = evaluate(ctx);
     if (rc) return rc;
     ctx->host_dev->res = rule_res;
@@ -1026,6 +1028,7 @@ extern "C" int lamp_step_host(lamp_ctx* ctx, const float* C_or_x, const float* y
     CK(cudaMemcpyAsync(ctx->own_b, y, (size_t)k.m * k.d * sizeof(float), cudaMemcpyHostToDevice, ctx->stream));
   CK(cudaMemcpyAsync(ctx->own_r, r, k.n * sizeof(double), cudaMemcpyHostToDevice, ctx->stream));
   CK(cudaMemcpyAsync(ctx->own_c, c, k.m * sizeof(double), cudaMemcpyHostToDevice, ctx->stream));
+  CK(launch_mirror_gain(ctx->in, k, ctx->w, ctx->stream));
   const float* px = ctx->own_a;
   const float* py = ctx->own_b;
   if (ctx->pub_kind == LAMP_COST_COSINE) {

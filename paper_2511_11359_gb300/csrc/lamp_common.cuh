@@ -50,11 +50,13 @@ constexpr double kLn2 = 0.69314718055994530942;
 
 enum CostKind : int { COST_DENSE = 0, COST_SQEUCLID = 1 };
 
-// threads per block of the O(n + m) finalize kernels; rowred / colred hold one partial
-// per block.  Their time is the float64 instruction latency of one thread's chain (the
-// FP64 rate of this part is ~1/64 of FP32), so smaller blocks do not make them faster.
+// threads per block of the O(n + m) kernels of the evaluation passes, with one partial per
+// block in rscr
 constexpr int kFinThreads = 128;
 inline int64_t fin_blocks(int64_t len) { return (len + kFinThreads - 1) / kFinThreads; }
+// points per block of the finalize kernels RF and CF; rowred / colred hold their block partials
+constexpr int kFinPoints = 64;
+inline int64_t fin_groups(int64_t len) { return (len + kFinPoints - 1) / kFinPoints; }
 // doubles of Work::rscr: per-block partials of up to 4 + d fields for rows and columns,
 // the reduced fields and the results
 inline size_t rscr_doubles(int64_t n, int64_t m, int d) {
@@ -302,6 +304,7 @@ struct DevState {
   double swf_kap;
   SweepF swf;
   SweepParams spc, spn;
+  SweepParams spq;  // make_sweep_params of kappa_{t+2}, from the row finalize to the column finalize
 };
 
 __host__ __device__ inline SweepF sweep_floats(const SweepParams& p) {
@@ -357,7 +360,9 @@ struct Work {
   float4* colq2[2];
   float4* g2row2;
   double* rowpart;     // [splits_rows][2][n] partial row sums
-  double* colpart;     // [splits_cols][3][m] partial column sums (A, B, cost-weighted A)
+  double* colpart;     // [splits_cols][2][m] partial column sums (A, B); evaluation passes
+                       // [splits_cols][3][m] (A, B, cost-weighted A)
+  double* gj;          // [m] 2 tau2 K / c^alpha_j, the gain of the mirror step
   double* logZ;        // [n] natural-log normalisers of X^t
   double* colA;        // [m] col(X^t)
   double* colz;        // [m] sum_i C_ij X_ij of the last pass that accumulated the cost, without
@@ -409,8 +414,8 @@ cudaError_t launch_prime(const Inputs& in, const Consts& k, const Work& w, const
 // applied (Work::rowmax, stream A slot); the column data's second field holds Br_j
 cudaError_t launch_rowmax_refined(const Inputs& in, const Consts& k, const Work& w, const Geometry& g, int prec,
                                   cudaStream_t st);
-// eval = 1: an evaluation pass, whose column sweep also accumulates <C, X^t> (the
-// packed direct-form column sweep leaves it out of the regular iterations)
+// eval = 1: an evaluation pass (no update): log Z of every row, and a column sweep that also
+// accumulates <C, X^t>; the regular iterations leave both out
 cudaError_t launch_iteration(const Inputs& in, const Consts& k, const Work& w, const Geometry& g, int prec,
                              int eval, cudaStream_t st);
 void prepare_kernels();
@@ -470,6 +475,12 @@ cudaError_t launch_round(const Inputs& in, const Consts& k, const Work& w, const
 // <c, phi>}, with rowmin the row min (eta = 0) or row softmin (eta > 0) of C_ij + 2K phi_j
 cudaError_t launch_dual(const Inputs& in, const Consts& k, const Work& w, const Geometry& g, int prec, int cur,
                         int which, double* out2, cudaStream_t st);
+// finalize kernels (lamp_fin.cu)
+cudaError_t launch_mirror_gain(const Inputs& in, const Consts& k, const Work& w, cudaStream_t st);
+cudaError_t launch_row_fin(const Inputs& in, const Consts& k, const Work& w, const Geometry& g, int eval,
+                           cudaStream_t st);
+cudaError_t launch_col_fin(const Inputs& in, const Consts& k, const Work& w, const Geometry& g, int eval,
+                           cudaStream_t st);
 int launches_per_iteration(const Consts& k, int prec);
 // record a message for lamp_last_error(NULL) (errors raised without a context)
 void set_last_error_null(const char* msg);

@@ -192,8 +192,8 @@ k_dense_tma(const __grid_constant__ CUtensorMap map_c, const Work w, int64_t n, 
           const float zz = tC[a * kTC];
           const float vA = __fmaf_rn(alA, zz, __fmaf_rn(ahA, zz, -(oA + rd.x)));
           const float vB = __fmaf_rn(alB, zz, __fmaf_rn(ahB, zz, -(oB + rd.z)));
-          const float pA = ex2(vA) * rd.y;
-          sA += pA;
+          const float pA = __fmul_rn(ex2(vA), rd.y);
+          sA = __fadd_rn(sA, pA);
           if (WC) sCx = __fmaf_rn(zz, pA, sCx);
           sB = __fmaf_rn(ex2(vB), rd.w, sB);
         }

@@ -8,6 +8,7 @@
 //   CF  column finalize: the O(m) float64 dual step of Alg. 2 (thetabar, nu, thetahat,
 //                     tclip), residual ||col - c||_1, the next sweep's column data; its
 //                     last block reduces the block partials and applies or rejects the update.
+// RF and CF are in lamp_fin.cu.  Only the column sweeps of evaluation passes accumulate <C, X^t>.
 // See lamp_common.cuh for the compensated exponent.
 #include <cfloat>
 #include <cmath>
@@ -88,6 +89,7 @@ struct SweepIO {
   const float4* indat[2];
 };
 
+// M_COLSUM: DG = 1 also accumulates the cost-weighted sums (evaluation passes).
 // M_GRAD accumulates sum_b 2^{v_ab} weight_b V_b[0:DG] with V = Vin (n_in x DG, row-major)
 // when given, else coordinates q0 .. q0 + DG - 1 of the inner points (the gradient)
 template <int MODE, int DG, bool DIFF>
@@ -149,7 +151,8 @@ k_pts_sweep(const float* __restrict__ P_out, const float* __restrict__ P_in, int
 
   const float ahA = sp.ahA, alA = sp.alA, ahB = sp.ahB, alB = sp.alB;
 
-  constexpr int NACC = (MODE == M_COLSUM) ? 3 : 2;
+  constexpr bool WC = MODE == M_COLSUM && DG > 0;
+  constexpr int NACC = WC ? 3 : 2;
   float hi[8][NACC], lo[8][NACC];
   float mx[8][2];
   double gacc[8][DG > 0 ? DG : 1];
@@ -248,15 +251,15 @@ k_pts_sweep(const float* __restrict__ P_out, const float* __restrict__ P_in, int
           if (MODE == M_ROWSUM) {
             sA = __fmaf_rn(eA, dat[b].y, sA);
           } else {
-            const float pA = eA * dat[b].y;
-            sA += pA;
-            sC = __fmaf_rn(zz, pA, sC);
+            const float pA = __fmul_rn(eA, dat[b].y);
+            sA = __fadd_rn(sA, pA);
+            if (WC) sC = __fmaf_rn(zz, pA, sC);
           }
           sB = __fmaf_rn(eB, dat[b].w, sB);
         }
         ff_add(hi[a][0], lo[a][0], sA);
         ff_add(hi[a][1], lo[a][1], sB);
-        if (MODE == M_COLSUM) ff_add(hi[a][NACC - 1], lo[a][NACC - 1], sC);
+        if (WC) ff_add(hi[a][NACC - 1], lo[a][NACC - 1], sC);
       }
     } else if (MODE == M_MAX) {
 #pragma unroll
@@ -485,6 +488,7 @@ k_dense_rows(const float* __restrict__ C, int64_t ldc, int64_t n, int64_t m, con
 
 constexpr int kDColRows = 16;  // rows per step (row data staged in shared memory)
 
+template <int WC>  // 1: an evaluation pass, with the cost-weighted sums
 __global__ void __launch_bounds__(kThreads)
 k_dense_cols(const float* __restrict__ C, int64_t ldc, int64_t n, int64_t m, const Work w, int64_t rows_per_split,
              const Consts k) {
@@ -540,9 +544,9 @@ k_dense_cols(const float* __restrict__ C, int64_t ldc, int64_t n, int64_t m, con
         const float zz = cv[q];
         const float vA = __fmaf_rn(alA, zz, __fmaf_rn(ahA, zz, -(oA[q] + rd.x)));
         const float vB = __fmaf_rn(alB, zz, __fmaf_rn(ahB, zz, -(oB[q] + rd.z)));
-        const float pA = ex2(vA) * rd.y;
-        sA[q] += pA;
-        sC[q] = __fmaf_rn(zz, pA, sC[q]);
+        const float pA = __fmul_rn(ex2(vA), rd.y);
+        sA[q] = __fadd_rn(sA[q], pA);
+        if (WC) sC[q] = __fmaf_rn(zz, pA, sC[q]);
         sB[q] = __fmaf_rn(ex2(vB), rd.w, sB[q]);
       }
     }
@@ -550,15 +554,16 @@ k_dense_cols(const float* __restrict__ C, int64_t ldc, int64_t n, int64_t m, con
     for (int q = 0; q < 4; ++q) {
       ff_add(hiA[q], loA[q], sA[q]);
       ff_add(hiB[q], loB[q], sB[q]);
-      ff_add(hiC[q], loC[q], sC[q]);
+      if (WC) ff_add(hiC[q], loC[q], sC[q]);
     }
   }
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     if (!ok[q]) continue;
-    part[((int64_t)split * 3 + 0) * m + jj[q]] = (double)hiA[q] + (double)loA[q];
-    part[((int64_t)split * 3 + 1) * m + jj[q]] = (double)hiB[q] + (double)loB[q];
-    part[((int64_t)split * 3 + 2) * m + jj[q]] = (double)hiC[q] + (double)loC[q];
+    constexpr int na = WC ? 3 : 2;  // the layout k_col_fin reads for this pass
+    part[((int64_t)split * na + 0) * m + jj[q]] = (double)hiA[q] + (double)loA[q];
+    part[((int64_t)split * na + 1) * m + jj[q]] = (double)hiB[q] + (double)loB[q];
+    if (WC) part[((int64_t)split * na + 2) * m + jj[q]] = (double)hiC[q] + (double)loC[q];
   }
 }
 
@@ -689,224 +694,6 @@ __global__ void k_prime_fin(const Work w, int splits, const Consts k) {
   double qB = isfinite(mB) ? quantize((double)mB, sp.g) : 0.0;
   if (k.shared_shift) qB = qA;
   rowshift[i] = make_float2((float)qA, (float)qB);
-}
-
-// RF: row finalize of iteration t
-__global__ void __launch_bounds__(kFinThreads)
-k_row_fin(const Work w, int splits, const double* __restrict__ r, const Consts k) {
-  DevState* __restrict__ dev = w.dev;
-  if (dev->done) return;
-  const int cur = dev->cur;
-  const double* __restrict__ rowpart = w.rowpart;
-  const double* __restrict__ nx = w.nx;
-  const float2* __restrict__ rs_cur = w.rowshift[cur];
-  float2* __restrict__ rs_nxt = w.rowshift[cur ^ 1];
-  float4* __restrict__ g2row = w.g2row;
-  double* __restrict__ logZ = w.logZ;
-  double* __restrict__ rowred = w.rowred;
-  __shared__ double sred[kFinThreads / 32];
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  double contrib = 0.0;
-  if (i < k.n) {
-    SweepParams sp, spn;
-    iteration_params_of(dev, k, sp, spn);
-    double SA = 0.0, SB = 0.0;
-    // unrolled: the partials' loads are independent and in flight together; the sums keep
-    // the split order
-#pragma unroll 8
-    for (int s = 0; s < splits; ++s) {
-      SA += rowpart[((int64_t)s * 2 + 0) * k.n + i];
-      SB += rowpart[((int64_t)s * 2 + 1) * k.n + i];
-    }
-    const double lim = 1.0e36;
-    if (!(SA > 1.0 / lim && SA < lim && SB > 1.0 / lim && SB < lim)) {
-      atomicExch(&dev->status, 5 /* LAMP_E_NUMERIC */);
-      SA = SA > 0 ? SA : 1.0;
-      SB = SB > 0 ? SB : 1.0;
-    }
-    float2 rq = rs_cur[i];
-    double snx = k.zdot ? k.s * nx[i] : 0.0;
-    // float64 log2 and divisions: with float32 ones (log2f carries an absolute error of
-    // ~2^-22 near 1) the potentials of 100-iteration trajectories drifted from the oracle's
-    // by ~1e-6 instead of ~1e-8, and log Z, which amplifies nu by 2 K kappa, by ~1e-4
-    const double lsA = log2(SA), lsB = log2(SB);
-    double L2A = (double)rq.x - sp.lamA * snx + lsA;  // log2 Z of X^t
-    double L2B = (double)rq.y - sp.lamB * snx + lsB;  // log2 Z of Xbar^{t+1}
-    double lz = kLn2 * L2A;
-    logZ[i] = lz;
-    double ri = r[i];
-    contrib = ri * lz;
-    // the row weights q = r / S, float32 factors of the column sweep
-    const float qa = (float)(ri / SA), qb = (float)(ri / SB);
-    g2row[i] = make_float4(rq.x, qa, rq.y, qb);
-    if (w.g2row2) store_pair_entry(w.g2row2, i, rq.x, qa, 0.f, qb);
-    // shifts of iteration t+1: stream A there has kappa_{t+1} (stream B here);
-    // stream B there is extrapolated linearly in t.
-    double tA = (double)rq.y + lsB;
-    double tB = spn.lamB * snx + 2.0 * L2B - L2A;
-    const float qA = (float)quantize(tA, spn.g);
-    rs_nxt[i] = make_float2(qA, k.shared_shift ? qA : (float)quantize(tB, spn.g));
-  }
-  contrib = warp_sum_d(contrib);
-  int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (lane == 0) sred[wid] = contrib;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double v = 0.0;
-    for (int w = 0; w < kFinThreads / 32; ++w) v += sred[w];
-    rowred[blockIdx.x] = v;
-  }
-}
-
-// CF: column finalize of iteration t, dual step of Alg. 2, and the decision
-__global__ void __launch_bounds__(kFinThreads)
-k_col_fin(const Work w, int splits, const double* __restrict__ cvec, int rowblocks, int with_cost, const Consts k) {
-  DevState* __restrict__ dev = w.dev;
-  if (dev->done) return;
-  const int cur = dev->cur;
-  const double* __restrict__ colpart = w.colpart;
-  const double* __restrict__ ny = w.ny;
-  const float4* __restrict__ colq_cur = w.colq[cur];
-  float4* __restrict__ colq_nxt = w.colq[cur ^ 1];
-  const double* __restrict__ nu_cur = w.nu[cur];
-  const double* __restrict__ th_cur = w.theta[cur];
-  double* __restrict__ nu_nxt = w.nu[cur ^ 1];
-  double* __restrict__ th_nxt = w.theta[cur ^ 1];
-  double* __restrict__ colA = w.colA;
-  double* __restrict__ colred = w.colred;
-  const double* __restrict__ rowred = w.rowred;
-  __shared__ double sred[4][kFinThreads / 32];
-  __shared__ bool amLast;
-  int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  double res = 0.0, cost = 0.0, cnu = 0.0;
-  SweepParams sp, spn;
-  iteration_params_of(dev, k, sp, spn);
-  const int eval_only = dev->eval_only;
-  if (j < k.m) {
-    double aA = 0.0, aB = 0.0, aC = 0.0;
-    // partials of split s: [s][3][m] with the cost-weighted sums, [s][2][m] without
-    const int na = with_cost ? 3 : 2;
-    // unrolled: the partials' loads are independent and in flight together; the sums keep
-    // the split order
-#pragma unroll 8
-    for (int s = 0; s < splits; ++s) {
-      aA += colpart[((int64_t)s * na + 0) * k.m + j];
-      aB += colpart[((int64_t)s * na + 1) * k.m + j];
-      if (with_cost) aC += colpart[((int64_t)s * na + 2) * k.m + j];
-    }
-    float4 cq = colq_cur[j];
-    const double A = (double)cq.y * aA;  // col(X^t)_j
-    // col(Xbar^{t+1})_j; under the shared row shift the column weight of stream B is
-    // already inside the sweep's exponents
-    const double B = k.shared_shift ? aB : (double)cq.w * aB;
-    const double zsum = (double)cq.y * aC;
-    if (!k.zdot) {
-      cost = k.s * zsum;
-    } else {
-      cost = k.s * ny[j] * A - 2.0 * k.s * zsum;  // + sum_i r_i s|x_i|^2 added once below
-    }
-    const double cj = cvec[j];
-    const double nuj = nu_cur[j], thj = th_cur[j];
-    res = fabs(A - cj);
-    cnu = A * nuj;
-    colA[j] = A;
-    if (with_cost && w.colz) w.colz[j] = cost;
-    if (!eval_only) {
-      // the dual mirror steps (Eq. def:closed_form_opt) tanh(g (col - c) + atanh theta), in
-      // float64 through the addition theorem tanh(u + atanh theta) = (tanh u + theta) /
-      // (1 + theta tanh u): one tanh per stream and no atanh (|theta^t| <= tanh(beta/2) < 1,
-      // so the denominator is at least 1 - tanh(beta/2))
-      const double ca = cj + k.alpha_m;                  // c^alpha (Section 3.1)
-      const double gj = 2.0 * k.tau2 * k.K / ca;
-      const double wt = sp.wB;                           // tau1 eta_{t+1}
-      const double tA = tanh(gj * (A - cj));
-      const double thbar = (tA + thj) / fma(tA, thj, 1.0);  // M_{tau2}(theta^t; p^{eta_t}(nu^t))
-      const double nun = nuj + wt * (thbar - nuj);       // nu^{t+1}
-      const double tB = tanh(gj * (B - cj));
-      const double thhat = (tB + thj) / fma(tB, thj, 1.0);  // M_{tau2}(theta^t; p^{eta_{t+1}}(nubar^{t+1}))
-      const double thn = fmin(fmax(thhat, -k.clipb), k.clipb);  // tclip
-      nu_nxt[j] = nun;
-      th_nxt[j] = thn;
-      // column data of iteration t+1
-      const double wn = spn.wB;
-      const double nbn = nun + wn * (thn - nun);         // nubar^{t+2}
-      const double sny = k.zdot ? k.s * ny[j] : 0.0;
-      float dB;
-      const float4 cd = column_data(nun, nbn, sny, spn, k, &dB);
-      colq_nxt[j] = cd;
-      if (w.colq2[cur ^ 1]) store_pair_entry(w.colq2[cur ^ 1], j, cd.x, cd.y, dB, cd.w);
-    }
-  }
-  res = warp_sum_d(res);
-  cost = warp_sum_d(cost);
-  cnu = warp_sum_d(cnu);
-  int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (lane == 0) { sred[0][wid] = res; sred[1][wid] = cost; sred[2][wid] = cnu; }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double a = 0.0, b = 0.0, c = 0.0;
-    for (int w = 0; w < kFinThreads / 32; ++w) { a += sred[0][w]; b += sred[1][w]; c += sred[2][w]; }
-    colred[3 * blockIdx.x + 0] = a;
-    colred[3 * blockIdx.x + 1] = b;
-    colred[3 * blockIdx.x + 2] = c;
-    __threadfence();
-    unsigned int tk = atomicAdd(&dev->ticket, 1u);
-    amLast = (tk == gridDim.x - 1);
-  }
-  __syncthreads();
-  if (!amLast) return;
-  // last block: reduce all partials in a fixed order (thread t takes blocks t, t + 128, ..,
-  // then a fixed tree over the threads) and decide
-  __threadfence();
-  double R = 0.0, Cx = 0.0, Cn = 0.0, RL = 0.0;
-  for (unsigned int b = threadIdx.x; b < gridDim.x; b += blockDim.x) {
-    R += ((volatile double*)colred)[3 * b + 0];
-    Cx += ((volatile double*)colred)[3 * b + 1];
-    Cn += ((volatile double*)colred)[3 * b + 2];
-  }
-  for (int b = threadIdx.x; b < rowblocks; b += blockDim.x) RL += ((volatile const double*)rowred)[b];
-  R = warp_sum_d(R);
-  Cx = warp_sum_d(Cx);
-  Cn = warp_sum_d(Cn);
-  RL = warp_sum_d(RL);
-  __syncthreads();  // sred is reused
-  if (lane == 0) { sred[0][wid] = R; sred[1][wid] = Cx; sred[2][wid] = Cn; sred[3][wid] = RL; }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    R = Cx = Cn = RL = 0.0;
-    for (int w = 0; w < kFinThreads / 32; ++w) { R += sred[0][w]; Cx += sred[1][w]; Cn += sred[2][w]; RL += sred[3][w]; }
-    Cx += k.rnx;
-    dev->ticket = 0u;
-    dev->res = R;
-    dev->costA = with_cost ? Cx : NAN;
-    dev->colnu = Cn;
-    dev->rlogZ = RL;
-    dev->t_eval = dev->t;
-    dev->kappa_eval = dev->kappa;
-    if (dev->status != 0 || !isfinite(R)) {
-      if (dev->status == 0) dev->status = 5;
-      dev->done = 1;
-    } else if (eval_only) {
-      dev->done = 1;
-    } else if ((dev->t >= 1 && R <= dev->tol &&
-                (k.eta == 0.0 || k.infeas_only || 1.0 - dev->kappa * k.eta <= dev->tol)) ||
-               dev->t >= dev->tmax) {
-      dev->done = 1;
-    } else {
-      dev->t = dev->t + 1;
-      dev->kappa = sp.kapB;
-      dev->cur ^= 1;
-      if (k.kap_ovr < 0.0 && !k.same_kappa) {
-        // the next iteration's parameters, once per iteration instead of once per thread
-        // (float64 is slow on this part)
-        dev->spc = spn;
-        dev->spn = make_sweep_params(spn.kapB, k);
-        dev->swf = sweep_floats(spn);
-        dev->swf_kap = spn.kapA;
-      }
-    }
-    __threadfence();
-  }
 }
 
 // gradient finalize of coordinates q0 .. q0 + dg - 1 (partials hold dg values per point):
@@ -1061,14 +848,15 @@ static cudaError_t launch_row_sweep(const Inputs& in, const Consts& k, const Wor
 
 static cudaError_t launch_col_sweep(const Inputs& in, const Consts& k, const Work& w, const Geometry& g, int eval,
                                     cudaStream_t st) {
-  // stored costs accumulate <C, X^t> in every iteration (the column finalize reads three
-  // partials per split whenever the row shift is not shared)
-  if (k.kind == COST_DENSE && g.map_c) return dense_launch_sweep(false, 1, g, w, k, g.cols_split, st);
+  if (k.kind == COST_DENSE && g.map_c) return dense_launch_sweep(false, eval, g, w, k, g.cols_split, st);
   if (k.kind == COST_DENSE) {
     int64_t rps = cdiv(k.n, g.cols_split);
     rps = cdiv(rps, kDColRows) * kDColRows;
     dim3 grid((unsigned)cdiv(k.m, kDChunk), (unsigned)g.cols_split);
-    k_dense_cols<<<grid, kThreads, 0, st>>>(in.C, in.ldc, k.n, k.m, w, rps, k);
+    if (eval)
+      k_dense_cols<1><<<grid, kThreads, 0, st>>>(in.C, in.ldc, k.n, k.m, w, rps, k);
+    else
+      k_dense_cols<0><<<grid, kThreads, 0, st>>>(in.C, in.ldc, k.n, k.m, w, rps, k);
     return cudaGetLastError();
   }
   if (k.shared_shift) return launch_direct_sweep(false, eval, in, k, w, g, st);
@@ -1078,6 +866,8 @@ static cudaError_t launch_col_sweep(const Inputs& in, const Consts& k, const Wor
     io.off4[b] = w.colq[b];
     io.indat[b] = w.g2row;
   }
+  if (eval)
+    return launch_pts<M_COLSUM, 1>(in.y, in.x, k.m, k.n, k.d, io, w.colpart, nullptr, g.cols_split, w.dev, k, st);
   return launch_pts<M_COLSUM, 0>(in.y, in.x, k.m, k.n, k.d, io, w.colpart, nullptr, g.cols_split, w.dev, k, st);
 }
 
@@ -1100,23 +890,18 @@ cudaError_t launch_rowmax_refined(const Inputs& in, const Consts& k, const Work&
 
 cudaError_t launch_iteration_part(const Inputs& in, const Consts& k, const Work& w, const Geometry& g, int prec,
                                   int part, int eval, cudaStream_t st) {
-  const int rb = (int)fin_blocks(k.n);
   const bool tcpath = prec == 1 /* LAMP_PREC_BF16_TC */;
   switch (part) {
     case 0:
       if (tcpath) return tc_launch_sweep(true, 0, g, w, k, g.rows_split, st);
       return launch_row_sweep(in, k, w, g, M_ROWSUM, st);
     case 1:
-      k_row_fin<<<rb, kFinThreads, 0, st>>>(w, g.rows_split, in.r, k);
-      return cudaGetLastError();
+      return launch_row_fin(in, k, w, g, eval, st);
     case 2:
       if (tcpath) return tc_launch_sweep(false, eval, g, w, k, g.cols_split, st);
       return launch_col_sweep(in, k, w, g, eval, st);
     default:
-      // the packed direct-form column sweep accumulates <C, X> in evaluation passes only
-      k_col_fin<<<(unsigned)fin_blocks(k.m), kFinThreads, 0, st>>>(w, g.cols_split, in.c, rb,
-                                                                    eval || !k.shared_shift, k);
-      return cudaGetLastError();
+      return launch_col_fin(in, k, w, g, eval, st);
   }
 }
 
@@ -1144,6 +929,7 @@ void prepare_kernels() {
   if (done) return;
   set_attr<M_ROWSUM, 0>();
   set_attr<M_COLSUM, 0>();
+  set_attr<M_COLSUM, 1>();
   set_attr<M_MAX, 0>();
   set_attr<M_MAX2, 0>();
   set_attr<M_KMAX, 0>();
@@ -1164,12 +950,12 @@ int sweep_blocks_per_sm(const Consts& k, int prec, int which) {
     if (which == 0)
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_dense_rows<M_ROWSUM>, kThreads, 0);
     else
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_dense_cols, kThreads, 0);
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_dense_cols<1>, kThreads, 0);
   } else if (uses_direct_sweeps(k, prec)) {
     nb = direct_blocks_per_sm();
   } else {
     auto kern = which == 0 ? (k.zdot ? k_pts_sweep<M_ROWSUM, 0, false> : k_pts_sweep<M_ROWSUM, 0, true>)
-                           : (k.zdot ? k_pts_sweep<M_COLSUM, 0, false> : k_pts_sweep<M_COLSUM, 0, true>);
+                           : (k.zdot ? k_pts_sweep<M_COLSUM, 1, false> : k_pts_sweep<M_COLSUM, 1, true>);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, kThreads, pts_smem(k.d));
   }
   return nb > 0 ? nb : 1;

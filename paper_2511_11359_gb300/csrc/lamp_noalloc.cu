@@ -217,8 +217,12 @@ extern "C" int lamp_marginals_noalloc(const lamp_problem* prob, double K, double
   w.colpart = cv.take<double>((size_t)g.cols_split * 3 * m);
   w.nx = cv.take<double>(n);
   w.ny = cv.take<double>(m);
-  w.rowred = cv.take<double>((size_t)fin_blocks(k.n));
-  w.colred = cv.take<double>(3 * (size_t)fin_blocks(k.m));
+  cv.take<double>((size_t)fin_blocks(k.n));  // reserved: what a request needs stays as it was
+  cv.take<double>(3 * (size_t)fin_blocks(k.m));
+  // an evaluation pass updates neither nu nor the row shifts: their second buffers hold the
+  // finalize kernels' block partials (every part of the workspace has at least 32 doubles)
+  w.rowred = reinterpret_cast<double*>(w.rowshift[1]);
+  w.colred = w.nu[1];
   w.rowmax = cv.take<float>((size_t)g.rows_split * 2 * n);
   w.scratch = cv.take<double>(1);
   w.dev = cv.take<DevState>(1);
