@@ -63,6 +63,10 @@ struct lamp_ctx {
   size_t tcg_part_floats = 0;
   cudaStream_t gside = nullptr;  // the gradient's second side runs on this stream
   cudaEvent_t gfork = nullptr, gjoin = nullptr;
+  // partial sums of the float32 gradient and of the transport map
+  double* gpart = nullptr;
+  size_t gpart_doubles = 0;
+  bool dot_fresh = false;  // the transposed copies w.xt, w.yt match the current points
   alignas(64) unsigned char map_xT[128];
   alignas(64) unsigned char map_yT[128];
   std::string err;
@@ -101,6 +105,24 @@ static int dalloc(lamp_ctx* ctx, T** p, size_t count) {
                                     cudaGetErrorString(e));
   ctx->allocs.push_back(q);
   *p = reinterpret_cast<T*>(q);
+  return LAMP_OK;
+}
+
+// the transposed copies of the points that the float32 dot-form kernels read, (re)made from the
+// points the context solves with
+static int ensure_dot_copies(lamp_ctx* ctx) {
+  const Consts& k = ctx->k;
+  int rc;
+  if (!ctx->w.xt) {
+    if ((rc = dalloc(ctx, &ctx->w.xt, (size_t)dot_pad(k.n) * k.d))) return rc;
+    if ((rc = dalloc(ctx, &ctx->w.yt, (size_t)dot_pad(k.m) * k.d))) return rc;
+    ctx->dot_fresh = false;
+  }
+  if (!ctx->dot_fresh) {
+    CK(dot_transpose(ctx->in.x, k.n, k.d, ctx->w.xt, ctx->stream));
+    CK(dot_transpose(ctx->in.y, k.m, k.d, ctx->w.yt, ctx->stream));
+    ctx->dot_fresh = true;
+  }
   return LAMP_OK;
 }
 
@@ -520,6 +542,8 @@ static int create_impl(lamp_ctx** out, const lamp_problem* prob, const lamp_para
     g.map_y64 = ctx->map_y64;
   }
 
+  if (k.zdot && ctx->prec == LAMP_PREC_FP32 && (rc = ensure_dot_copies(ctx))) return bail(rc);
+
   // cost scale and K = ||C||_inf of the cost the kernels use
   {
     cudaError_t e = launch_norms(in, k, w, ctx->stream);
@@ -788,16 +812,50 @@ static int ensure_part_width(lamp_ctx* ctx, int width) {
   return LAMP_OK;
 }
 
+static inline int64_t cdiv64(int64_t a, int64_t b) { return (a + b - 1) / b; }
+
+// inner splits of the dot-form gradient pass: one CTA per SM, and each split writes a partial
+// sum per output (1 % of a wave each)
+static int dot_splits(const lamp_ctx* ctx, bool rows) {
+  const int64_t out = cdiv64(rows ? ctx->k.n : ctx->k.m, dot_tile()), in = cdiv64(rows ? ctx->k.m : ctx->k.n, dot_tile());
+  return choose_split(out, in, ctx->g.sms, 4, 0.01);
+}
+
+// room for `doubles` partial sums of the float32 gradient and transport-map passes
+static int ensure_gpart(lamp_ctx* ctx, size_t doubles) {
+  if (doubles <= ctx->gpart_doubles) return LAMP_OK;
+  if (ctx->gpart) {
+    CK(cudaStreamSynchronize(ctx->stream));
+    auto it = std::find(ctx->allocs.begin(), ctx->allocs.end(), (void*)ctx->gpart);
+    if (it != ctx->allocs.end()) ctx->allocs.erase(it);
+    cudaFree(ctx->gpart);
+    ctx->gpart = nullptr;
+    ctx->gpart_doubles = 0;
+  }
+  int rc = dalloc(ctx, &ctx->gpart, doubles);
+  if (rc) return rc;
+  ctx->gpart_doubles = doubles;
+  return LAMP_OK;
+}
+
 extern "C" int lamp_apply_map(lamp_ctx* ctx, const float* V, int64_t k, float* out, int side) {
   if (!ctx || !V || !out) return fail(ctx, LAMP_E_INVALID, "lamp_apply_map: null argument");
   if (k < 1 || k > 8) return fail(ctx, LAMP_E_INVALID, "lamp_apply_map: 1 <= k <= 8 value columns (got %lld)",
                                   (long long)k);
   if (side != 0 && side != 1) return fail(ctx, LAMP_E_INVALID, "lamp_apply_map: side must be 0 (p V) or 1 (p^T U)");
-  int rc = ensure_part_width(ctx, (int)k);
+  int rc, splits = 0;
+  if (ctx->k.zdot) {
+    if ((rc = ensure_dot_copies(ctx))) return rc;
+    splits = dot_splits(ctx, side == 0);
+    rc = ensure_gpart(ctx, (size_t)splits * (side == 0 ? ctx->k.n : ctx->k.m) * k);
+  } else {
+    rc = ensure_part_width(ctx, (int)k);
+  }
   if (rc) return rc;
   rc = evaluate(ctx);
   if (rc) return rc;
-  CK(launch_map(ctx->in, ctx->k, ctx->w, ctx->g, ctx->host_dev->cur, V, (int)k, out, side, ctx->stream));
+  CK(launch_map(ctx->in, ctx->k, ctx->w, ctx->g, ctx->host_dev->cur, V, (int)k, out, side, splits, ctx->gpart,
+                ctx->stream));
   return LAMP_OK;
 }
 
@@ -874,8 +932,6 @@ static int objective_values(lamp_ctx* ctx, double* out) {
   return LAMP_OK;
 }
 
-static inline int64_t cdiv64(int64_t a, int64_t b) { return (a + b - 1) / b; }
-
 // the envelope gradient on tensor cores: one fused recompute pass per side (S = x.y^T by
 // MMA, P = 2^v w in the epilogue, P.Y by a second MMA), then a float-float finalize
 static int grad_tc(lamp_ctx* ctx, float* dx, float* dy) {
@@ -945,12 +1001,25 @@ static int grad_tc(lamp_ctx* ctx, float* dx, float* dy) {
   return LAMP_OK;
 }
 
+// the envelope gradient in float32 for d > 8: one pass per side with all coordinates
+static int grad_dot(lamp_ctx* ctx, float* dx, float* dy) {
+  const Consts& k = ctx->k;
+  const int sx = dot_splits(ctx, true), sy = dot_splits(ctx, false);
+  int rc = ensure_gpart(ctx, std::max(dx ? (size_t)sx * k.n : 0, dy ? (size_t)sy * k.m : 0) * k.d);
+  if (rc) return rc;
+  if ((rc = evaluate_if_stale(ctx))) return rc;
+  const int cur = ctx->host_dev->cur;
+  if (dx) CK(dot_grad(true, ctx->in, ctx->w, k, cur, sx, ctx->gpart, dx, ctx->stream));
+  if (dy) CK(dot_grad(false, ctx->in, ctx->w, k, cur, sy, ctx->gpart, dy, ctx->stream));
+  return LAMP_OK;
+}
+
 extern "C" int lamp_grad(lamp_ctx* ctx, float* dx, float* dy) {
   if (!ctx) return fail(nullptr, LAMP_E_INVALID, "lamp_grad: null context");
   if (ctx->pub_kind != LAMP_COST_SQEUCLID) return fail(ctx, LAMP_E_UNSUPPORTED, "lamp_grad needs LAMP_COST_SQEUCLID");
   if (ctx->prec == LAMP_PREC_BF16_TC) return grad_tc(ctx, dx, dy);
-  // d > 8: the gradient is computed in chunks of 8 coordinates (partials of 8 values per point)
-  int rc = ensure_part_width(ctx, std::min<int>((int)ctx->k.d, 8));
+  if (ctx->k.zdot) return grad_dot(ctx, dx, dy);
+  int rc = ensure_part_width(ctx, (int)ctx->k.d);
   if (rc) return rc;
   rc = evaluate_if_stale(ctx);
   if (rc) return rc;
@@ -1044,6 +1113,11 @@ extern "C" int lamp_step_host(lamp_ctx* ctx, const float* C_or_x, const float* y
     CK(tc_convert(px, k.n, k.d, ctx->xr, ctx->xb, ctx->stream));
     CK(tc_convert(py, k.m, k.d, ctx->yr, ctx->yb, ctx->stream));
     ctx->tcg_fresh = false;  // the gradient pass transposes the new points on its next call
+  }
+  ctx->dot_fresh = false;
+  if (k.zdot && ctx->prec == LAMP_PREC_FP32) {
+    int e = ensure_dot_copies(ctx);
+    if (e) return e;
   }
   int rc = lamp_iterate(ctx, iters);
   if (rc) return rc;

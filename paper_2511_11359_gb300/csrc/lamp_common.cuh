@@ -372,6 +372,8 @@ struct Work {
   double* ny;          // [m] |y_j|^2 (SQEUCLID)
   double* rowred;      // [rowfin blocks] partial <r, log Z>
   double* colred;      // [colfin blocks][3] partial (res, cost, colnu)
+  float* xt;           // [d][dot_pad(n)], [d][dot_pad(m)]: transposed copies of the points, zero padded
+  float* yt;           // (float32 dot-form sweeps and gradient; null elsewhere)
   float* rowmax;       // [splits_rows][2][n] partial row maxima (prime pass)
   double* scratch;     // small reduction scratch (K pass, marginal checks)
   DevState* dev;
@@ -464,9 +466,10 @@ int tile_outer_cols(const Consts& k, int prec);
 int tile_inner_cols(const Consts& k, int prec);
 cudaError_t launch_grad(const Inputs& in, const Consts& k, const Work& w, const Geometry& g, int prec,
                         float* dx, float* dy, cudaStream_t st);
-// transport-map application (lamp_kernels.cu): out = p V (side 0) or p^T U (side 1), 1 <= dk <= 8
+// transport-map application (lamp_kernels.cu): out = p V (side 0) or p^T U (side 1), 1 <= dk <= 8;
+// dot-form costs: sums per `splits` inner splits in `part` (splits x outer points x dk)
 cudaError_t launch_map(const Inputs& in, const Consts& k, const Work& w, const Geometry& g, int cur, const float* V,
-                       int dk, float* out, int side, cudaStream_t st);
+                       int dk, float* out, int side, int splits, double* part, cudaStream_t st);
 // evaluation passes (lamp_eval.cu); `cur` is the state-buffer parity, read by the host beforehand.
 // Round: out4 (device, 4 doubles) = {<C, Round(X^t)>, ||delta_r||_1, ||delta_c||_1, <C, X''>}
 cudaError_t launch_round(const Inputs& in, const Consts& k, const Work& w, const Geometry& g, int prec, int cur,
@@ -475,6 +478,17 @@ cudaError_t launch_round(const Inputs& in, const Consts& k, const Work& w, const
 // <c, phi>}, with rowmin the row min (eta = 0) or row softmin (eta > 0) of C_ij + 2K phi_j
 cudaError_t launch_dual(const Inputs& in, const Consts& k, const Work& w, const Geometry& g, int prec, int cur,
                         int which, double* out2, cudaStream_t st);
+// float32 dot-form sweeps (lamp_dot.cu)
+enum DotMode : int { kDotRowSum, kDotColSum, kDotColSumCost, kDotMax, kDotMax2, kDotKmax };
+int64_t dot_pad(int64_t np);
+cudaError_t dot_transpose(const float* P, int64_t np, int d, float* out, cudaStream_t st);
+void dot_prepare();
+int dot_tile();
+cudaError_t dot_launch(int mode, const Work& w, const Consts& k, const Geometry& g, cudaStream_t st);
+cudaError_t dot_weighted(bool rows, const Work& w, const Consts& k, const float* values, int dv, const float4* off,
+                         const float4* dat, int splits, double* part, cudaStream_t st);
+cudaError_t dot_grad(bool rows, const Inputs& in, const Work& w, const Consts& k, int cur, int splits, double* part,
+                     float* out, cudaStream_t st);
 // finalize kernels (lamp_fin.cu)
 cudaError_t launch_mirror_gain(const Inputs& in, const Consts& k, const Work& w, cudaStream_t st);
 cudaError_t launch_row_fin(const Inputs& in, const Consts& k, const Work& w, const Geometry& g, int eval,

@@ -92,7 +92,7 @@ struct SweepIO {
 // M_COLSUM: DG = 1 also accumulates the cost-weighted sums (evaluation passes).
 // M_GRAD accumulates sum_b 2^{v_ab} weight_b V_b[0:DG] with V = Vin (n_in x DG, row-major)
 // when given, else coordinates q0 .. q0 + DG - 1 of the inner points (the gradient)
-template <int MODE, int DG, bool DIFF>
+template <int MODE, int DG>
 __global__ void __launch_bounds__(kThreads, MODE == M_GRAD ? 1 : 2)
 k_pts_sweep(const float* __restrict__ P_out, const float* __restrict__ P_in, int64_t n_out, int64_t n_in, int d,
             const SweepIO io, double* __restrict__ part, float* __restrict__ pmax, int tiles_per_split,
@@ -204,7 +204,7 @@ k_pts_sweep(const float* __restrict__ P_out, const float* __restrict__ P_in, int
       float4 b1 = *reinterpret_cast<const float4*>(&sIn[kk * kPT + 64 + tx * 4]);
       float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
       float bv[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-      if (DIFF) {
+      {
         // the ground cost of the direct form (Consts::cost_op; uniform branch)
         if (k.cost_op == 0) {
 #pragma unroll
@@ -225,11 +225,6 @@ k_pts_sweep(const float* __restrict__ P_out, const float* __restrict__ P_in, int
 #pragma unroll
             for (int b = 0; b < 8; ++b) z[a][b] = fmaxf(z[a][b], fabsf(av[a] - bv[b]));
         }
-      } else {
-#pragma unroll
-        for (int a = 0; a < 8; ++a)
-#pragma unroll
-          for (int b = 0; b < 8; ++b) z[a][b] = __fmaf_rn(av[a], bv[b], z[a][b]);
       }
     }
 
@@ -281,13 +276,13 @@ k_pts_sweep(const float* __restrict__ P_out, const float* __restrict__ P_in, int
           mx[a][0] = fmaxf(mx[a][0], u);
         }
     } else if (MODE == M_KMAX) {
-      // unscaled squared distance |x|^2 + |y|^2 - 2 x.y in float32; oA holds |x_o|^2
+      // the unscaled cost
 #pragma unroll
       for (int a = 0; a < 8; ++a)
 #pragma unroll
         for (int b = 0; b < 8; ++b) {
           const bool pad = (dat[b].x == -INFINITY);
-          const float dd = DIFF ? z[a][b] : __fmaf_rn(-2.0f, z[a][b], oA[a] + dat[b].x);
+          const float dd = z[a][b];
           mx[a][0] = fmaxf(mx[a][0], pad ? -INFINITY : dd);
           mx[a][1] = fmaxf(mx[a][1], pad ? -INFINITY : -dd);
         }
@@ -750,7 +745,7 @@ template <int MODE, int DG>
 static cudaError_t launch_pts(const float* Pout, const float* Pin, int64_t nout, int64_t nin, int d, const SweepIO& io,
                               double* part, float* pmax, int splits, const DevState* dev, const Consts& k,
                               cudaStream_t st, const float* V = nullptr, int q0 = 0) {
-  auto kern = k.zdot ? k_pts_sweep<MODE, DG, false> : k_pts_sweep<MODE, DG, true>;
+  auto kern = k_pts_sweep<MODE, DG>;
   size_t sm = pts_smem(d, V ? DG : 0);
   int64_t tin = cdiv(nin, kPT);
   int tps = (int)cdiv(tin, splits);
@@ -801,6 +796,12 @@ cudaError_t launch_kmax(const Inputs& in, const Consts& k, const Work& w, const 
     w2.colq2[0] = w2.colq2[1] = w.colq2[1];
     return tc_launch_rowmax(3, g, w2, k, g.rows_split, st);
   }
+  if (w.xt) {
+    Work w2 = w;
+    w2.rowshift[0] = w2.rowshift[1] = w.rowshift[1];
+    w2.colq[0] = w2.colq[1] = w.colq[1];
+    return dot_launch(kDotKmax, w2, k, g, st);
+  }
   // rowmax[split][0][n] = max_j D_ij, rowmax[split][1][n] = max_j -D_ij, D = |x|^2 + |y|^2 - 2 x.y
   return launch_pts<M_KMAX, 0>(in.x, in.y, k.n, k.m, k.d, io_same(w.rowshift[1], nullptr, w.colq[1]), nullptr,
                                w.rowmax, g.rows_split, w.dev, k, st);
@@ -833,6 +834,7 @@ static cudaError_t launch_row_sweep(const Inputs& in, const Consts& k, const Wor
     return cudaGetLastError();
   }
   if (mode == M_ROWSUM && k.shared_shift) return launch_direct_sweep(true, 0, in, k, w, g, st);
+  if (k.zdot) return dot_launch(mode == M_ROWSUM ? kDotRowSum : mode == M_MAX2 ? kDotMax2 : kDotMax, w, k, g, st);
   SweepIO io;
   for (int b = 0; b < 2; ++b) {
     io.off2[b] = w.rowshift[b];
@@ -860,6 +862,7 @@ static cudaError_t launch_col_sweep(const Inputs& in, const Consts& k, const Wor
     return cudaGetLastError();
   }
   if (k.shared_shift) return launch_direct_sweep(false, eval, in, k, w, g, st);
+  if (k.zdot) return dot_launch(eval ? kDotColSumCost : kDotColSum, w, k, g, st);
   SweepIO io;
   for (int b = 0; b < 2; ++b) {
     io.off2[b] = nullptr;
@@ -919,8 +922,7 @@ int launches_per_iteration(const Consts& k, int prec) { return 4; }
 template <int MODE, int DG>
 static void set_attr() {
   const int sm = (int)pts_smem(64, DG);
-  cudaFuncSetAttribute(k_pts_sweep<MODE, DG, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-  cudaFuncSetAttribute(k_pts_sweep<MODE, DG, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+  cudaFuncSetAttribute(k_pts_sweep<MODE, DG>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
 }
 
 // raise the dynamic shared-memory limit of every sweep instantiation once, before any capture
@@ -941,6 +943,7 @@ void prepare_kernels() {
   set_attr<M_GRAD, 6>();
   set_attr<M_GRAD, 7>();
   set_attr<M_GRAD, 8>();
+  dot_prepare();
   done = true;
 }
 
@@ -954,8 +957,10 @@ int sweep_blocks_per_sm(const Consts& k, int prec, int which) {
   } else if (uses_direct_sweeps(k, prec)) {
     nb = direct_blocks_per_sm();
   } else {
-    auto kern = which == 0 ? (k.zdot ? k_pts_sweep<M_ROWSUM, 0, false> : k_pts_sweep<M_ROWSUM, 0, true>)
-                           : (k.zdot ? k_pts_sweep<M_COLSUM, 1, false> : k_pts_sweep<M_COLSUM, 1, true>);
+    // the splits of the dot form are those of two CTAs per SM too: they decide how the float32
+    // partial sums are grouped, and its persistent sweep takes any number of them
+    if (k.zdot) return 2;
+    auto kern = which == 0 ? k_pts_sweep<M_ROWSUM, 0> : k_pts_sweep<M_COLSUM, 1>;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, kThreads, pts_smem(k.d));
   }
   return nb > 0 ? nb : 1;
@@ -1134,7 +1139,7 @@ k_dense_map_cols(const float* __restrict__ C, int64_t ldc, int64_t n, int64_t m,
 
 template <int DK>
 static cudaError_t launch_map_k(const Inputs& in, const Consts& k, const Work& w, const Geometry& g, int cur,
-                                const float* V, float* out, int side, cudaStream_t st) {
+                                const float* V, float* out, int side, int splits, double* part, cudaStream_t st) {
   if (k.kind == COST_DENSE) {
     if (side == 0)
       k_dense_map_rows<DK><<<(unsigned)cdiv(k.n, kThreads / 32), kThreads, 0, st>>>(
@@ -1142,6 +1147,20 @@ static cudaError_t launch_map_k(const Inputs& in, const Consts& k, const Work& w
     else
       k_dense_map_cols<DK><<<(unsigned)cdiv(k.m, kThreads), kThreads, 0, st>>>(
           in.C, in.ldc, k.n, k.m, w.colq[cur], w.g2row, in.r, V, out, w.dev, k);
+    return cudaGetLastError();
+  }
+  if (k.zdot) {
+    const float4* inner = w.colq[cur];
+    if (side == 1) {
+      float4* rw = reinterpret_cast<float4*>(w.rowpart);
+      k_map_rowweights<<<(unsigned)cdiv(k.n, 256), 256, 0, st>>>(w.g2row, in.r, k.n, rw);
+      inner = rw;
+    }
+    const float4* outer = side == 0 ? w.g2row : w.colq[cur];
+    const int64_t np = side == 0 ? k.n : k.m;
+    cudaError_t e = dot_weighted(side == 0, w, k, V, DK, outer, inner, splits, part, st);
+    if (e != cudaSuccess) return e;
+    k_map_fin<<<(unsigned)cdiv(np, 256), 256, 0, st>>>(part, splits, np, DK, outer, side == 0 ? in.r : nullptr, out);
     return cudaGetLastError();
   }
   if (side == 0) {
@@ -1167,16 +1186,16 @@ static cudaError_t launch_map_k(const Inputs& in, const Consts& k, const Work& w
 }
 
 cudaError_t launch_map(const Inputs& in, const Consts& k, const Work& w, const Geometry& g, int cur, const float* V,
-                       int dk, float* out, int side, cudaStream_t st) {
+                       int dk, float* out, int side, int splits, double* part, cudaStream_t st) {
   switch (dk) {
-    case 1: return launch_map_k<1>(in, k, w, g, cur, V, out, side, st);
-    case 2: return launch_map_k<2>(in, k, w, g, cur, V, out, side, st);
-    case 3: return launch_map_k<3>(in, k, w, g, cur, V, out, side, st);
-    case 4: return launch_map_k<4>(in, k, w, g, cur, V, out, side, st);
-    case 5: return launch_map_k<5>(in, k, w, g, cur, V, out, side, st);
-    case 6: return launch_map_k<6>(in, k, w, g, cur, V, out, side, st);
-    case 7: return launch_map_k<7>(in, k, w, g, cur, V, out, side, st);
-    case 8: return launch_map_k<8>(in, k, w, g, cur, V, out, side, st);
+    case 1: return launch_map_k<1>(in, k, w, g, cur, V, out, side, splits, part, st);
+    case 2: return launch_map_k<2>(in, k, w, g, cur, V, out, side, splits, part, st);
+    case 3: return launch_map_k<3>(in, k, w, g, cur, V, out, side, splits, part, st);
+    case 4: return launch_map_k<4>(in, k, w, g, cur, V, out, side, splits, part, st);
+    case 5: return launch_map_k<5>(in, k, w, g, cur, V, out, side, splits, part, st);
+    case 6: return launch_map_k<6>(in, k, w, g, cur, V, out, side, splits, part, st);
+    case 7: return launch_map_k<7>(in, k, w, g, cur, V, out, side, splits, part, st);
+    case 8: return launch_map_k<8>(in, k, w, g, cur, V, out, side, splits, part, st);
     default: return cudaErrorNotSupported;
   }
 }
