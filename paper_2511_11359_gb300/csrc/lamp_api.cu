@@ -250,6 +250,7 @@ __global__ void k_set_state(DevState* dev, long long t, double kappa) {
   dev->status = 0;
   dev->ticket = 0u;
   dev->t_eval = -1;
+  dev->t_logz = -1;
 }
 
 static int poll(lamp_ctx* ctx) {
@@ -411,10 +412,9 @@ static int create_impl(lamp_ctx** out, const lamp_problem* prob, const lamp_para
   // workspace
   Work& w = ctx->w;
   const size_t n = (size_t)k.n, m = (size_t)k.m;
-  // partial-sum width: the sweeps' 2 / 3 values per point, and the gradient's d values;
-  // the transport map widens the buffers on first use (ensure_part_width)
-  const size_t gradd = k.kind == COST_SQEUCLID ? (size_t)std::min<int64_t>(std::max<int64_t>(k.d, 2), 8) : 2;
-  ctx->part_width = (int)std::max<size_t>(3, gradd);
+  // partial-sum width: the sweeps' 2 / 3 values per point (the transport map of an l1 or l-inf
+  // cost with d > 8 widens the buffers on first use, ensure_part_width)
+  ctx->part_width = 3;
   // the bf16 point copies are padded to whole 128-point units (tc_pad); the per-point
   // column / row data to whole tiles of every sweep (a multiple of 256: the stored-cost
   // row sweep reads the data of 256 columns per tile); padding entries contribute nothing
@@ -453,6 +453,7 @@ static int create_impl(lamp_ctx** out, const lamp_problem* prob, const lamp_para
   std::memset(ctx->host_dev, 0, sizeof(DevState));
   ctx->host_dev->swf_kap = -1.0;  // no cached sweep constants yet (kappa >= 0 always)
   ctx->host_dev->t_eval = -1;
+  ctx->host_dev->t_logz = -1;
   {
     cudaError_t e = cudaMemcpyAsync(w.dev, ctx->host_dev, sizeof(DevState), cudaMemcpyHostToDevice, ctx->stream);
     if (e != cudaSuccess) return bail(fail(ctx, LAMP_E_CUDA, "init copy: %s", cudaGetErrorString(e)));
@@ -821,6 +822,13 @@ static int dot_splits(const lamp_ctx* ctx, bool rows) {
   return choose_split(out, in, ctx->g.sms, 4, 0.01);
 }
 
+// inner splits of a low-dimensional weighted-sum pass with `sums` sums per point (lamp_wsum.cu)
+static int wsum_splits(const lamp_ctx* ctx, bool rows, int sums) {
+  const int64_t out = cdiv64(rows ? ctx->k.n : ctx->k.m, wsum_outer(ctx->k.d, sums));
+  const int64_t in = cdiv64(rows ? ctx->k.m : ctx->k.n, wsum_inner());
+  return choose_split(out, in, (int64_t)ctx->g.sms * 2, 1, 0.005);
+}
+
 // room for `doubles` partial sums of the float32 gradient and transport-map passes
 static int ensure_gpart(lamp_ctx* ctx, size_t doubles) {
   if (doubles <= ctx->gpart_doubles) return LAMP_OK;
@@ -844,6 +852,18 @@ extern "C" int lamp_apply_map(lamp_ctx* ctx, const float* V, int64_t k, float* o
                                   (long long)k);
   if (side != 0 && side != 1) return fail(ctx, LAMP_E_INVALID, "lamp_apply_map: side must be 0 (p V) or 1 (p^T U)");
   int rc, splits = 0;
+  if (uses_direct_sweeps(ctx->k, ctx->prec)) {
+    // one pass with the row sums inside (side 0), or the row sums and one pass (side 1): no
+    // column sums, so no evaluation pass
+    const int sr = wsum_splits(ctx, true, side == 0 ? (int)k + 1 : 1), sc = wsum_splits(ctx, false, (int)k);
+    const size_t pairs = (size_t)cdiv64(ctx->k.n, wsum_inner()) * wsum_inner() * 2;  // float4 per entry, in doubles
+    const size_t rows = (size_t)sr * ctx->k.n * (side == 0 ? k + 1 : 1);
+    const size_t part = side == 0 ? rows : std::max(rows, (size_t)sc * ctx->k.m * k);
+    if ((rc = ensure_gpart(ctx, pairs + part))) return rc;
+    CK(direct_map(side, ctx->in, ctx->w, ctx->k, V, (int)k, sr, sc, ctx->gpart + pairs,
+                  reinterpret_cast<float4*>(ctx->gpart), out, ctx->stream));
+    return LAMP_OK;
+  }
   if (ctx->k.zdot) {
     if ((rc = ensure_dot_copies(ctx))) return rc;
     splits = dot_splits(ctx, side == 0);
@@ -1001,16 +1021,18 @@ static int grad_tc(lamp_ctx* ctx, float* dx, float* dy) {
   return LAMP_OK;
 }
 
-// the envelope gradient in float32 for d > 8: one pass per side with all coordinates
-static int grad_dot(lamp_ctx* ctx, float* dx, float* dy) {
+// the envelope gradient in float32: one pass per side with all coordinates
+static int grad_fp32(lamp_ctx* ctx, float* dx, float* dy) {
   const Consts& k = ctx->k;
-  const int sx = dot_splits(ctx, true), sy = dot_splits(ctx, false);
+  const int sx = k.zdot ? dot_splits(ctx, true) : wsum_splits(ctx, true, k.d);
+  const int sy = k.zdot ? dot_splits(ctx, false) : wsum_splits(ctx, false, k.d);
   int rc = ensure_gpart(ctx, std::max(dx ? (size_t)sx * k.n : 0, dy ? (size_t)sy * k.m : 0) * k.d);
   if (rc) return rc;
   if ((rc = evaluate_if_stale(ctx))) return rc;
   const int cur = ctx->host_dev->cur;
-  if (dx) CK(dot_grad(true, ctx->in, ctx->w, k, cur, sx, ctx->gpart, dx, ctx->stream));
-  if (dy) CK(dot_grad(false, ctx->in, ctx->w, k, cur, sy, ctx->gpart, dy, ctx->stream));
+  const auto pass = k.zdot ? dot_grad : direct_grad;
+  if (dx) CK(pass(true, ctx->in, ctx->w, k, cur, sx, ctx->gpart, dx, ctx->stream));
+  if (dy) CK(pass(false, ctx->in, ctx->w, k, cur, sy, ctx->gpart, dy, ctx->stream));
   return LAMP_OK;
 }
 
@@ -1018,13 +1040,7 @@ extern "C" int lamp_grad(lamp_ctx* ctx, float* dx, float* dy) {
   if (!ctx) return fail(nullptr, LAMP_E_INVALID, "lamp_grad: null context");
   if (ctx->pub_kind != LAMP_COST_SQEUCLID) return fail(ctx, LAMP_E_UNSUPPORTED, "lamp_grad needs LAMP_COST_SQEUCLID");
   if (ctx->prec == LAMP_PREC_BF16_TC) return grad_tc(ctx, dx, dy);
-  if (ctx->k.zdot) return grad_dot(ctx, dx, dy);
-  int rc = ensure_part_width(ctx, (int)ctx->k.d);
-  if (rc) return rc;
-  rc = evaluate_if_stale(ctx);
-  if (rc) return rc;
-  CK(launch_grad(ctx->in, ctx->k, ctx->w, ctx->g, ctx->prec, dx, dy, ctx->stream));
-  return LAMP_OK;
+  return grad_fp32(ctx, dx, dy);
 }
 
 extern "C" int lamp_get_state(lamp_ctx* ctx, double* nu, double* theta, double* logZ, double* kappa, int64_t* t,
@@ -1042,7 +1058,7 @@ extern "C" int lamp_get_state(lamp_ctx* ctx, double* nu, double* theta, double* 
     CK(cudaMemcpyAsync(row_shifts, ctx->w.rowshift[cur], ctx->k.n * sizeof(float2), cudaMemcpyDeviceToHost,
                        ctx->stream));
   CK(cudaStreamSynchronize(ctx->stream));
-  if (logZ && d.t_eval != d.t)
+  if (logZ && d.t_eval != d.t && d.t_logz != d.t)
     for (int64_t i = 0; i < ctx->k.n; ++i) logZ[i] = NAN;
   if (kappa) *kappa = d.kappa;
   if (t) *t = d.t;

@@ -291,6 +291,7 @@ struct DevState {
   long long tmax;     // stop when t >= tmax
   unsigned int ticket;  // last-block counter of the column finalize kernel
   unsigned int pad;
+  long long t_logz;   // iteration index whose log Z a transport-map pass wrote (-1: none)
   // results for the last evaluated X^t
   long long t_eval;
   double kappa_eval;
@@ -464,8 +465,6 @@ cudaError_t launch_iteration_part(const Inputs& in, const Consts& k, const Work&
                                   int part, int eval, cudaStream_t st);
 int tile_outer_cols(const Consts& k, int prec);
 int tile_inner_cols(const Consts& k, int prec);
-cudaError_t launch_grad(const Inputs& in, const Consts& k, const Work& w, const Geometry& g, int prec,
-                        float* dx, float* dy, cudaStream_t st);
 // transport-map application (lamp_kernels.cu): out = p V (side 0) or p^T U (side 1), 1 <= dk <= 8;
 // dot-form costs: sums per `splits` inner splits in `part` (splits x outer points x dk)
 cudaError_t launch_map(const Inputs& in, const Consts& k, const Work& w, const Geometry& g, int cur, const float* V,
@@ -489,6 +488,17 @@ cudaError_t dot_weighted(bool rows, const Work& w, const Consts& k, const float*
                          const float4* dat, int splits, double* part, cudaStream_t st);
 cudaError_t dot_grad(bool rows, const Inputs& in, const Work& w, const Consts& k, int cur, int splits, double* part,
                      float* out, cudaStream_t st);
+// weighted sums and maxima over low-dimensional point clouds (lamp_wsum.cu)
+enum DirectMaxMode : int { kDirectMax, kDirectMax2, kDirectKmax };
+int wsum_outer(int d, int sums);
+int wsum_inner();
+cudaError_t direct_grad(bool rows, const Inputs& in, const Work& w, const Consts& k, int cur, int splits, double* part,
+                        float* out, cudaStream_t st);
+// side 0: p V with the row sums in the same pass; side 1: the row sums (splits_rows), then p^T U
+// (splits_cols) with `pairs` as the rows' data.  Writes log Z.
+cudaError_t direct_map(int side, const Inputs& in, const Work& w, const Consts& k, const float* V, int nv,
+                       int splits_rows, int splits_cols, double* part, float4* pairs, float* out, cudaStream_t st);
+cudaError_t direct_max(int mode, const Inputs& in, const Work& w, const Consts& k, int splits, cudaStream_t st);
 // finalize kernels (lamp_fin.cu)
 cudaError_t launch_mirror_gain(const Inputs& in, const Consts& k, const Work& w, cudaStream_t st);
 cudaError_t launch_row_fin(const Inputs& in, const Consts& k, const Work& w, const Geometry& g, int eval,

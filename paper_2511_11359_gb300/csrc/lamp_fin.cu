@@ -428,8 +428,10 @@ k_col_fin(const Work w, int splits, const double* __restrict__ cvec, int rowbloc
     dev->costA = EVAL ? Cx + k.rnx : NAN;
     dev->colnu = EVAL ? Cn : NAN;
     dev->rlogZ = EVAL ? RL : NAN;
-    dev->t_eval = dev->t;
-    dev->kappa_eval = dev->kappa;
+    if (EVAL) {
+      dev->t_eval = dev->t;
+      dev->kappa_eval = dev->kappa;
+    }
     if (dev->status != 0 || !isfinite(R)) {
       if (dev->status == 0) dev->status = 5;
       dev->done = 1;

@@ -90,13 +90,13 @@ struct SweepIO {
 };
 
 // M_COLSUM: DG = 1 also accumulates the cost-weighted sums (evaluation passes).
-// M_GRAD accumulates sum_b 2^{v_ab} weight_b V_b[0:DG] with V = Vin (n_in x DG, row-major)
-// when given, else coordinates q0 .. q0 + DG - 1 of the inner points (the gradient)
+// M_GRAD accumulates sum_b 2^{v_ab} weight_b V_b[0:DG], V = Vin (n_in x DG, row-major): the
+// transport map of costs that the packed kernels do not serve (l1, l-inf with d > 8)
 template <int MODE, int DG>
 __global__ void __launch_bounds__(kThreads, MODE == M_GRAD ? 1 : 2)
 k_pts_sweep(const float* __restrict__ P_out, const float* __restrict__ P_in, int64_t n_out, int64_t n_in, int d,
             const SweepIO io, double* __restrict__ part, float* __restrict__ pmax, int tiles_per_split,
-            const DevState* __restrict__ dev, const Consts k, const float* __restrict__ Vin, int q0) {
+            const DevState* __restrict__ dev, const Consts k, const float* __restrict__ Vin) {
   if ((MODE == M_ROWSUM || MODE == M_COLSUM) && dev->done) return;
   const int cur = dev->cur;
   const float2* __restrict__ off2 = cur ? io.off2[1] : io.off2[0];
@@ -170,7 +170,7 @@ k_pts_sweep(const float* __restrict__ P_out, const float* __restrict__ P_in, int
     const int64_t i0 = it * kPT;
     __syncthreads();
     stage_points(sIn, P_in, i0, n_in, d, tid, kThreads);
-    if (MODE == M_GRAD && Vin) {
+    if (MODE == M_GRAD) {
       for (int idx = tid; idx < DG * kPT; idx += kThreads) {
         int p = idx / (DG > 0 ? DG : 1), q = idx - p * (DG > 0 ? DG : 1);
         int64_t gi = i0 + p;
@@ -299,9 +299,8 @@ k_pts_sweep(const float* __restrict__ P_out, const float* __restrict__ P_in, int
           const float vA = __fmaf_rn(alA, zz, __fmaf_rn(ahA, zz, -(oA[a] + dat[b].x)));
           const float pA = ex2(vA) * dat[b].y;
           const int ib = (b < 4) ? (tx * 4 + b) : (64 + tx * 4 + b - 4);
-          const float* src = Vin ? sV : sIn + q0 * kPT;
 #pragma unroll
-          for (int q = 0; q < DG; ++q) g[q] = __fmaf_rn(pA, src[q * kPT + ib], g[q]);
+          for (int q = 0; q < DG; ++q) g[q] = __fmaf_rn(pA, sV[q * kPT + ib], g[q]);
         }
 #pragma unroll
         for (int q = 0; q < DG; ++q) gacc[a][q] += (double)g[q];
@@ -691,39 +690,6 @@ __global__ void k_prime_fin(const Work w, int splits, const Consts k) {
   rowshift[i] = make_float2((float)qA, (float)qB);
 }
 
-// gradient finalize of coordinates q0 .. q0 + dg - 1 (partials hold dg values per point):
-// dx_i = 2 s (r_i x_i - q_i acc_i)
-__global__ void k_grad_fin(const double* __restrict__ part, int splits, int64_t np, int dg, int q0, int d,
-                           const float* __restrict__ P, const double* __restrict__ mass,
-                           const float4* __restrict__ wsrc, int wcomp, double s, float* __restrict__ out) {
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= np) return;
-  float4 wq = wsrc[i];
-  double wgt = (double)(wcomp == 1 ? wq.y : wq.w);
-  double ms = mass[i];
-  for (int q = 0; q < dg; ++q) {
-    double acc = 0.0;
-    for (int sp = 0; sp < splits; ++sp) acc += part[((int64_t)sp * np + i) * dg + q];
-    out[i * d + q0 + q] = (float)(2.0 * s * (ms * (double)P[i * d + q0 + q] - wgt * acc));
-  }
-}
-
-// column gradient finalize of coordinates q0 .. q0 + dg - 1: dy_j = 2 s (A_j y_j - w_j acc_j),
-// w_j from the current column data
-__global__ void k_grad_fin_cols(const Work w, int splits, int64_t np, int dg, int q0, int d,
-                                const float* __restrict__ P, double s, float* __restrict__ out) {
-  int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= np) return;
-  float4 cq = w.colq[w.dev->cur][j];
-  double wgt = (double)cq.y;
-  double ms = w.colA[j];
-  for (int q = 0; q < dg; ++q) {
-    double acc = 0.0;
-    for (int sp = 0; sp < splits; ++sp) acc += w.colpart[((int64_t)sp * np + j) * dg + q];
-    out[j * d + q0 + q] = (float)(2.0 * s * (ms * (double)P[j * d + q0 + q] - wgt * acc));
-  }
-}
-
 // ------------------------------------------------------------------------------------------
 // launch glue
 
@@ -744,13 +710,13 @@ static SweepIO io_same(const float2* o2, const float4* o4, const float4* in) {
 template <int MODE, int DG>
 static cudaError_t launch_pts(const float* Pout, const float* Pin, int64_t nout, int64_t nin, int d, const SweepIO& io,
                               double* part, float* pmax, int splits, const DevState* dev, const Consts& k,
-                              cudaStream_t st, const float* V = nullptr, int q0 = 0) {
+                              cudaStream_t st, const float* V = nullptr) {
   auto kern = k_pts_sweep<MODE, DG>;
   size_t sm = pts_smem(d, V ? DG : 0);
   int64_t tin = cdiv(nin, kPT);
   int tps = (int)cdiv(tin, splits);
   dim3 grid((unsigned)cdiv(nout, kPT), (unsigned)splits);
-  kern<<<grid, kThreads, sm, st>>>(Pout, Pin, nout, nin, d, io, part, pmax, tps, dev, k, V, q0);
+  kern<<<grid, kThreads, sm, st>>>(Pout, Pin, nout, nin, d, io, part, pmax, tps, dev, k, V);
   return cudaGetLastError();
 }
 
@@ -802,6 +768,7 @@ cudaError_t launch_kmax(const Inputs& in, const Consts& k, const Work& w, const 
     w2.colq[0] = w2.colq[1] = w.colq[1];
     return dot_launch(kDotKmax, w2, k, g, st);
   }
+  if (k.shared_shift) return direct_max(kDirectKmax, in, w, k, g.rows_split, st);
   // rowmax[split][0][n] = max_j D_ij, rowmax[split][1][n] = max_j -D_ij, D = |x|^2 + |y|^2 - 2 x.y
   return launch_pts<M_KMAX, 0>(in.x, in.y, k.n, k.m, k.d, io_same(w.rowshift[1], nullptr, w.colq[1]), nullptr,
                                w.rowmax, g.rows_split, w.dev, k, st);
@@ -834,6 +801,7 @@ static cudaError_t launch_row_sweep(const Inputs& in, const Consts& k, const Wor
     return cudaGetLastError();
   }
   if (mode == M_ROWSUM && k.shared_shift) return launch_direct_sweep(true, 0, in, k, w, g, st);
+  if (k.shared_shift) return direct_max(mode == M_MAX2 ? kDirectMax2 : kDirectMax, in, w, k, g.rows_split, st);
   if (k.zdot) return dot_launch(mode == M_ROWSUM ? kDotRowSum : mode == M_MAX2 ? kDotMax2 : kDotMax, w, k, g, st);
   SweepIO io;
   for (int b = 0; b < 2; ++b) {
@@ -982,58 +950,6 @@ int tile_outer_cols(const Consts& k, int prec) {
 int tile_inner_cols(const Consts& k, int prec) {
   if (prec == 1) return tc_tile_stream();
   return k.kind == COST_DENSE ? kDColRows : uses_direct_sweeps(k, prec) ? kDirectTile : kPT;
-}
-
-// gradient coordinates q0 .. q0 + DG - 1 (one recompute sweep per side)
-template <int DG>
-static cudaError_t launch_grad_d(const Inputs& in, const Consts& k, const Work& w, const Geometry& g, float* dx,
-                                 float* dy, int q0, cudaStream_t st) {
-  if (dx) {
-    // outer = rows (x), inner = columns (y): weights w_j of colq, outer offsets RqA of g2row
-    SweepIO io;
-    for (int b = 0; b < 2; ++b) { io.off2[b] = nullptr; io.off4[b] = w.g2row; io.indat[b] = w.colq[b]; }
-    cudaError_t e = launch_pts<M_GRAD, DG>(in.x, in.y, k.n, k.m, k.d, io, w.rowpart, nullptr, g.rows_split, w.dev,
-                                           k, st, nullptr, q0);
-    if (e != cudaSuccess) return e;
-    k_grad_fin<<<(unsigned)cdiv(k.n, 256), 256, 0, st>>>(w.rowpart, g.rows_split, k.n, DG, q0, k.d, in.x, in.r,
-                                                        w.g2row, 1, k.s, dx);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-  }
-  if (dy) {
-    // outer = columns (y), inner = rows (x): weights q_i of g2row, outer offsets BqA of colq
-    SweepIO io;
-    for (int b = 0; b < 2; ++b) { io.off2[b] = nullptr; io.off4[b] = w.colq[b]; io.indat[b] = w.g2row; }
-    cudaError_t e = launch_pts<M_GRAD, DG>(in.y, in.x, k.m, k.n, k.d, io, w.colpart, nullptr, g.cols_split, w.dev,
-                                           k, st, nullptr, q0);
-    if (e != cudaSuccess) return e;
-    k_grad_fin_cols<<<(unsigned)cdiv(k.m, 256), 256, 0, st>>>(w, g.cols_split, k.m, DG, q0, k.d, in.y, k.s, dy);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
-}
-
-// the gradient in chunks of up to 8 coordinates (the partial-sum buffers hold 8 values per
-// point when d > 8): ceil(d / 8) recompute sweeps per side
-cudaError_t launch_grad(const Inputs& in, const Consts& k, const Work& w, const Geometry& g, int prec, float* dx,
-                        float* dy, cudaStream_t st) {
-  for (int q0 = 0; q0 < k.d; q0 += 8) {
-    const int dg = k.d - q0 < 8 ? k.d - q0 : 8;
-    cudaError_t e;
-    switch (dg) {
-      case 1: e = launch_grad_d<1>(in, k, w, g, dx, dy, q0, st); break;
-      case 2: e = launch_grad_d<2>(in, k, w, g, dx, dy, q0, st); break;
-      case 3: e = launch_grad_d<3>(in, k, w, g, dx, dy, q0, st); break;
-      case 4: e = launch_grad_d<4>(in, k, w, g, dx, dy, q0, st); break;
-      case 5: e = launch_grad_d<5>(in, k, w, g, dx, dy, q0, st); break;
-      case 6: e = launch_grad_d<6>(in, k, w, g, dx, dy, q0, st); break;
-      case 7: e = launch_grad_d<7>(in, k, w, g, dx, dy, q0, st); break;
-      default: e = launch_grad_d<8>(in, k, w, g, dx, dy, q0, st); break;
-    }
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
 }
 
 // ------------------------------------------------------------------------------------------
