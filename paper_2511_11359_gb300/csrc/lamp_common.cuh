@@ -517,6 +517,10 @@ bool uses_direct_sweeps(const Consts& k, int prec);
 constexpr int kDirectTile = 128;
 int direct_outer(int d);
 int direct_blocks_per_sm();
+// the same sweeps for grids below one wave (lamp_direct_small.cu)
+bool direct_small_serves(int64_t nout, int64_t nin, int d, int splits, int sms);
+cudaError_t launch_direct_small(bool rows, int eval, const Inputs& in, const Consts& k, const Work& w,
+                                const Geometry& g, cudaStream_t st);
 cudaError_t launch_direct_sweep(bool rows, int eval, const Inputs& in, const Consts& k, const Work& w,
                                 const Geometry& g, cudaStream_t st);
 

@@ -6,14 +6,13 @@
 #include <cmath>
 #include <cstdint>
 
-#include "lamp_common.cuh"
+#include "lamp_direct.cuh"
 
 namespace lamp {
 
 namespace {
 
 constexpr int kThreads = 256;
-enum SweepMode : int { M_ROWSUM = 0, M_COLSUM = 1 };
 
 inline int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
@@ -35,61 +34,6 @@ inline int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
 // (y - x)^2 == (x - y)^2 in IEEE arithmetic, so the row and the column sweep see
 // bit-identical exponents.  The inner data are the packed-pair arrays (see Work).
 
-constexpr int kDTile = kDirectTile;  // inner points per shared-memory tile
-constexpr int kDPairs = kDTile / 2;  // pairs per tile
-constexpr int kDFold = 32;           // pairs between float-float folds of the packed sums
-
-template <int D>
-struct DirectCfg {
-  static constexpr int R = D <= 4 ? 4 : 2;  // outer points per thread
-  static constexpr int DP = (D + 1) & ~1;   // coordinates per pair record, even
-  static constexpr int REC = DP * 2 + 8;    // floats per pair record: coords [DP][2], offsets/weights A, B
-  static constexpr int OUTER = kThreads * R;
-};
-
-__device__ __forceinline__ void cp_async4(void* dst, const void* src, bool valid) {
-  const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d), "l"(src), "r"(valid ? 4 : 0) : "memory");
-}
-__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
-  const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-
-// stage inner tile `it` (points it*128 ..) into the record buffer `rec`
-template <int D>
-__device__ __forceinline__ void direct_stage(float* rec, const float* __restrict__ P_in, int64_t n_in,
-                                             const float4* __restrict__ pairs, int64_t it, int tid) {
-  using C = DirectCfg<D>;
-  const int64_t i0 = it * kDTile;
-  for (int idx = tid; idx < kDTile * D; idx += kThreads) {
-    const int b = idx / D, k = idx - (idx / D) * D;
-    const bool ok = i0 + b < n_in;
-    const float* src = ok ? P_in + (i0 + b) * D + k : P_in;
-    cp_async4(rec + (b >> 1) * C::REC + k * 2 + (b & 1), src, ok);
-  }
-  // offsets / weights: pairs [2(i0/2 + p)] (stream A) and [2(i0/2 + p) + 1] (stream B);
-  // the pair arrays are padded to 128 entries, so a whole tile is always in bounds
-  for (int idx = tid; idx < kDPairs * 2; idx += kThreads) {
-    const int p = idx >> 1, s = idx & 1;
-    cp_async16(rec + p * C::REC + C::DP * 2 + 4 * s, pairs + (i0 >> 1) * 2 + idx);
-  }
-}
-
-// |x_k - y_k| for a pair of entries: clear both sign bits
-__device__ __forceinline__ uint64_t f2abs(uint64_t v) {
-  uint64_t r;
-  asm("and.b64 %0, %1, 0x7FFFFFFF7FFFFFFF;" : "=l"(r) : "l"(v));
-  return r;
-}
-__device__ __forceinline__ uint64_t f2max(uint64_t a, uint64_t b) {
-  const float2 x = upk(a), y = upk(b);
-  return pk(fmaxf(x.x, y.x), fmaxf(x.y, y.y));
-}
-
 // MODE = M_ROWSUM, or M_COLSUM with WC = 1 (evaluation pass: cost-weighted column sums too) or 0;
 // CK = the ground cost (Consts::cost_op): 0 |x - y|^2, 1 l1, 2 l-inf
 template <int MODE, int D, int WC, int CK>
@@ -107,13 +51,13 @@ k_pts_direct(const float* __restrict__ P_out, const float* __restrict__ P_in, in
   __shared__ __align__(16) float srec[2][kDPairs * REC];
 
   const int tid = threadIdx.x;
-  const int64_t o0 = (int64_t)blockIdx.x * C::OUTER;
+  const int64_t o0 = (int64_t)blockIdx.x * kThreads * R;
   const int split = blockIdx.y;
   const int64_t ntiles = (n_in + kDTile - 1) / kDTile;
   const int64_t it0 = (int64_t)split * tiles_per_split;
   const int64_t it1 = it0 + tiles_per_split < ntiles ? it0 + tiles_per_split : ntiles;
 
-  if (it0 < it1) direct_stage<D>(srec[0], P_in, n_in, pairs, it0, tid);
+  if (it0 < it1) direct_stage<D>(srec[0], P_in, n_in, pairs, it0, tid, kThreads);
   cp_async_commit();
   if (DP > D) {  // the padding coordinate of odd d is read by the 16-byte loads, never used
     for (int p = tid; p < 2 * kDPairs; p += kThreads) {
@@ -162,7 +106,7 @@ k_pts_direct(const float* __restrict__ P_out, const float* __restrict__ P_in, in
 
   for (int64_t it = it0; it < it1; ++it) {
     const int buf = (int)((it - it0) & 1);
-    if (it + 1 < it1) direct_stage<D>(srec[buf ^ 1], P_in, n_in, pairs, it + 1, tid);
+    if (it + 1 < it1) direct_stage<D>(srec[buf ^ 1], P_in, n_in, pairs, it + 1, tid, kThreads);
     cp_async_commit();
     cp_async_wait<1>();
     __syncthreads();
@@ -171,55 +115,11 @@ k_pts_direct(const float* __restrict__ P_out, const float* __restrict__ P_in, in
     for (int p0 = 0; p0 < kDPairs; p0 += kDFold) {
 #pragma unroll 2
       for (int p = p0; p < p0 + kDFold; ++p) {
-        const float* rp = rec + p * REC;
-        uint64_t y2[DP];
+        DirectPair<D> t;
+        t.load(rec + p * REC);
 #pragma unroll
-        for (int kk = 0; kk < DP; kk += 2) {
-          const float4 t = *reinterpret_cast<const float4*>(rp + 2 * kk);
-          y2[kk] = pk(t.x, t.y);
-          y2[kk + 1] = pk(t.z, t.w);
-        }
-        const float4 dA = *reinterpret_cast<const float4*>(rp + 2 * DP);
-        const float4 dB = *reinterpret_cast<const float4*>(rp + 2 * DP + 4);
-        const uint64_t oA2 = pk(dA.x, dA.y), wA2 = pk(dA.z, dA.w);
-        const uint64_t wB2 = pk(dB.z, dB.w);
-        // row sweep: the inner columns' dB_j = BqA_j - BcolB_j from the pair data
-        const uint64_t dC2 = pk(dB.x, dB.y);
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-          uint64_t z2;
-          if constexpr (CK == 0) {
-            uint64_t df = f2sub(x2[r][0], y2[0]);
-            z2 = f2mul(df, df);
-#pragma unroll
-            for (int kk = 1; kk < D; ++kk) {
-              df = f2sub(x2[r][kk], y2[kk]);
-              z2 = f2fma(df, df, z2);
-            }
-          } else {
-            z2 = f2abs(f2sub(x2[r][0], y2[0]));
-#pragma unroll
-            for (int kk = 1; kk < D; ++kk) {
-              const uint64_t ad = f2abs(f2sub(x2[r][kk], y2[kk]));
-              z2 = CK == 1 ? f2add(z2, ad) : f2max(z2, ad);
-            }
-          }
-          const uint64_t vA = f2fma(alA2, z2, f2fma(ahA2, z2, f2add(ownA[r], oA2)));
-          const uint64_t vB = f2fma(da2, z2, f2add(vA, MODE == M_ROWSUM ? dC2 : ownD[r]));
-          const float2 vAf = upk(vA), vBf = upk(vB);
-          const uint64_t eA = pk(ex2(vAf.x), ex2(vAf.y));
-          const uint64_t eB = pk(ex2(vBf.x), ex2(vBf.y));
-          if constexpr (WC) {
-            const uint64_t pA = f2mul(eA, wA2);
-            acc[r][0] = f2add(acc[r][0], pA);
-            acc[r][2] = f2fma(z2, pA, acc[r][2]);
-          } else {
-            acc[r][0] = f2fma(eA, wA2, acc[r][0]);
-          }
-          // row sums of stream B carry no weight (it is inside dB_j); column sums weight by q^B_i
-          if constexpr (MODE == M_ROWSUM) acc[r][1] = f2add(acc[r][1], eB);
-          else acc[r][1] = f2fma(eB, wB2, acc[r][1]);
-        }
+        for (int r = 0; r < R; ++r)
+          direct_pair<MODE, D, WC, CK>(x2[r], ownA[r], ownD[r], t, ahA2, alA2, da2, acc[r]);
       }
 #pragma unroll
       for (int r = 0; r < R; ++r)
@@ -248,7 +148,7 @@ static cudaError_t launch_direct_d(const float* Pout, const float* Pin, int64_t 
                                    double* part, int splits, const Consts& k, cudaStream_t st) {
   int64_t tin = cdiv(nin, kDTile);
   int tps = (int)cdiv(tin, splits);
-  dim3 grid((unsigned)cdiv(nout, DirectCfg<D>::OUTER), (unsigned)splits);
+  dim3 grid((unsigned)cdiv(nout, kThreads * DirectCfg<D>::R), (unsigned)splits);
   k_pts_direct<MODE, D, WC, CK><<<grid, kThreads, 0, st>>>(Pout, Pin, nout, nin, w, part, tps, k);
   return cudaGetLastError();
 }
@@ -294,6 +194,8 @@ int direct_blocks_per_sm() {
 
 cudaError_t launch_direct_sweep(bool rows, int eval, const Inputs& in, const Consts& k, const Work& w,
                                 const Geometry& g, cudaStream_t st) {
+  if (direct_small_serves(rows ? k.n : k.m, rows ? k.m : k.n, k.d, rows ? g.rows_split : g.cols_split, g.sms))
+    return launch_direct_small(rows, eval, in, k, w, g, st);
   if (rows) return launch_direct<M_ROWSUM, 0>(in.x, in.y, k.n, k.m, w, w.rowpart, g.rows_split, k, st);
   if (eval) return launch_direct<M_COLSUM, 1>(in.y, in.x, k.m, k.n, w, w.colpart, g.cols_split, k, st);
   return launch_direct<M_COLSUM, 0>(in.y, in.x, k.m, k.n, w, w.colpart, g.cols_split, k, st);
