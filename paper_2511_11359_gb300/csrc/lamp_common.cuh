@@ -148,6 +148,13 @@ __host__ __device__ inline double quantize(double x, double g) {
 }
 
 #ifdef __CUDACC__
+// launch and report
+template <class... P, class... A>
+inline cudaError_t launch_kernel(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+  kern<<<grid, block, smem, st>>>(static_cast<P>(args)...);
+  return cudaGetLastError();
+}
+
 // write entry e of a packed-pair array (layout described in Work)
 __device__ __forceinline__ void store_pair_entry(float4* __restrict__ a, int64_t e, float offA, float wA, float dB,
                                                  float wB) {

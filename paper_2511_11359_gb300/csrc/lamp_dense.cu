@@ -268,13 +268,8 @@ cudaError_t dense_launch_sweep(bool rows, int eval, const Geometry& g, const Wor
   const int tps = (int)((ntiles + splits - 1) / splits);
   dim3 grid((unsigned)nblk, (unsigned)splits);
   const CUtensorMap& map = *reinterpret_cast<const CUtensorMap*>(g.map_c);
-  if (rows)
-    dense::k_dense_tma<true, 0><<<grid, dense::kThreads, dense::kSmemBytes, st>>>(map, w, k.n, k.m, tps, k);
-  else if (eval)
-    dense::k_dense_tma<false, 1><<<grid, dense::kThreads, dense::kSmemBytes, st>>>(map, w, k.n, k.m, tps, k);
-  else
-    dense::k_dense_tma<false, 0><<<grid, dense::kThreads, dense::kSmemBytes, st>>>(map, w, k.n, k.m, tps, k);
-  return cudaGetLastError();
+  const auto kern = rows ? dense::k_dense_tma<true, 0> : eval ? dense::k_dense_tma<false, 1> : dense::k_dense_tma<false, 0>;
+  return launch_kernel(kern, grid, dense::kThreads, dense::kSmemBytes, st, map, w, k.n, k.m, tps, k);
 }
 
 }  // namespace lamp

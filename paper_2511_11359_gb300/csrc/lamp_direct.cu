@@ -149,8 +149,7 @@ static cudaError_t launch_direct_d(const float* Pout, const float* Pin, int64_t 
   int64_t tin = cdiv(nin, kDTile);
   int tps = (int)cdiv(tin, splits);
   dim3 grid((unsigned)cdiv(nout, kThreads * DirectCfg<D>::R), (unsigned)splits);
-  k_pts_direct<MODE, D, WC, CK><<<grid, kThreads, 0, st>>>(Pout, Pin, nout, nin, w, part, tps, k);
-  return cudaGetLastError();
+  return launch_kernel(k_pts_direct<MODE, D, WC, CK>, grid, kThreads, 0, st, Pout, Pin, nout, nin, w, part, tps, k);
 }
 
 template <int MODE, int WC, int CK>

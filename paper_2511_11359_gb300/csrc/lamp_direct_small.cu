@@ -129,9 +129,8 @@ cudaError_t go(const Launch& l, const Work& w, const Consts& k, cudaStream_t st)
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
     if (e != cudaSuccess) return e;
   }
-  k_direct_small<MODE, D, WC, CK, R><<<dim3((unsigned)cdiv(l.nout, 32 * R), (unsigned)l.splits), threads, smem, st>>>(
-      l.Pout, l.Pin, l.nout, l.nin, w, l.part, l.tps, k);
-  return cudaGetLastError();
+  return launch_kernel(k_direct_small<MODE, D, WC, CK, R>, dim3((unsigned)cdiv(l.nout, 32 * R), (unsigned)l.splits), threads,
+                    smem, st, l.Pout, l.Pin, l.nout, l.nin, w, l.part, l.tps, k);
 }
 
 template <int MODE, int D, int WC>

@@ -638,8 +638,7 @@ template <int MODE>
 cudaError_t launch_mode(const dot::Args& a, const Work& w, const Consts& k, int sms, cudaStream_t st) {
   const int64_t items = (int64_t)a.out_tiles * a.splits;
   const unsigned grid = (unsigned)(items < sms ? items : sms);
-  dot::k_dot_sweep<MODE><<<grid, dot::kThreads, dot::smem_floats(a.d) * sizeof(float), st>>>(a, w.dev, k);
-  return cudaGetLastError();
+  return launch_kernel(dot::k_dot_sweep<MODE>, grid, dot::kThreads, dot::smem_floats(a.d) * sizeof(float), st, a, w.dev, k);
 }
 
 template <int MODE>

@@ -473,25 +473,15 @@ cudaError_t launch_mirror_gain(const Inputs& in, const Consts& k, const Work& w,
 
 cudaError_t launch_row_fin(const Inputs& in, const Consts& k, const Work& w, const Geometry& g, int eval,
                            cudaStream_t st) {
-  if (eval) {
-    const unsigned nb = blocks_of(k.n, kPts);
-    k_row_fin<true><<<nb, kThreads, 0, st>>>(w, g.rows_split, in.r, (int)nb, k);
-  } else {
-    const unsigned nb = blocks_of(k.n, kPts);
-    k_row_fin<false><<<nb + 1, kThreads, 0, st>>>(w, g.rows_split, in.r, (int)nb, k);
-  }
-  return cudaGetLastError();
+  const unsigned nb = blocks_of(k.n, kPts);
+  if (eval) return launch_kernel(k_row_fin<true>, nb, kThreads, 0, st, w, g.rows_split, in.r, (int)nb, k);
+  return launch_kernel(k_row_fin<false>, nb + 1, kThreads, 0, st, w, g.rows_split, in.r, (int)nb, k);
 }
 
 cudaError_t launch_col_fin(const Inputs& in, const Consts& k, const Work& w, const Geometry& g, int eval,
                            cudaStream_t st) {
-  if (eval)
-    k_col_fin<true><<<blocks_of(k.m, kPts), kThreads, 0, st>>>(
-        w, g.cols_split, in.c, (int)blocks_of(k.n, kPts), k);
-  else
-    k_col_fin<false><<<blocks_of(k.m, kPts), kThreads, 0, st>>>(w, g.cols_split, in.c,
-                                                                                              0, k);
-  return cudaGetLastError();
+  return launch_kernel(eval ? k_col_fin<true> : k_col_fin<false>, blocks_of(k.m, kPts), kThreads, 0, st, w, g.cols_split,
+                    in.c, (int)blocks_of(k.n, kPts), k);
 }
 
 }  // namespace lamp

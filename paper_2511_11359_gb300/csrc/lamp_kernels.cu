@@ -351,11 +351,47 @@ k_pts_sweep(const float* __restrict__ P_out, const float* __restrict__ P_in, int
 // ------------------------------------------------------------------------------------------
 // sweeps over a stored dense cost (LAMP_COST_DENSE), streamed from HBM with coalesced loads
 
-constexpr int kDR = 8;        // rows per CTA in the row sweep
-constexpr int kDChunk = 1024; // columns per CTA step (4 per thread, stride 256)
+// Row sweep: a CTA of 256 threads owns kDR rows and steps over chunks of 1024 columns (thread t
+// takes columns t + 256 q); column sweep: a CTA of 128 threads owns 256 columns (two per thread)
+// and walks a split's rows in groups of 16.  These serve stored costs whose rows are not a
+// multiple of 16 bytes apart (lamp_dense.cu streams the others) and the row-max passes of all
+// stored costs.  Bound by the latency of the loads at the sizes that fit the L2 and by HBM above:
+// the next chunk's (group's) entries are loaded while the current one is evaluated, and the grid
+// is fine enough to fill the SMs.  3001 x 2777: 19.9 -> 12.3 us (rows; 8 rows per CTA, no load
+// ahead, a butterfly of five steps per sum), 20.4 -> 13.9 us (columns; 1024 columns per CTA).
+constexpr int kDR = 4;          // rows per CTA in the row sweep
+constexpr int kDSplitRows = 8;  // rows per tile in the choice of its splits
+constexpr int kDChunk = 1024;   // columns per CTA step (4 per thread, stride 256)
+
+// sums over a warp of NV = 16, 8 or 4 float-float values per lane, as warp_sum_ff adds them (xor
+// 16, 8, 4, 2, 1); each level halves the values a lane carries until one is left (the operands of
+// TwoSum and of its low parts' sum commute, so the results are the same), NV + 1 TwoSums for 16
+// values instead of 80.  Value q ends in the lanes with lane * NV / 32 == q.
+template <int NV>
+__device__ __forceinline__ void warp_sums_ff(float (&hi)[NV], float (&lo)[NV], int lane) {
+  int nv = NV;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const bool up = (lane & o) != 0;
+    const int half = nv > 1 ? nv / 2 : 0;
+    const int cnt = nv > 1 ? half : 1;
+#pragma unroll
+    for (int q = 0; q < NV; ++q) {
+      if (q >= cnt) continue;
+      const float kh = half ? (up ? hi[half + q] : hi[q]) : hi[q], kl = half ? (up ? lo[half + q] : lo[q]) : lo[q];
+      const float gh = half ? (up ? hi[q] : hi[half + q]) : hi[q], gl = half ? (up ? lo[q] : lo[half + q]) : lo[q];
+      const float h2 = __shfl_xor_sync(0xffffffffu, gh, o), l2 = __shfl_xor_sync(0xffffffffu, gl, o);
+      float sum, err;
+      two_sum(kh, h2, sum, err);
+      hi[q] = sum;
+      lo[q] = kl + l2 + err;
+    }
+    nv = cnt;
+  }
+}
 
 template <int MODE>  // M_ROWSUM, M_MAX or M_MAX2
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, 3)
 k_dense_rows(const float* __restrict__ C, int64_t ldc, int64_t n, int64_t m, const Work w,
              int chunks_per_split, const Consts k) {
   const DevState* __restrict__ dev = w.dev;
@@ -363,9 +399,8 @@ k_dense_rows(const float* __restrict__ C, int64_t ldc, int64_t n, int64_t m, con
   const int cur = dev->cur;
   const float2* __restrict__ rowshift = w.rowshift[cur];
   const float4* __restrict__ colq = w.colq[cur];
-  double* __restrict__ part = w.rowpart;
-  float* __restrict__ pmax = w.rowmax;
-  __shared__ double sred[kThreads / 32][kDR * 2];
+  constexpr int NV = 2 * kDR;  // values per thread: both streams of kDR rows
+  __shared__ double sred[kThreads / 32][NV];
   const int tid = threadIdx.x;
   const int64_t r0 = (int64_t)blockIdx.x * kDR;
   const int split = blockIdx.y;
@@ -374,7 +409,8 @@ k_dense_rows(const float* __restrict__ C, int64_t ldc, int64_t n, int64_t m, con
   int64_t c1 = c0 + chunks_per_split;
   if (c1 > nchunks) c1 = nchunks;
   const SweepF sp = sweep_floats_of(dev, k);
-  const float ahA = sp.ahA, alA = sp.alA, ahB = sp.ahB, alB = sp.alB;
+  const uint64_t ahA2 = pk(sp.ahA, sp.ahA), alA2 = pk(sp.alA, sp.alA);
+  const uint64_t ahB2 = pk(sp.ahB, sp.ahB), alB2 = pk(sp.alB, sp.alB);
 
   float oA[kDR], oB[kDR];
   const float* crow[kDR];
@@ -383,107 +419,104 @@ k_dense_rows(const float* __restrict__ C, int64_t ldc, int64_t n, int64_t m, con
     int64_t gr = r0 + a;
     if (gr >= n) gr = n - 1;
     float2 q = MODE == M_MAX ? make_float2(0.f, 0.f) : rowshift[gr];
-    oA[a] = q.x;
-    oB[a] = q.y;
+    oA[a] = -q.x;
+    oB[a] = -q.y;
     crow[a] = C + gr * ldc;
   }
-  float hiA[kDR], loA[kDR], hiB[kDR], loB[kDR];
-  float mA[kDR], mB[kDR];
+  // sums: float-float values [2 a + stream]; maxima: hi alone
+  float hi[NV], lo[NV];
 #pragma unroll
-  for (int a = 0; a < kDR; ++a) {
-    hiA[a] = loA[a] = hiB[a] = loB[a] = 0.f;
-    mA[a] = mB[a] = -INFINITY;
+  for (int q = 0; q < NV; ++q) {
+    hi[q] = MODE == M_ROWSUM ? 0.f : -INFINITY;
+    lo[q] = 0.f;
   }
-
-  for (int64_t ch = c0; ch < c1; ++ch) {
-    float4 cd[4];
-    int64_t jj[4];
+  const auto load = [&](int64_t ch, float (&cv)[kDR][4]) {
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      jj[q] = ch * kDChunk + tid + q * kThreads;
-      cd[q] = jj[q] < m ? colq[jj[q]] : make_float4(INFINITY, 0.f, INFINITY, 0.f);
+      const int64_t j = ch * kDChunk + tid + q * kThreads;
+#pragma unroll
+      for (int a = 0; a < kDR; ++a) cv[a][q] = j < m ? __ldg(crow[a] + j) : 0.f;
     }
+  };
+  float nx[kDR][4];
+  if (c0 < c1) load(c0, nx);
+  for (int64_t ch = c0; ch < c1; ++ch) {
     float cv[kDR][4];
 #pragma unroll
     for (int a = 0; a < kDR; ++a)
 #pragma unroll
-      for (int q = 0; q < 4; ++q) cv[a][q] = jj[q] < m ? __ldg(crow[a] + jj[q]) : 0.f;
+      for (int q = 0; q < 4; ++q) cv[a][q] = nx[a][q];
+    float4 cd[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int64_t j = ch * kDChunk + tid + q * kThreads;
+      cd[q] = j < m ? colq[j] : make_float4(INFINITY, 0.f, INFINITY, 0.f);
+    }
+    if (ch + 1 < c1) load(ch + 1, nx);
 #pragma unroll
     for (int a = 0; a < kDR; ++a) {
+      float sA = 0.f, sB = 0.f;
+#pragma unroll
+      for (int p = 0; p < 2; ++p) {
+        const float4 d0 = cd[2 * p], d1 = cd[2 * p + 1];
+        const uint64_t z2 = pk(cv[a][2 * p], cv[a][2 * p + 1]);
+        if (MODE == M_ROWSUM) {
+          const float2 eA = upk(exp2_pair(ahA2, alA2, z2, f2sub(pk(oA[a], oA[a]), pk(d0.x, d1.x))));
+          const float2 eB = upk(exp2_pair(ahB2, alB2, z2, f2sub(pk(oB[a], oB[a]), pk(d0.z, d1.z))));
+          sA = __fmaf_rn(eA.y, d1.y, __fmaf_rn(eA.x, d0.y, sA));
+          sB = __fmaf_rn(eB.y, d1.w, __fmaf_rn(eB.x, d0.w, sB));
+        } else if (MODE == M_MAX2) {
+          // refinement pass of the eta = 0 dual bound (see k_pts_sweep, M_MAX2)
+          const float2 u = upk(f2sub(f2fma(alA2, z2, f2fma(ahA2, z2, f2sub(pk(oA[a], oA[a]), pk(d0.x, d1.x)))),
+                                     pk(d0.y, d1.y)));
+          hi[2 * a] = fmaxf(hi[2 * a], fmaxf(u.x, u.y));
+        } else {
+          const float2 uA = upk(f2fma(ahA2, z2, pk(-d0.x, -d1.x))), uB = upk(f2fma(ahB2, z2, pk(-d0.z, -d1.z)));
+          hi[2 * a] = fmaxf(hi[2 * a], fmaxf(uA.x, uA.y));
+          hi[2 * a + 1] = fmaxf(hi[2 * a + 1], fmaxf(uB.x, uB.y));
+        }
+      }
       if (MODE == M_ROWSUM) {
-        float sA = 0.f, sB = 0.f;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const float zz = cv[a][q];
-          const float vA = __fmaf_rn(alA, zz, __fmaf_rn(ahA, zz, -(oA[a] + cd[q].x)));
-          const float vB = __fmaf_rn(alB, zz, __fmaf_rn(ahB, zz, -(oB[a] + cd[q].z)));
-          sA = __fmaf_rn(ex2(vA), cd[q].y, sA);
-          sB = __fmaf_rn(ex2(vB), cd[q].w, sB);
-        }
-        ff_add(hiA[a], loA[a], sA);
-        ff_add(hiB[a], loB[a], sB);
-      } else if (MODE == M_MAX2) {
-        // refinement pass of the eta = 0 dual bound (see k_pts_sweep, M_MAX2)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const float zz = cv[a][q];
-          mA[a] = fmaxf(mA[a], __fmaf_rn(alA, zz, __fmaf_rn(ahA, zz, -(oA[a] + cd[q].x))) - cd[q].y);
-        }
-      } else {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          mA[a] = fmaxf(mA[a], __fmaf_rn(ahA, cv[a][q], -cd[q].x));
-          mB[a] = fmaxf(mB[a], __fmaf_rn(ahB, cv[a][q], -cd[q].z));
-        }
+        ff_add(hi[2 * a], lo[2 * a], sA);
+        ff_add(hi[2 * a + 1], lo[2 * a + 1], sB);
       }
     }
   }
 
   const int lane = tid & 31, wid = tid >> 5;
   if (MODE == M_ROWSUM) {
-#pragma unroll
-    for (int a = 0; a < kDR; ++a) {
-      warp_sum_ff(hiA[a], loA[a]);
-      warp_sum_ff(hiB[a], loB[a]);
-      const double vA = (double)hiA[a] + (double)loA[a];
-      const double vB = (double)hiB[a] + (double)loB[a];
-      if (lane == 0) {
-        sred[wid][2 * a] = vA;
-        sred[wid][2 * a + 1] = vB;
-      }
-    }
+    warp_sums_ff<NV>(hi, lo, lane);
+    if ((lane & (32 / NV - 1)) == 0) sred[wid][lane / (32 / NV)] = (double)hi[0] + (double)lo[0];
     __syncthreads();
-    if (tid < 2 * kDR) {
+    if (tid < NV) {
       double v = 0.0;
-      for (int w = 0; w < kThreads / 32; ++w) v += sred[w][tid];
-      int a = tid >> 1, s = tid & 1;
-      if (r0 + a < n) part[((int64_t)split * 2 + s) * n + r0 + a] = v;
+      for (int u = 0; u < kThreads / 32; ++u) v += sred[u][tid];
+      const int a = tid >> 1, s = tid & 1;
+      if (r0 + a < n) w.rowpart[((int64_t)split * 2 + s) * n + r0 + a] = v;
     }
   } else {
-    __shared__ float fred[kThreads / 32][kDR * 2];
+    __shared__ float fred[kThreads / 32][NV];
 #pragma unroll
-    for (int a = 0; a < kDR; ++a) {
-      float vA = warp_max_f(mA[a]);
-      float vB = warp_max_f(mB[a]);
-      if (lane == 0) {
-        fred[wid][2 * a] = vA;
-        fred[wid][2 * a + 1] = vB;
-      }
+    for (int q = 0; q < NV; ++q) {
+      const float v = warp_max_f(hi[q]);
+      if (lane == 0) fred[wid][q] = v;
     }
     __syncthreads();
-    if (tid < 2 * kDR) {
+    if (tid < NV) {
       float v = -INFINITY;
-      for (int w = 0; w < kThreads / 32; ++w) v = fmaxf(v, fred[w][tid]);
-      int a = tid >> 1, s = tid & 1;
-      if (r0 + a < n) pmax[((int64_t)split * 2 + s) * n + r0 + a] = v;
+      for (int u = 0; u < kThreads / 32; ++u) v = fmaxf(v, fred[u][tid]);
+      const int a = tid >> 1, s = tid & 1;
+      if (r0 + a < n) w.rowmax[((int64_t)split * 2 + s) * n + r0 + a] = v;
     }
   }
 }
 
-constexpr int kDColRows = 16;  // rows per step (row data staged in shared memory)
+constexpr int kDColRows = 16;      // rows per group: the unit of the column sums
+constexpr int kDColThreads = 128;  // two columns per thread
+constexpr int kDCols = 2 * kDColThreads;
 
 template <int WC>  // 1: an evaluation pass, with the cost-weighted sums
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kDColThreads, 6)
 k_dense_cols(const float* __restrict__ C, int64_t ldc, int64_t n, int64_t m, const Work w, int64_t rows_per_split,
              const Consts k) {
   const DevState* __restrict__ dev = w.dev;
@@ -491,68 +524,69 @@ k_dense_cols(const float* __restrict__ C, int64_t ldc, int64_t n, int64_t m, con
   const float4* __restrict__ g2row = w.g2row;
   const float4* __restrict__ colq = w.colq[dev->cur];
   double* __restrict__ part = w.colpart;
-  __shared__ float4 srow[kDColRows];
   const int tid = threadIdx.x;
-  const int64_t jb = (int64_t)blockIdx.x * kDChunk;
   const int split = blockIdx.y;
   const int64_t i0 = (int64_t)split * rows_per_split;
   int64_t i1 = i0 + rows_per_split;
   if (i1 > n) i1 = n;
   const SweepF sp = sweep_floats_of(dev, k);
-  const float ahA = sp.ahA, alA = sp.alA, ahB = sp.ahB, alB = sp.alB;
+  const uint64_t ahA2 = pk(sp.ahA, sp.ahA), alA2 = pk(sp.alA, sp.alA);
+  const uint64_t ahB2 = pk(sp.ahB, sp.ahB), alB2 = pk(sp.alB, sp.alB);
 
-  float oA[4], oB[4];
-  int64_t jj[4];
-  bool ok[4];
+  int64_t jj[2];
+  bool ok[2];
+  float oA[2], oB[2];
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    jj[q] = jb + tid + q * kThreads;
+  for (int q = 0; q < 2; ++q) {
+    jj[q] = (int64_t)blockIdx.x * kDCols + tid + q * kDColThreads;
     ok[q] = jj[q] < m;
-    float4 cd = ok[q] ? colq[jj[q]] : make_float4(0.f, 0.f, 0.f, 0.f);
-    oA[q] = cd.x;
-    oB[q] = cd.z;
+    const float4 cd = ok[q] ? colq[jj[q]] : make_float4(0.f, 0.f, 0.f, 0.f);
+    oA[q] = -cd.x;
+    oB[q] = -cd.z;
   }
-  float hiA[4], loA[4], hiB[4], loB[4], hiC[4], loC[4];
+  const uint64_t oA2 = pk(oA[0], oA[1]), oB2 = pk(oB[0], oB[1]);
+  float hiA[2], loA[2], hiB[2], loB[2], hiC[2], loC[2];
 #pragma unroll
-  for (int q = 0; q < 4; ++q) hiA[q] = loA[q] = hiB[q] = loB[q] = hiC[q] = loC[q] = 0.f;
+  for (int q = 0; q < 2; ++q) hiA[q] = loA[q] = hiB[q] = loB[q] = hiC[q] = loC[q] = 0.f;
 
-  for (int64_t ib = i0; ib < i1; ib += kDColRows) {
-    __syncthreads();
-    if (tid < kDColRows) {
-      int64_t gi = ib + tid;
-      srow[tid] = gi < i1 ? g2row[gi] : make_float4(INFINITY, 0.f, INFINITY, 0.f);
-    }
-    __syncthreads();
-    float sA[4] = {0.f, 0.f, 0.f, 0.f}, sB[4] = {0.f, 0.f, 0.f, 0.f}, sC[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 4
+  // the entries of a group; rows past the split's end read its last row and are not added
+  const auto load = [&](int64_t ib, float (&cv)[kDColRows][2]) {
+#pragma unroll
     for (int a = 0; a < kDColRows; ++a) {
-      int64_t gi = ib + a;
-      if (gi >= i1) break;
-      const float4 rd = srow[a];
-      const float* crow = C + gi * ldc;
-      float cv[4];
+      const int64_t gi = ib + a < i1 ? ib + a : i1 - 1;
 #pragma unroll
-      for (int q = 0; q < 4; ++q) cv[q] = ok[q] ? __ldg(crow + jj[q]) : 0.f;
+      for (int q = 0; q < 2; ++q) cv[a][q] = ok[q] ? __ldg(C + gi * ldc + jj[q]) : 0.f;
+    }
+  };
+  for (int64_t ib = i0; ib < i1; ib += kDColRows) {
+    float cv[kDColRows][2];
+    load(ib, cv);
+    float sA[2] = {0.f, 0.f}, sB[2] = {0.f, 0.f}, sC[2] = {0.f, 0.f};
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const float zz = cv[q];
-        const float vA = __fmaf_rn(alA, zz, __fmaf_rn(ahA, zz, -(oA[q] + rd.x)));
-        const float vB = __fmaf_rn(alB, zz, __fmaf_rn(ahB, zz, -(oB[q] + rd.z)));
-        const float pA = __fmul_rn(ex2(vA), rd.y);
-        sA[q] = __fadd_rn(sA[q], pA);
-        if (WC) sC[q] = __fmaf_rn(zz, pA, sC[q]);
-        sB[q] = __fmaf_rn(ex2(vB), rd.w, sB[q]);
+    for (int a = 0; a < kDColRows; ++a) {
+      if (ib + a >= i1) break;
+      const float4 rd = __ldg(g2row + ib + a);
+      const uint64_t z2 = pk(cv[a][0], cv[a][1]);
+      const float2 eA = upk(exp2_pair(ahA2, alA2, z2, f2sub(oA2, pk(rd.x, rd.x))));
+      const float2 eB = upk(exp2_pair(ahB2, alB2, z2, f2sub(oB2, pk(rd.z, rd.z))));
+      const float pA[2] = {__fmul_rn(eA.x, rd.y), __fmul_rn(eA.y, rd.y)};
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        sA[q] = __fadd_rn(sA[q], pA[q]);
+        if (WC) sC[q] = __fmaf_rn(cv[a][q], pA[q], sC[q]);
       }
+      sB[0] = __fmaf_rn(eB.x, rd.w, sB[0]);
+      sB[1] = __fmaf_rn(eB.y, rd.w, sB[1]);
     }
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
+    for (int q = 0; q < 2; ++q) {
       ff_add(hiA[q], loA[q], sA[q]);
       ff_add(hiB[q], loB[q], sB[q]);
       if (WC) ff_add(hiC[q], loC[q], sC[q]);
     }
   }
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
+  for (int q = 0; q < 2; ++q) {
     if (!ok[q]) continue;
     constexpr int na = WC ? 3 : 2;  // the layout k_col_fin reads for this pass
     part[((int64_t)split * na + 0) * m + jj[q]] = (double)hiA[q] + (double)loA[q];
@@ -716,8 +750,7 @@ static cudaError_t launch_pts(const float* Pout, const float* Pin, int64_t nout,
   int64_t tin = cdiv(nin, kPT);
   int tps = (int)cdiv(tin, splits);
   dim3 grid((unsigned)cdiv(nout, kPT), (unsigned)splits);
-  kern<<<grid, kThreads, sm, st>>>(Pout, Pin, nout, nin, d, io, part, pmax, tps, dev, k, V);
-  return cudaGetLastError();
+  return launch_kernel(kern, grid, kThreads, sm, st, Pout, Pin, nout, nin, d, io, part, pmax, tps, dev, k, V);
 }
 
 // the packed direct-form sweeps serve |x - y|^2 with d <= 8 in float32
@@ -792,13 +825,8 @@ static cudaError_t launch_row_sweep(const Inputs& in, const Consts& k, const Wor
     int64_t nch = cdiv(k.m, kDChunk);
     int cps = (int)cdiv(nch, g.rows_split);
     dim3 grid((unsigned)cdiv(k.n, kDR), (unsigned)g.rows_split);
-    if (mode == M_ROWSUM)
-      k_dense_rows<M_ROWSUM><<<grid, kThreads, 0, st>>>(in.C, in.ldc, k.n, k.m, w, cps, k);
-    else if (mode == M_MAX2)
-      k_dense_rows<M_MAX2><<<grid, kThreads, 0, st>>>(in.C, in.ldc, k.n, k.m, w, cps, k);
-    else
-      k_dense_rows<M_MAX><<<grid, kThreads, 0, st>>>(in.C, in.ldc, k.n, k.m, w, cps, k);
-    return cudaGetLastError();
+    const auto kern = mode == M_ROWSUM ? k_dense_rows<M_ROWSUM> : mode == M_MAX2 ? k_dense_rows<M_MAX2> : k_dense_rows<M_MAX>;
+    return launch_kernel(kern, grid, kThreads, 0, st, in.C, in.ldc, k.n, k.m, w, cps, k);
   }
   if (mode == M_ROWSUM && k.shared_shift) return launch_direct_sweep(true, 0, in, k, w, g, st);
   if (k.shared_shift) return direct_max(mode == M_MAX2 ? kDirectMax2 : kDirectMax, in, w, k, g.rows_split, st);
@@ -822,12 +850,8 @@ static cudaError_t launch_col_sweep(const Inputs& in, const Consts& k, const Wor
   if (k.kind == COST_DENSE) {
     int64_t rps = cdiv(k.n, g.cols_split);
     rps = cdiv(rps, kDColRows) * kDColRows;
-    dim3 grid((unsigned)cdiv(k.m, kDChunk), (unsigned)g.cols_split);
-    if (eval)
-      k_dense_cols<1><<<grid, kThreads, 0, st>>>(in.C, in.ldc, k.n, k.m, w, rps, k);
-    else
-      k_dense_cols<0><<<grid, kThreads, 0, st>>>(in.C, in.ldc, k.n, k.m, w, rps, k);
-    return cudaGetLastError();
+    dim3 grid((unsigned)cdiv(k.m, kDCols), (unsigned)g.cols_split);
+    return launch_kernel(eval ? k_dense_cols<1> : k_dense_cols<0>, grid, kDColThreads, 0, st, in.C, in.ldc, k.n, k.m, w, rps, k);
   }
   if (k.shared_shift) return launch_direct_sweep(false, eval, in, k, w, g, st);
   if (k.zdot) return dot_launch(eval ? kDotColSumCost : kDotColSum, w, k, g, st);
@@ -918,10 +942,9 @@ void prepare_kernels() {
 int sweep_blocks_per_sm(const Consts& k, int prec, int which) {
   int nb = 0;
   if (k.kind == COST_DENSE) {
-    if (which == 0)
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_dense_rows<M_ROWSUM>, kThreads, 0);
-    else
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_dense_cols<1>, kThreads, 0);
+    // the splits decide how the float32 partial sums are grouped: they stay those of the tiles
+    // below at two (rows) and three (columns) CTAs per SM, whatever the kernels' grids
+    nb = which == 0 ? 2 : 3;
   } else if (uses_direct_sweeps(k, prec)) {
     nb = direct_blocks_per_sm();
   } else {
@@ -937,7 +960,7 @@ int sweep_blocks_per_sm(const Consts& k, int prec, int which) {
 // fixed / streamed points per CTA of each sweep (the split choice of lamp_create uses them)
 int tile_outer(const Consts& k, int prec) {
   if (prec == 1 /* LAMP_PREC_BF16_TC */) return tc_tile_fixed();
-  return k.kind == COST_DENSE ? kDR : uses_direct_sweeps(k, prec) ? direct_outer(k.d) : kPT;
+  return k.kind == COST_DENSE ? kDSplitRows : uses_direct_sweeps(k, prec) ? direct_outer(k.d) : kPT;
 }
 int tile_inner(const Consts& k, int prec) {
   if (prec == 1) return tc_tile_stream();

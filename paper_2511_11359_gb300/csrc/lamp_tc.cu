@@ -622,13 +622,8 @@ cudaError_t tc_launch_sweep(bool rows, int eval, const Geometry& g, const Work& 
   // G1: x fixed (128-row boxes), y streamed (64-row boxes); G2: the reverse
   const CUtensorMap& mf = *reinterpret_cast<const CUtensorMap*>(rows ? g.map_x : g.map_y);
   const CUtensorMap& ms = *reinterpret_cast<const CUtensorMap*>(rows ? g.map_y64 : g.map_x64);
-  if (rows)
-    tc::k_tc_sweep<true, 0><<<grid, tc::kThreads, tc_smem_bytes(), st>>>(mf, ms, w, k.n, k.m, tps, k);
-  else if (eval)
-    tc::k_tc_sweep<false, 1><<<grid, tc::kThreads, tc_smem_bytes(), st>>>(mf, ms, w, k.n, k.m, tps, k);
-  else
-    tc::k_tc_sweep<false, 0><<<grid, tc::kThreads, tc_smem_bytes(), st>>>(mf, ms, w, k.n, k.m, tps, k);
-  return cudaGetLastError();
+  const auto kern = rows ? tc::k_tc_sweep<true, 0> : eval ? tc::k_tc_sweep<false, 1> : tc::k_tc_sweep<false, 0>;
+  return launch_kernel(kern, grid, tc::kThreads, tc_smem_bytes(), st, mf, ms, w, k.n, k.m, tps, k);
 }
 
 // row maxima on the tensor cores: mode 1 = the prime pass (a z - Bq, no row shift), mode 2 =
