@@ -438,8 +438,9 @@ static int create_impl(lamp_ctx** out, const lamp_problem* prob, const lamp_para
   if (ctx->prec == LAMP_PREC_BF16_TC || k.shared_shift) {
     for (int b = 0; b < 2; ++b)
       if ((rc = dalloc(ctx, &w.colq2[b], pm_pad))) return bail(rc);
-    if ((rc = dalloc(ctx, &w.g2row2, pn_pad))) return bail(rc);
   }
+  // the packed row data also feed the column sweep of a stored cost
+  if ((w.colq2[0] || g.map_c) && (rc = dalloc(ctx, &w.g2row2, pn_pad))) return bail(rc);
   if ((rc = dalloc(ctx, &w.rowpart, (size_t)g.rows_split * ctx->part_width * n))) return bail(rc);
   if ((rc = dalloc(ctx, &w.colpart, (size_t)g.cols_split * ctx->part_width * m))) return bail(rc);
   if ((rc = dalloc(ctx, &w.logZ, n))) return bail(rc);
@@ -468,11 +469,11 @@ static int create_impl(lamp_ctx** out, const lamp_problem* prob, const lamp_para
     tc_fill_pads(w.colq[0], k.m, (int64_t)pm_pad, ctx->stream);
     tc_fill_pads(w.colq[1], k.m, (int64_t)pm_pad, ctx->stream);
     tc_fill_pads(w.g2row, k.n, (int64_t)pn_pad, ctx->stream);
-    if (w.g2row2) {
+    if (w.colq2[0]) {
       tc_fill_pairs(w.colq2[0], (int64_t)pm_pad, ctx->stream);
       tc_fill_pairs(w.colq2[1], (int64_t)pm_pad, ctx->stream);
-      tc_fill_pairs(w.g2row2, (int64_t)pn_pad, ctx->stream);
     }
+    if (w.g2row2) tc_fill_pairs(w.g2row2, (int64_t)pn_pad, ctx->stream);
     cudaMemsetAsync(w.nu[0], 0, m * sizeof(double), ctx->stream);
     cudaMemsetAsync(w.theta[0], 0, m * sizeof(double), ctx->stream);
     cudaMemsetAsync(w.nu[1], 0, m * sizeof(double), ctx->stream);

@@ -263,18 +263,32 @@ __device__ __forceinline__ void ff_add(float& hi, float& lo, float x) {
   lo += e;
 }
 
-// warp sum of float-float values (hi, lo): TwoSum of the high parts, low parts and their
-// errors added; the sweeps' per-thread sums are reduced in float32 arithmetic (the FP64
-// rate of this part is a small fraction of FP32) and converted once
-__device__ __forceinline__ void warp_sum_ff(float& hi, float& lo) {
+// sums over a warp of NV = 16, 8 or 4 float-float values (hi, lo) per lane: TwoSum of the high
+// parts, low parts and their errors added, in the order of a butterfly xor 16, 8, 4, 2, 1 (the
+// sweeps' per-thread sums are reduced in float32 arithmetic and converted once; the FP64 rate of
+// this part is a small fraction of FP32).  Each level halves the values a lane carries until one is left (the operands of
+// TwoSum and of its low parts' sum commute, so the results are the same), NV + 1 TwoSums for 16
+// values instead of 80.  Value q ends in the lanes with lane * NV / 32 == q.
+template <int NV>
+__device__ __forceinline__ void warp_sums_ff(float (&hi)[NV], float (&lo)[NV], int lane) {
+  int nv = NV;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
-    const float h2 = __shfl_xor_sync(0xffffffffu, hi, o);
-    const float l2 = __shfl_xor_sync(0xffffffffu, lo, o);
-    float sum, err;
-    two_sum(hi, h2, sum, err);
-    hi = sum;
-    lo = lo + l2 + err;
+    const bool up = (lane & o) != 0;
+    const int half = nv > 1 ? nv / 2 : 0;
+    const int cnt = nv > 1 ? half : 1;
+#pragma unroll
+    for (int q = 0; q < NV; ++q) {
+      if (q >= cnt) continue;
+      const float kh = half ? (up ? hi[half + q] : hi[q]) : hi[q], kl = half ? (up ? lo[half + q] : lo[q]) : lo[q];
+      const float gh = half ? (up ? hi[q] : hi[half + q]) : hi[q], gl = half ? (up ? lo[q] : lo[half + q]) : lo[q];
+      const float h2 = __shfl_xor_sync(0xffffffffu, gh, o), l2 = __shfl_xor_sync(0xffffffffu, gl, o);
+      float sum, err;
+      two_sum(kh, h2, sum, err);
+      hi[q] = sum;
+      lo[q] = kl + l2 + err;
+    }
+    nv = cnt;
   }
 }
 #endif
@@ -364,7 +378,8 @@ struct Work {
   // for entries 2p, 2p+1 two float4, [2p] = {-offA_2p, -offA_2p+1, wgtA_2p, wgtA_2p+1}
   // and [2p+1] = {dB_2p, dB_2p+1, wgtB_2p, wgtB_2p+1}: columns dB = BqA - BcolB, the
   // term stream B adds to stream A's exponent under the shared row shift; rows dB = 0
-  // (unused); padding halves hold {-2^100, 0}
+  // (unused), or -RqB where the streams have shifts of their own (stored costs); padding
+  // halves hold {-2^100, 0}
   float4* colq2[2];
   float4* g2row2;
   double* rowpart;     // [splits_rows][2][n] partial row sums

@@ -228,7 +228,7 @@ k_row_fin(const Work w, int splits, const double* __restrict__ r, int rowblocks,
       const float q = (float)div_seeded(ri, S);
       reinterpret_cast<float2*>(w.g2row + i)[1] = make_float2(rq.y, q);
       if (w.g2row2) {
-        store_pair_field(w.g2row2, i, 2, 0.f);
+        store_pair_field(w.g2row2, i, 2, k.shared_shift ? 0.f : -rq.y);
         store_pair_field(w.g2row2, i, 3, q);
       }
       if (!EVAL) ls = log2_table(S, stab);

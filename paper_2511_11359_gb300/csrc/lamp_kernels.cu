@@ -363,33 +363,6 @@ constexpr int kDR = 4;          // rows per CTA in the row sweep
 constexpr int kDSplitRows = 8;  // rows per tile in the choice of its splits
 constexpr int kDChunk = 1024;   // columns per CTA step (4 per thread, stride 256)
 
-// sums over a warp of NV = 16, 8 or 4 float-float values per lane, as warp_sum_ff adds them (xor
-// 16, 8, 4, 2, 1); each level halves the values a lane carries until one is left (the operands of
-// TwoSum and of its low parts' sum commute, so the results are the same), NV + 1 TwoSums for 16
-// values instead of 80.  Value q ends in the lanes with lane * NV / 32 == q.
-template <int NV>
-__device__ __forceinline__ void warp_sums_ff(float (&hi)[NV], float (&lo)[NV], int lane) {
-  int nv = NV;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const bool up = (lane & o) != 0;
-    const int half = nv > 1 ? nv / 2 : 0;
-    const int cnt = nv > 1 ? half : 1;
-#pragma unroll
-    for (int q = 0; q < NV; ++q) {
-      if (q >= cnt) continue;
-      const float kh = half ? (up ? hi[half + q] : hi[q]) : hi[q], kl = half ? (up ? lo[half + q] : lo[q]) : lo[q];
-      const float gh = half ? (up ? hi[q] : hi[half + q]) : hi[q], gl = half ? (up ? lo[q] : lo[half + q]) : lo[q];
-      const float h2 = __shfl_xor_sync(0xffffffffu, gh, o), l2 = __shfl_xor_sync(0xffffffffu, gl, o);
-      float sum, err;
-      two_sum(kh, h2, sum, err);
-      hi[q] = sum;
-      lo[q] = kl + l2 + err;
-    }
-    nv = cnt;
-  }
-}
-
 template <int MODE>  // M_ROWSUM, M_MAX or M_MAX2
 __global__ void __launch_bounds__(kThreads, 3)
 k_dense_rows(const float* __restrict__ C, int64_t ldc, int64_t n, int64_t m, const Work w,
