@@ -1,5 +1,5 @@
 // Host side of the LAMP C ABI (include/lamp.h): validation, the O(n + m) workspace,
-// the device loop (CUDA graphs of whole iterations, polled every check_every
+// the device loop (whole iterations, as CUDA graphs in longer runs, polled every check_every
 // iterations) and the O(1) bookkeeping of the objective (App. D identity,
 // Prop. infeas_bound (a)).
 #include <algorithm>
@@ -35,10 +35,13 @@ struct lamp_ctx {
   float* own_b = nullptr;  // y
   double* own_r = nullptr;
   double* own_c = nullptr;
-  // graph slots: 0 = one iteration, 1 = check_every iterations, 2 = one evaluation pass
-  cudaGraphExec_t gexec[3] = {nullptr, nullptr, nullptr};
-  int64_t glen[3] = {0, 0, 0};
-  DevState* host_dev = nullptr;  // pinned mirror for polling
+  // graph slots: 0 = one iteration, 1 = check_every iterations (see run_passes)
+  cudaGraphExec_t gexec[2] = {nullptr, nullptr};
+  int64_t glen[2] = {0, 0};
+  DevState host_mirror{};        // host copy of the control block, filled by poll()
+  DevState* host_dev = &host_mirror;
+  int64_t t_host = 0;    // the state's iteration index as far as the host knows (errors stop it short)
+  int64_t launched = 0;  // passes launched so far, see run_passes
   // LAMP_PREC_BF16_TC: bf16 copies (zero padded to 128-row multiples x 64 coordinates),
   // float32 copies of the rounded points, and their TMA descriptors
   void* xb = nullptr;
@@ -208,13 +211,14 @@ static int choose_split(int64_t tout, int64_t tin, int64_t wave, int64_t min_inn
 
 static int build_graph(lamp_ctx* ctx, int slot, int64_t len) {
   if (ctx->gexec[slot] && ctx->glen[slot] == len) return LAMP_OK;
+  if (!ctx->cap) CK(cudaStreamCreateWithFlags(&ctx->cap, cudaStreamNonBlocking));
   if (ctx->gexec[slot]) {
     cudaGraphExecDestroy(ctx->gexec[slot]);
     ctx->gexec[slot] = nullptr;
   }
   CK(cudaStreamBeginCapture(ctx->cap, cudaStreamCaptureModeThreadLocal));
   for (int64_t i = 0; i < len; ++i) {
-    cudaError_t e = launch_iteration(ctx->in, ctx->k, ctx->w, ctx->g, ctx->prec, slot == 2, ctx->cap);
+    cudaError_t e = launch_iteration(ctx->in, ctx->k, ctx->w, ctx->g, ctx->prec, 0, ctx->cap);
     if (e != cudaSuccess) {
       cudaGraph_t gg;
       cudaStreamEndCapture(ctx->cap, &gg);
@@ -256,6 +260,7 @@ __global__ void k_set_state(DevState* dev, long long t, double kappa) {
 static int poll(lamp_ctx* ctx) {
   CK(cudaMemcpyAsync(ctx->host_dev, ctx->w.dev, sizeof(DevState), cudaMemcpyDeviceToHost, ctx->stream));
   CK(cudaStreamSynchronize(ctx->stream));
+  ctx->t_host = ctx->host_dev->t;
   return LAMP_OK;
 }
 
@@ -326,11 +331,6 @@ static int create_impl(lamp_ctx** out, const lamp_problem* prob, const lamp_para
   k.clipb = std::tanh(params->beta / 2.0);
   ctx->log_m = std::log((double)k.m);
 
-  if (cudaStreamCreateWithFlags(&ctx->cap, cudaStreamNonBlocking) != cudaSuccess) {
-    fail(nullptr, LAMP_E_CUDA, "cudaStreamCreate failed");
-    delete ctx;
-    return LAMP_E_CUDA;
-  }
   // inputs
   Inputs& in = ctx->in;
   if (owned) {
@@ -374,10 +374,8 @@ static int create_impl(lamp_ctx** out, const lamp_problem* prob, const lamp_para
   // geometry
   Geometry& g = ctx->g;
   {
-    cudaDeviceProp prop;
-    cudaError_t e = cudaGetDeviceProperties(&prop, ctx->device);
-    if (e != cudaSuccess) return bail(fail(ctx, LAMP_E_CUDA, "cudaGetDeviceProperties: %s", cudaGetErrorString(e)));
-    g.sms = prop.multiProcessorCount;
+    cudaError_t e = cudaDeviceGetAttribute(&g.sms, cudaDevAttrMultiProcessorCount, ctx->device);
+    if (e != cudaSuccess) return bail(fail(ctx, LAMP_E_CUDA, "cudaDeviceGetAttribute: %s", cudaGetErrorString(e)));
   }
   {
     const bool tcp = ctx->prec == LAMP_PREC_BF16_TC;
@@ -428,36 +426,65 @@ static int create_impl(lamp_ctx** out, const lamp_problem* prob, const lamp_para
   // row sweep reads the data of 256 columns per tile); padding entries contribute nothing
   const size_t m_pad = (size_t)tc_pad(k.m), n_pad = (size_t)tc_pad(k.n);
   const size_t pm_pad = (m_pad + 255) / 256 * 256, pn_pad = (n_pad + 255) / 256 * 256;
+  // one allocation for everything the context keeps from here on (36 allocations and their frees
+  // took 0.5 ms of a context's life), each buffer on a 256-byte boundary
+  std::vector<std::pair<void**, size_t>> want;
+  const auto need = [&](auto** p, size_t count) {
+    want.emplace_back(reinterpret_cast<void**>(p), std::max<size_t>(count, 1) * sizeof(**p));
+  };
   for (int b = 0; b < 2; ++b) {
-    if ((rc = dalloc(ctx, &w.nu[b], m))) return bail(rc);
-    if ((rc = dalloc(ctx, &w.theta[b], m))) return bail(rc);
-    if ((rc = dalloc(ctx, &w.colq[b], pm_pad))) return bail(rc);
-    if ((rc = dalloc(ctx, &w.rowshift[b], n))) return bail(rc);
+    need(&w.nu[b], m);
+    need(&w.theta[b], m);
+    need(&w.colq[b], pm_pad);
+    need(&w.rowshift[b], n);
   }
-  if ((rc = dalloc(ctx, &w.g2row, pn_pad))) return bail(rc);
-  if (ctx->prec == LAMP_PREC_BF16_TC || k.shared_shift) {
-    for (int b = 0; b < 2; ++b)
-      if ((rc = dalloc(ctx, &w.colq2[b], pm_pad))) return bail(rc);
-  }
+  need(&w.g2row, pn_pad);
+  const bool packed = ctx->prec == LAMP_PREC_BF16_TC || k.shared_shift;
+  if (packed)
+    for (int b = 0; b < 2; ++b) need(&w.colq2[b], pm_pad);
   // the packed row data also feed the column sweep of a stored cost
-  if ((w.colq2[0] || g.map_c) && (rc = dalloc(ctx, &w.g2row2, pn_pad))) return bail(rc);
-  if ((rc = dalloc(ctx, &w.rowpart, (size_t)g.rows_split * ctx->part_width * n))) return bail(rc);
-  if ((rc = dalloc(ctx, &w.colpart, (size_t)g.cols_split * ctx->part_width * m))) return bail(rc);
-  if ((rc = dalloc(ctx, &w.logZ, n))) return bail(rc);
-  if ((rc = dalloc(ctx, &w.colA, m))) return bail(rc);
-  if ((rc = dalloc(ctx, &w.colz, m))) return bail(rc);
-  if ((rc = dalloc(ctx, &w.gj, m))) return bail(rc);
-  if ((rc = dalloc(ctx, &w.rscr, rscr_doubles(k.n, k.m, k.kind == LAMP_COST_SQEUCLID ? (int)k.d : 0)))) return bail(rc);
-  if ((rc = dalloc(ctx, &w.nx, n))) return bail(rc);
-  if ((rc = dalloc(ctx, &w.ny, m))) return bail(rc);
-  if ((rc = dalloc(ctx, &w.rowred, (size_t)fin_groups(k.n)))) return bail(rc);
-  if ((rc = dalloc(ctx, &w.colred, (size_t)fin_groups(k.m) * 3))) return bail(rc);
-  if ((rc = dalloc(ctx, &w.rowmax, (size_t)g.rows_split * 2 * n))) return bail(rc);
-  if ((rc = dalloc(ctx, &w.scratch, (size_t)std::max(3 * 4 * g.sms, 3 * 128)))) return bail(rc);
-  if ((rc = dalloc(ctx, &w.dev, 1))) return bail(rc);
+  if (packed || g.map_c) need(&w.g2row2, pn_pad);
+  need(&w.rowpart, (size_t)g.rows_split * ctx->part_width * n);
+  need(&w.colpart, (size_t)g.cols_split * ctx->part_width * m);
+  need(&w.logZ, n);
+  need(&w.colA, m);
+  need(&w.colz, m);
+  need(&w.gj, m);
+  need(&w.rscr, rscr_doubles(k.n, k.m, k.kind == LAMP_COST_SQEUCLID ? (int)k.d : 0));
+  need(&w.nx, n);
+  need(&w.ny, m);
+  need(&w.rowred, (size_t)fin_groups(k.n));
+  need(&w.colred, (size_t)fin_groups(k.m) * 3);
+  need(&w.rowmax, (size_t)g.rows_split * 2 * n);
+  need(&w.scratch, (size_t)std::max(3 * 4 * g.sms, 3 * 128));
+  need(&w.stats, (size_t)kStatBlocks * kStatFields);
+  need(&w.dev, 1);
+  if (ctx->pub_kind == LAMP_COST_COSINE) {
+    need(&ctx->xn, n * (size_t)k.d);
+    need(&ctx->yn, m * (size_t)k.d);
+  }
+  uint16_t *xb = nullptr, *yb = nullptr;
+  if (ctx->prec == LAMP_PREC_BF16_TC) {
+    need(&xb, n_pad * 64);
+    need(&yb, m_pad * 64);
+    need(&ctx->xr, n * (size_t)k.d);
+    need(&ctx->yr, m * (size_t)k.d);
+  } else if (k.zdot) {
+    need(&w.xt, (size_t)dot_pad(k.n) * k.d);
+    need(&w.yt, (size_t)dot_pad(k.m) * k.d);
+  }
   {
-    cudaError_t e = cudaMallocHost(&ctx->host_dev, sizeof(DevState));
-    if (e != cudaSuccess) return bail(fail(ctx, LAMP_E_NOMEM, "cudaMallocHost: %s", cudaGetErrorString(e)));
+    const auto padded = [](size_t bytes) { return (bytes + 255) / 256 * 256; };
+    size_t total = 0;
+    for (const auto& q : want) total += padded(q.second);
+    unsigned char* base = nullptr;
+    if ((rc = dalloc(ctx, &base, total))) return bail(rc);
+    for (const auto& q : want) {
+      *q.first = base;
+      base += padded(q.second);
+    }
+    ctx->xb = xb;
+    ctx->yb = yb;
   }
   std::memset(ctx->host_dev, 0, sizeof(DevState));
   ctx->host_dev->swf_kap = -1.0;  // no cached sweep constants yet (kappa >= 0 always)
@@ -480,51 +507,16 @@ static int create_impl(lamp_ctx** out, const lamp_problem* prob, const lamp_para
     cudaMemsetAsync(w.theta[1], 0, m * sizeof(double), ctx->stream);
   }
 
-  // marginals: positive, finite, summing to one (r in Delta^n, c in Delta^m, full support)
-  {
-    cudaError_t e = launch_check_marginals(in, k, w, ctx->stream);
-    if (e != cudaSuccess) return bail(fail(ctx, LAMP_E_CUDA, "marginal check: %s", cudaGetErrorString(e)));
-    std::vector<double> h(3 * 128);
-    e = cudaMemcpyAsync(h.data(), w.scratch, h.size() * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
-    if (e != cudaSuccess) return bail(fail(ctx, LAMP_E_CUDA, "marginal check: %s", cudaGetErrorString(e)));
-    for (int which = 0; which < 2; ++which) {
-      double S = 0, M = INFINITY, B = 0;
-      for (int b = 0; b < 64; ++b) {
-        S += h[which * 192 + 3 * b];
-        M = std::min(M, h[which * 192 + 3 * b + 1]);
-        B = std::max(B, h[which * 192 + 3 * b + 2]);
-      }
-      if (B != 0.0 || !(M > 0.0) || std::fabs(S - 1.0) > 1e-9)
-        return bail(fail(ctx, LAMP_E_INVALID, "%s must be positive, finite and sum to 1 (sum-1=%.3e, min=%.3e)",
-                         which ? "c" : "r", S - 1.0, M));
-    }
-  }
-  // H(r) on the host needs r: copy it once (O(n))
-  {
-    std::vector<double> hr(n);
-    cudaError_t e = cudaMemcpyAsync(hr.data(), in.r, n * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
-    if (e != cudaSuccess) return bail(fail(ctx, LAMP_E_CUDA, "copy r: %s", cudaGetErrorString(e)));
-    double H = 0.0;
-    for (double v : hr) H -= v * std::log(v);
-    ctx->Hr = H;
-  }
-
+  unsigned int hbad = 0;  // points without a direction (cosine cost)
   // cosine cost: every kernel reads unit-scaled copies u = x / (sqrt 2 |x|), v = y / (sqrt 2 |y|)
   // (then |u - v|^2 = 1 - cos(x, y), see lamp.h)
   if (ctx->pub_kind == LAMP_COST_COSINE) {
-    if ((rc = dalloc(ctx, &ctx->xn, n * (size_t)k.d))) return bail(rc);
-    if ((rc = dalloc(ctx, &ctx->yn, m * (size_t)k.d))) return bail(rc);
     unsigned int* bad = reinterpret_cast<unsigned int*>(w.scratch);
-    unsigned int hbad = 0;
     cudaError_t e = cudaMemsetAsync(bad, 0, sizeof(unsigned int), ctx->stream);
     if (e == cudaSuccess) e = launch_unit_rows(in.x, k.n, k.d, ctx->xn, bad, ctx->stream);
     if (e == cudaSuccess) e = launch_unit_rows(in.y, k.m, k.d, ctx->yn, bad, ctx->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(&hbad, bad, sizeof(hbad), cudaMemcpyDeviceToHost, ctx->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
     if (e != cudaSuccess) return bail(fail(ctx, LAMP_E_CUDA, "cosine normalisation: %s", cudaGetErrorString(e)));
-    if (hbad) return bail(fail(ctx, LAMP_E_INVALID, "cosine cost needs nonzero finite points (%u are not)", hbad));
     in.x = ctx->xn;
     in.y = ctx->yn;
   }
@@ -533,10 +525,6 @@ static int create_impl(lamp_ctx** out, const lamp_problem* prob, const lamp_para
   // gradient) then read the float32 copies of the rounded points, so every kernel
   // solves the problem of the rounded points
   if (ctx->prec == LAMP_PREC_BF16_TC) {
-    if ((rc = dalloc(ctx, reinterpret_cast<uint16_t**>(&ctx->xb), n_pad * 64))) return bail(rc);
-    if ((rc = dalloc(ctx, reinterpret_cast<uint16_t**>(&ctx->yb), m_pad * 64))) return bail(rc);
-    if ((rc = dalloc(ctx, &ctx->xr, n * (size_t)k.d))) return bail(rc);
-    if ((rc = dalloc(ctx, &ctx->yr, m * (size_t)k.d))) return bail(rc);
     cudaError_t e = tc_convert(in.x, k.n, k.d, ctx->xr, ctx->xb, ctx->stream);
     if (e == cudaSuccess) e = tc_convert(in.y, k.m, k.d, ctx->yr, ctx->yb, ctx->stream);
     if (e == cudaSuccess) e = tc_make_map(ctx->map_x, ctx->xb, (int64_t)n_pad, tc_tile_fixed() / 2);
@@ -554,7 +542,8 @@ static int create_impl(lamp_ctx** out, const lamp_problem* prob, const lamp_para
 
   if (k.zdot && ctx->prec == LAMP_PREC_FP32 && (rc = ensure_dot_copies(ctx))) return bail(rc);
 
-  // cost scale and K = ||C||_inf of the cost the kernels use
+  // cost scale and K = ||C||_inf of the cost the kernels use, and the checks of the inputs
+  double nxmax = 0.0, nymax = 0.0, rnx = 0.0;
   {
     cudaError_t e = launch_norms(in, k, w, ctx->stream);
     if (e != cudaSuccess) return bail(fail(ctx, LAMP_E_CUDA, "norms: %s", cudaGetErrorString(e)));
@@ -562,41 +551,56 @@ static int create_impl(lamp_ctx** out, const lamp_problem* prob, const lamp_para
     bool need_scale = pts && prob->cost_scale < 0.0;
     double s = pts ? (prob->cost_scale > 0.0 ? prob->cost_scale : 1.0) : 1.0;
     double Dmax = NAN, Dmin = NAN;
-    if (need_K || need_scale || prob->kind == LAMP_COST_DENSE) {
+    const bool dense = prob->kind == LAMP_COST_DENSE, kpass = need_K || need_scale || dense;
+    std::vector<double> hd(dense ? 3 * 4 * g.sms : 0), hs((size_t)kStatBlocks * kStatFields);
+    if (kpass) {
       k.K = 1.0;
       k.s = s;
       e = launch_kmax(in, k, w, g, ctx->prec, ctx->stream);
       if (e != cudaSuccess) return bail(fail(ctx, LAMP_E_CUDA, "K pass: %s", cudaGetErrorString(e)));
-      if (prob->kind == LAMP_COST_DENSE) {
-        std::vector<double> h(3 * 4 * g.sms);
-        e = cudaMemcpyAsync(h.data(), w.scratch, h.size() * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
-        if (e != cudaSuccess) return bail(fail(ctx, LAMP_E_CUDA, "K pass: %s", cudaGetErrorString(e)));
-        Dmax = -INFINITY;
-        Dmin = INFINITY;
-        double bad = 0;
-        for (int b = 0; b < 4 * g.sms; ++b) {
-          Dmax = std::max(Dmax, h[3 * b]);
-          Dmin = std::min(Dmin, h[3 * b + 1]);
-          bad = std::max(bad, h[3 * b + 2]);
-        }
-        if (bad != 0.0 || !(Dmin >= 0.0))
-          return bail(fail(ctx, LAMP_E_INVALID, "C must be finite and >= 0 (min %.3e)", Dmin));
-      } else {
-        std::vector<float> h((size_t)g.rows_split * 2 * n);
-        e = cudaMemcpyAsync(h.data(), w.rowmax, h.size() * sizeof(float), cudaMemcpyDeviceToHost, ctx->stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
-        if (e != cudaSuccess) return bail(fail(ctx, LAMP_E_CUDA, "K pass: %s", cudaGetErrorString(e)));
-        float mx = -INFINITY, mnneg = -INFINITY;
-        for (int sp = 0; sp < g.rows_split; ++sp)
-          for (size_t i = 0; i < n; ++i) {
-            mx = std::max(mx, h[(sp * 2 + 0) * n + i]);
-            mnneg = std::max(mnneg, h[(sp * 2 + 1) * n + i]);
-          }
-        Dmax = mx;
-        Dmin = -(double)mnneg;
-        if (!std::isfinite(Dmax)) return bail(fail(ctx, LAMP_E_INVALID, "points must be finite"));
+    }
+    // everything the host needs of the inputs, in one reduction and one synchronisation
+    e = launch_create_stats(in, k, w, g, kpass, ctx->stream);
+    if (e == cudaSuccess && dense)
+      e = cudaMemcpyAsync(hd.data(), w.scratch, hd.size() * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(hs.data(), w.stats, hs.size() * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
+    if (e != cudaSuccess) return bail(fail(ctx, LAMP_E_CUDA, "input statistics: %s", cudaGetErrorString(e)));
+    double v[kStatFields];
+    for (int q = 0; q < kStatFields; ++q) v[q] = hs[q];
+    for (int b = 1; b < kStatBlocks; ++b)
+      for (int q = 0; q < kStatFields; ++q) {
+        const double x = hs[(size_t)b * kStatFields + q];
+        v[q] = q == 0 || q == 3 || q == 4 || q == 6 ? v[q] + x : q == 1 || q == 7 ? std::min(v[q], x) : std::max(v[q], x);
       }
+    // marginals: positive, finite, summing to one (r in Delta^n, c in Delta^m, full support)
+    for (int which = 0; which < 2; ++which) {
+      const double S = v[6 * which], M = v[6 * which + 1], B = v[6 * which + 2];
+      if (B != 0.0 || !(M > 0.0) || !(std::fabs(S - 1.0) <= 1e-9))
+        return bail(fail(ctx, LAMP_E_INVALID, "%s must be positive, finite and sum to 1 (sum-1=%.3e, min=%.3e)",
+                         which ? "c" : "r", S - 1.0, M));
+    }
+    ctx->Hr = v[3];
+    if (hbad) return bail(fail(ctx, LAMP_E_INVALID, "cosine cost needs nonzero finite points (%u are not)", hbad));
+    nxmax = v[5];
+    nymax = v[9];
+    rnx = v[4];
+    if (dense) {
+      Dmax = -INFINITY;
+      Dmin = INFINITY;
+      double bad = 0;
+      for (int b = 0; b < 4 * g.sms; ++b) {
+        Dmax = std::max(Dmax, hd[3 * b]);
+        Dmin = std::min(Dmin, hd[3 * b + 1]);
+        bad = std::max(bad, hd[3 * b + 2]);
+      }
+      if (bad != 0.0 || !(Dmin >= 0.0))
+        return bail(fail(ctx, LAMP_E_INVALID, "C must be finite and >= 0 (min %.3e)", Dmin));
+    } else if (kpass) {
+      Dmax = v[10];
+      Dmin = -v[11];
+      if (!std::isfinite(Dmax)) return bail(fail(ctx, LAMP_E_INVALID, "points must be finite"));
     }
     if (need_scale) {
       if (!(Dmax > 0.0)) return bail(fail(ctx, LAMP_E_INVALID, "cost_scale < 0 needs a positive maximum cost"));
@@ -617,19 +621,7 @@ static int create_impl(lamp_ctx** out, const lamp_problem* prob, const lamp_para
     k.W = 5.0 * k.K;
     k.rnx = 0.0;
   } else {
-    std::vector<double> hx(n), hy(m), hr(n);
-    cudaError_t e = cudaMemcpyAsync(hx.data(), w.nx, n * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(hy.data(), w.ny, m * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(hr.data(), in.r, n * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
-    if (e != cudaSuccess) return bail(fail(ctx, LAMP_E_CUDA, "norm copy: %s", cudaGetErrorString(e)));
-    double nxm = 0, nym = 0, rnx = 0;
-    for (size_t i = 0; i < n; ++i) {
-      nxm = std::max(nxm, hx[i]);
-      rnx += hr[i] * hx[i];
-    }
-    for (size_t j = 0; j < m; ++j) nym = std::max(nym, hy[j]);
-    k.W = k.s * (nxm + 3.0 * nym) + 4.0 * k.K + 2.0 * k.s * (nxm + nym);
+    k.W = k.s * (nxmax + 3.0 * nymax) + 4.0 * k.K + 2.0 * k.s * (nxmax + nymax);
     k.rnx = k.s * rnx;
   }
 
@@ -655,10 +647,29 @@ extern "C" int lamp_create_owned(lamp_ctx** out, const lamp_problem* prob, const
   return create_impl(out, prob, params, stream, true);
 }
 
-static int run_graph(lamp_ctx* ctx, int slot, int64_t len) {
-  int rc = build_graph(ctx, slot, len);
-  if (rc) return rc;
-  CK(cudaGraphLaunch(ctx->gexec[slot], ctx->stream));
+// `passes` iterations' kernels on the context's stream.  A context's first kDirectPasses are
+// launched one by one: a graph of 50 iterations takes 0.17 ms to instantiate and 0.07 ms to
+// release, with the GPU idle, while the launches (about 2 us each) run ahead of kernels that take
+// longer.  Later ones are graphs of check_every iterations, or of one.
+constexpr int64_t kDirectPasses = 256;
+static int run_passes(lamp_ctx* ctx, int64_t passes) {
+  const int64_t L = ctx->params.check_every;
+  while (passes > 0) {
+    if (ctx->launched < kDirectPasses) {
+      cudaError_t e = launch_iteration(ctx->in, ctx->k, ctx->w, ctx->g, ctx->prec, 0, ctx->stream);
+      if (e != cudaSuccess) return fail(ctx, LAMP_E_CUDA, "launching an iteration: %s", cudaGetErrorString(e));
+      --passes;
+      ++ctx->launched;
+      continue;
+    }
+    const int slot = passes >= L ? 1 : 0;
+    const int64_t len = slot ? L : 1;
+    int rc = build_graph(ctx, slot, len);
+    if (rc) return rc;
+    CK(cudaGraphLaunch(ctx->gexec[slot], ctx->stream));
+    passes -= len;
+    ctx->launched += len;
+  }
   return LAMP_OK;
 }
 
@@ -695,7 +706,9 @@ extern "C" int lamp_solve(lamp_ctx* ctx, lamp_result* out) {
   int stop = 0;
   double gap = NAN;
   for (;;) {
-    int rc = run_graph(ctx, 1, L);
+    // X^t is evaluated for t = t_host .. max_iter at most; the gap test looks at every L-th state
+    const int64_t left = std::max<int64_t>(pa.max_iter - ctx->t_host, 0) + 1;
+    int rc = run_passes(ctx, use_gap ? L : std::min(L, left));
     if (rc) return rc;
     if ((rc = poll(ctx))) return rc;
     if (ctx->host_dev->done) break;
@@ -751,26 +764,14 @@ extern "C" int lamp_iterate(lamp_ctx* ctx, int64_t iters) {
   if (iters == 0) return LAMP_OK;
   k_ctrl<<<1, 1, 0, ctx->stream>>>(ctx->w.dev, 0, -1.0, 0, iters, 0);
   CK(cudaGetLastError());
-  const int64_t L = ctx->params.check_every;
-  int64_t left = iters;
-  while (left >= L && L > 1) {
-    int rc = run_graph(ctx, 1, L);
-    if (rc) return rc;
-    left -= L;
-  }
-  while (left > 0) {
-    int rc = run_graph(ctx, 0, 1);
-    if (rc) return rc;
-    --left;
-  }
-  return LAMP_OK;
+  ctx->t_host += iters;
+  return run_passes(ctx, iters);
 }
 
 static int evaluate(lamp_ctx* ctx) {
   k_ctrl<<<1, 1, 0, ctx->stream>>>(ctx->w.dev, 1, -1.0, 0, 0, 0);
   CK(cudaGetLastError());
-  int rc = run_graph(ctx, 2, 1);
-  if (rc) return rc;
+  CK(launch_iteration(ctx->in, ctx->k, ctx->w, ctx->g, ctx->prec, 1, ctx->stream));
   return poll(ctx);
 }
 
@@ -804,13 +805,14 @@ static int end_passes(lamp_ctx* ctx) {
 static int ensure_part_width(lamp_ctx* ctx, int width) {
   if (width <= ctx->part_width) return LAMP_OK;
   CK(cudaStreamSynchronize(ctx->stream));
+  // the first ones are part of the context's one allocation
   for (double* old : {ctx->w.rowpart, ctx->w.colpart}) {
     auto it = std::find(ctx->allocs.begin(), ctx->allocs.end(), (void*)old);
-    if (it != ctx->allocs.end()) ctx->allocs.erase(it);
+    if (it == ctx->allocs.end()) continue;
+    ctx->allocs.erase(it);
     cudaFree(old);
   }
-  ctx->w.rowpart = ctx->w.colpart = nullptr;
-  for (int s = 0; s < 3; ++s) {
+  for (int s = 0; s < 2; ++s) {
     if (ctx->gexec[s]) cudaGraphExecDestroy(ctx->gexec[s]);
     ctx->gexec[s] = nullptr;
     ctx->glen[s] = 0;
@@ -1088,6 +1090,7 @@ extern "C" int lamp_set_state(lamp_ctx* ctx, const double* nu, const double* the
   CK(cudaMemcpyAsync(ctx->w.theta[cur], theta, ctx->k.m * sizeof(double), cudaMemcpyHostToDevice, ctx->stream));
   k_set_state<<<1, 1, 0, ctx->stream>>>(ctx->w.dev, t, kappa);
   CK(cudaGetLastError());
+  ctx->t_host = t;
   if (row_shifts) {
     for (int64_t i = 0; i < 2 * ctx->k.n; ++i)
       if (!std::isfinite(row_shifts[i])) return fail(ctx, LAMP_E_INVALID, "row_shifts must be finite");
@@ -1222,10 +1225,9 @@ extern "C" const char* lamp_last_error(const lamp_ctx* ctx) { return ctx ? ctx->
 extern "C" void lamp_destroy(lamp_ctx* ctx) {
   if (!ctx) return;
   if (ctx->stream) cudaStreamSynchronize(ctx->stream);
-  for (int s = 0; s < 3; ++s)
+  for (int s = 0; s < 2; ++s)
     if (ctx->gexec[s]) cudaGraphExecDestroy(ctx->gexec[s]);
   for (void* p : ctx->allocs) cudaFree(p);
-  if (ctx->host_dev) cudaFreeHost(ctx->host_dev);
   if (ctx->cap) cudaStreamDestroy(ctx->cap);
   if (ctx->gside) {
     cudaStreamSynchronize(ctx->gside);

@@ -367,6 +367,8 @@ __device__ __forceinline__ void iteration_params_of(const DevState* dev, const C
 }
 #endif
 
+constexpr int kStatBlocks = 128, kStatFields = 12;  // k_create_stats
+
 // Device buffers of one context (all owned by the context).
 struct Work {
   double* nu[2];
@@ -398,7 +400,8 @@ struct Work {
   float* xt;           // [d][dot_pad(n)], [d][dot_pad(m)]: transposed copies of the points, zero padded
   float* yt;           // (float32 dot-form sweeps and gradient; null elsewhere)
   float* rowmax;       // [splits_rows][2][n] partial row maxima (prime pass)
-  double* scratch;     // small reduction scratch (K pass, marginal checks)
+  double* scratch;     // small reduction scratch (K pass of a stored cost, evaluation results)
+  double* stats;       // [kStatBlocks][kStatFields] (lamp_create)
   DevState* dev;
 };
 
@@ -431,7 +434,10 @@ cudaError_t launch_norms(const Inputs& in, const Consts& k, const Work& w, cudaS
 cudaError_t launch_unit_rows(const float* P, int64_t np, int d, float* out, unsigned int* bad, cudaStream_t st);
 cudaError_t launch_kmax(const Inputs& in, const Consts& k, const Work& w, const Geometry& g,
                         int prec, cudaStream_t st);
-cudaError_t launch_check_marginals(const Inputs& in, const Consts& k, const Work& w, cudaStream_t st);
+// what lamp_create reads back of its inputs (k_create_stats), per block in Work::stats; kpass: the K
+// pass of a point cloud has run
+cudaError_t launch_create_stats(const Inputs& in, const Consts& k, const Work& w, const Geometry& g, bool kpass,
+                                cudaStream_t st);
 cudaError_t launch_init_state(const Inputs& in, const Consts& k, const Work& w, int zero, cudaStream_t st);
 cudaError_t launch_prime(const Inputs& in, const Consts& k, const Work& w, const Geometry& g, int prec,
                          cudaStream_t st);

@@ -20,12 +20,6 @@ namespace lamp {
 // ------------------------------------------------------------------------------------------
 // small helpers
 
-__device__ __forceinline__ double warp_sum_d(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
 __device__ __forceinline__ float warp_max_f(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
@@ -630,30 +624,66 @@ __global__ void k_unit_rows(const float* __restrict__ P, int64_t np, int d, floa
   for (int q = 0; q < d; ++q) out[i * d + q] = (float)((double)P[i * d + q] * sc);
 }
 
-// marginal checks: sum, min, finiteness (block partials, 3 doubles per block)
-__global__ void k_vec_stats(const double* __restrict__ v, int64_t len, double* out) {
-  __shared__ double ssum[kThreads / 32], smn[kThreads / 32], sbad[kThreads / 32];
-  double s = 0.0, mn = INFINITY, bad = 0.0;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < len; i += (int64_t)gridDim.x * blockDim.x) {
-    double x = v[i];
-    if (!isfinite(x)) bad = 1.0;
-    s += x;
-    mn = fmin(mn, x);
+// what lamp_create reads back of its inputs, in one pass: per block kStatFields doubles
+//   0 sum r   1 min r   2 r not finite   3 -sum r log r   4 sum r |x|^2   5 max |x|^2
+//   6 sum c   7 min c   8 c not finite   9 max |y|^2   10 max of rowmax[.][0]   11 max of rowmax[.][1]
+// (nx, ny null: no norms; rows = 0: no K pass)
+__global__ void __launch_bounds__(kThreads)
+k_create_stats(const double* __restrict__ r, int64_t n, const double* __restrict__ c, int64_t m,
+               const double* __restrict__ nx, const double* __restrict__ ny, const float* __restrict__ rowmax,
+               int64_t rows, int splits, double* __restrict__ out) {
+  double v[kStatFields];
+#pragma unroll
+  for (int q = 0; q < kStatFields; ++q) v[q] = 0.0;
+  v[1] = v[7] = INFINITY;
+  float mx = -INFINITY, mn = -INFINITY;
+  const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t i = i0; i < n; i += step) {
+    const double x = r[i];
+    if (!isfinite(x)) v[2] = 1.0;
+    v[0] += x;
+    v[1] = fmin(v[1], x);
+    v[3] -= x * log(x);
+    if (nx) {
+      v[4] += x * nx[i];
+      v[5] = fmax(v[5], nx[i]);
+    }
   }
-  s = warp_sum_d(s);
-  for (int o = 16; o > 0; o >>= 1) {
-    mn = fmin(mn, __shfl_xor_sync(0xffffffffu, mn, o));
-    bad = fmax(bad, __shfl_xor_sync(0xffffffffu, bad, o));
+  for (int64_t j = i0; j < m; j += step) {
+    const double x = c[j];
+    if (!isfinite(x)) v[8] = 1.0;
+    v[6] += x;
+    v[7] = fmin(v[7], x);
+    if (ny) v[9] = fmax(v[9], ny[j]);
   }
-  int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (lane == 0) { ssum[wid] = s; smn[wid] = mn; sbad[wid] = bad; }
+  for (int s = 0; s < splits; ++s)
+    for (int64_t i = i0; i < rows; i += step) {
+      mx = fmaxf(mx, rowmax[((int64_t)s * 2 + 0) * rows + i]);
+      mn = fmaxf(mn, rowmax[((int64_t)s * 2 + 1) * rows + i]);
+    }
+  v[10] = mx;
+  v[11] = mn;
+  __shared__ double sh[kThreads / 32][kStatFields];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  // sums in the fields 0, 3, 4, 6; minima in 1, 7; maxima in the others
+#pragma unroll
+  for (int q = 0; q < kStatFields; ++q) {
+    const bool add = q == 0 || q == 3 || q == 4 || q == 6, low = q == 1 || q == 7;
+    double x = v[q];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const double y = __shfl_xor_sync(0xffffffffu, x, o);
+      x = add ? x + y : low ? fmin(x, y) : fmax(x, y);
+    }
+    if (lane == 0) sh[wid][q] = x;
+  }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double S = 0.0, M = INFINITY, B = 0.0;
-    for (int w = 0; w < kThreads / 32; ++w) { S += ssum[w]; M = fmin(M, smn[w]); B = fmax(B, sbad[w]); }
-    out[3 * blockIdx.x + 0] = S;
-    out[3 * blockIdx.x + 1] = M;
-    out[3 * blockIdx.x + 2] = B;
+  if (threadIdx.x < kStatFields) {
+    const int q = threadIdx.x;
+    const bool add = q == 0 || q == 3 || q == 4 || q == 6, low = q == 1 || q == 7;
+    double x = sh[0][q];
+    for (int u = 1; u < kThreads / 32; ++u) x = add ? x + sh[u][q] : low ? fmin(x, sh[u][q]) : fmax(x, sh[u][q]);
+    out[kStatFields * blockIdx.x + q] = x;
   }
 }
 
@@ -780,9 +810,11 @@ cudaError_t launch_kmax(const Inputs& in, const Consts& k, const Work& w, const 
                                w.rowmax, g.rows_split, w.dev, k, st);
 }
 
-cudaError_t launch_check_marginals(const Inputs& in, const Consts& k, const Work& w, cudaStream_t st) {
-  k_vec_stats<<<64, kThreads, 0, st>>>(in.r, k.n, w.scratch);
-  k_vec_stats<<<64, kThreads, 0, st>>>(in.c, k.m, w.scratch + 3 * 64);
+cudaError_t launch_create_stats(const Inputs& in, const Consts& k, const Work& w, const Geometry& g, bool kpass,
+                                cudaStream_t st) {
+  const bool pts = k.kind == COST_SQEUCLID;
+  k_create_stats<<<kStatBlocks, kThreads, 0, st>>>(in.r, k.n, in.c, k.m, pts ? w.nx : nullptr, pts ? w.ny : nullptr,
+                                                   w.rowmax, kpass && pts ? k.n : 0, g.rows_split, w.stats);
   return cudaGetLastError();
 }
 
