@@ -385,8 +385,9 @@ struct Work {
   float4* colq2[2];
   float4* g2row2;
   double* rowpart;     // [splits_rows][2][n] partial row sums
+                       // (evaluation passes: [splits_rows][n], stream A alone)
   double* colpart;     // [splits_cols][2][m] partial column sums (A, B); evaluation passes
-                       // [splits_cols][3][m] (A, B, cost-weighted A)
+                       // (A, cost-weighted A)
   double* gj;          // [m] 2 tau2 K / c^alpha_j, the gain of the mirror step
   double* logZ;        // [n] natural-log normalisers of X^t
   double* colA;        // [m] col(X^t)
@@ -445,8 +446,8 @@ cudaError_t launch_prime(const Inputs& in, const Consts& k, const Work& w, const
 // applied (Work::rowmax, stream A slot); the column data's second field holds Br_j
 cudaError_t launch_rowmax_refined(const Inputs& in, const Consts& k, const Work& w, const Geometry& g, int prec,
                                   cudaStream_t st);
-// eval = 1: an evaluation pass (no update): log Z of every row, and a column sweep that also
-// accumulates <C, X^t>; the regular iterations leave both out
+// eval = 1: an evaluation pass (no update): the sweeps take stream A (X^t) alone, RF writes log Z
+// of every row and the column sweep also accumulates <C, X^t>
 cudaError_t launch_iteration(const Inputs& in, const Consts& k, const Work& w, const Geometry& g, int prec,
                              int eval, cudaStream_t st);
 void prepare_kernels();
@@ -506,7 +507,7 @@ cudaError_t launch_round(const Inputs& in, const Consts& k, const Work& w, const
 cudaError_t launch_dual(const Inputs& in, const Consts& k, const Work& w, const Geometry& g, int prec, int cur,
                         int which, double* out2, cudaStream_t st);
 // float32 dot-form sweeps (lamp_dot.cu)
-enum DotMode : int { kDotRowSum, kDotColSum, kDotColSumCost, kDotMax, kDotMax2, kDotKmax };
+enum DotMode : int { kDotRowSum, kDotColSum, kDotRowEval, kDotColEval, kDotMax, kDotMax2, kDotKmax };
 int64_t dot_pad(int64_t np);
 cudaError_t dot_transpose(const float* P, int64_t np, int d, float* out, cudaStream_t st);
 void dot_prepare();

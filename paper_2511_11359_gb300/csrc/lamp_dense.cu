@@ -49,6 +49,7 @@ struct __align__(8) Bars {
 // tiles, per-point data, barriers, and slack to align the dynamic buffer to 128 bytes
 constexpr size_t kSmemBytes = (size_t)kStages * kTileBytes + (size_t)kStages * kAuxMax * sizeof(float4) + 128 + 128;
 
+// WC = 1: an evaluation pass (stream A alone; the column sums also weighted by the cost)
 template <bool ROWS, int WC>
 __global__ void __launch_bounds__(kThreads, 2)
 k_dense_tma(const __grid_constant__ CUtensorMap map_c, const Work w, int64_t n, int64_t m, int tiles_per_split,
@@ -146,9 +147,11 @@ k_dense_tma(const __grid_constant__ CUtensorMap map_c, const Work w, int64_t n, 
           for (int a = 0; a < 4; ++a) {
             const uint64_t z2 = pk(tC[a * kTC + c0], tC[a * kTC + c1]);
             const float2 eA = upk(exp2_pair(ahA2, alA2, z2, f2sub(oA2[a], xA2)));
-            const float2 eB = upk(exp2_pair(ahB2, alB2, z2, f2sub(oB2[a], xB2)));
             sA[a] = __fmaf_rn(eA.y, d1.y, __fmaf_rn(eA.x, d0.y, sA[a]));
-            sB[a] = __fmaf_rn(eB.y, d1.w, __fmaf_rn(eB.x, d0.w, sB[a]));
+            if (!WC) {
+              const float2 eB = upk(exp2_pair(ahB2, alB2, z2, f2sub(oB2[a], xB2)));
+              sB[a] = __fmaf_rn(eB.y, d1.w, __fmaf_rn(eB.x, d0.w, sB[a]));
+            }
           }
         }
 #pragma unroll
@@ -165,8 +168,9 @@ k_dense_tma(const __grid_constant__ CUtensorMap map_c, const Work w, int64_t n, 
       if (__all_sync(0xffffffffu, ok && !*(volatile int*)&B->err)) {
         warp_sums_ff<8>(hi, lo, lane);  // value lane / 4: row (lane / 8), stream (lane / 4) % 2
         const int64_t gi = g0 + (lane >> 3);
-        if ((lane & 3) == 0 && gi < n)
-          w.rowpart[((int64_t)blockIdx.y * 2 + ((lane >> 2) & 1)) * n + gi] = (double)hi[0] + (double)lo[0];
+        const int q = (lane >> 2) & 1;
+        if ((lane & 3) == 0 && gi < n && q < 2 - WC)
+          w.rowpart[((int64_t)blockIdx.y * (2 - WC) + q) * n + gi] = (double)hi[0] + (double)lo[0];
       }
     } else {
       // ---------------- G2: column 32 warp + lane of this column block ----------------
@@ -192,25 +196,25 @@ k_dense_tma(const __grid_constant__ CUtensorMap map_c, const Work w, int64_t n, 
           const ulonglong2 rA = tR[a], rB = tR[a + 1];
           const uint64_t z2 = pk(tC[a * kTC], tC[(a + 1) * kTC]);
           const float2 pA = upk(f2mul(exp2_pair(ahA2, alA2, z2, f2add(oA2, rA.x)), rA.y));
-          const float2 eB = upk(exp2_pair(ahB2, alB2, z2, f2add(oB2, rB.x))), wB = upk(rB.y);
           sA = __fadd_rn(__fadd_rn(sA, pA.x), pA.y);
           if (WC) {
             const float2 zf = upk(z2);
             sCx = __fmaf_rn(zf.y, pA.y, __fmaf_rn(zf.x, pA.x, sCx));
           }
-          sB = __fmaf_rn(eB.y, wB.y, __fmaf_rn(eB.x, wB.x, sB));
+          if (!WC) {
+            const float2 eB = upk(exp2_pair(ahB2, alB2, z2, f2add(oB2, rB.x))), wB = upk(rB.y);
+            sB = __fmaf_rn(eB.y, wB.y, __fmaf_rn(eB.x, wB.x, sB));
+          }
         }
         ff_add(hA, lA, sA);
-        ff_add(hB, lB, sB);
         if (WC) ff_add(hC, lC, sCx);
+        else ff_add(hB, lB, sB);
         async::fence_proxy_async_smem();
         async::mbar_arrive(&B->empty[s]);
       }
       if (ok && !*(volatile int*)&B->err && gj < m) {
-        constexpr int na = WC ? 3 : 2;  // the layout k_col_fin reads for this pass
-        w.colpart[((int64_t)blockIdx.y * na + 0) * m + gj] = (double)hA + (double)lA;
-        w.colpart[((int64_t)blockIdx.y * na + 1) * m + gj] = (double)hB + (double)lB;
-        if (WC) w.colpart[((int64_t)blockIdx.y * na + 2) * m + gj] = (double)hC + (double)lC;
+        w.colpart[((int64_t)blockIdx.y * 2 + 0) * m + gj] = (double)hA + (double)lA;
+        w.colpart[((int64_t)blockIdx.y * 2 + 1) * m + gj] = WC ? (double)hC + (double)lC : (double)hB + (double)lB;
       }
     }
   }
@@ -246,7 +250,8 @@ cudaError_t dense_make_map(void* map_out, const float* C, int64_t n, int64_t m, 
 
 cudaError_t dense_prepare() {
   cudaError_t e = cudaSuccess;
-  for (const void* f : {(const void*)dense::k_dense_tma<true, 0>, (const void*)dense::k_dense_tma<false, 0>,
+  for (const void* f : {(const void*)dense::k_dense_tma<true, 0>, (const void*)dense::k_dense_tma<true, 1>,
+                        (const void*)dense::k_dense_tma<false, 0>,
                         (const void*)dense::k_dense_tma<false, 1>}) {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dense::kSmemBytes);
     if (e == cudaSuccess)
@@ -271,7 +276,7 @@ cudaError_t dense_launch_sweep(bool rows, int eval, const Geometry& g, const Wor
   const int tps = (int)((ntiles + splits - 1) / splits);
   dim3 grid((unsigned)nblk, (unsigned)splits);
   const CUtensorMap& map = *reinterpret_cast<const CUtensorMap*>(g.map_c);
-  const auto kern = rows ? dense::k_dense_tma<true, 0> : eval ? dense::k_dense_tma<false, 1> : dense::k_dense_tma<false, 0>;
+  const auto kern = rows ? (eval ? dense::k_dense_tma<true, 1> : dense::k_dense_tma<true, 0>) : eval ? dense::k_dense_tma<false, 1> : dense::k_dense_tma<false, 0>;
   return launch_kernel(kern, grid, dense::kThreads, dense::kSmemBytes, st, map, w, k.n, k.m, tps, k);
 }
 

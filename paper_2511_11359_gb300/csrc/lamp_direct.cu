@@ -34,15 +34,15 @@ inline int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
 // (y - x)^2 == (x - y)^2 in IEEE arithmetic, so the row and the column sweep see
 // bit-identical exponents.  The inner data are the packed-pair arrays (see Work).
 
-// MODE = M_ROWSUM, or M_COLSUM with WC = 1 (evaluation pass: cost-weighted column sums too) or 0;
+// MODE = M_ROWSUM or M_COLSUM; EV = 1: an evaluation pass (stream A alone, see direct_pair), else 0;
 // CK = the ground cost (Consts::cost_op): 0 |x - y|^2, 1 l1, 2 l-inf
-template <int MODE, int D, int WC, int CK>
+template <int MODE, int D, int EV, int CK>
 __global__ void __launch_bounds__(kThreads, 2)
 k_pts_direct(const float* __restrict__ P_out, const float* __restrict__ P_in, int64_t n_out, int64_t n_in,
              const Work w, double* __restrict__ part, int tiles_per_split, const Consts k) {
   using C = DirectCfg<D>;
   constexpr int R = C::R, DP = C::DP, REC = C::REC;
-  constexpr int NACC = WC ? 3 : 2;
+  constexpr int NACC = kDirectSums<MODE, EV>;
   const DevState* __restrict__ dev = w.dev;
   if (dev->done) return;
   const int cur = dev->cur;
@@ -119,7 +119,7 @@ k_pts_direct(const float* __restrict__ P_out, const float* __restrict__ P_in, in
         t.load(rec + p * REC);
 #pragma unroll
         for (int r = 0; r < R; ++r)
-          direct_pair<MODE, D, WC, CK>(x2[r], ownA[r], ownD[r], t, ahA2, alA2, da2, acc[r]);
+          direct_pair<MODE, D, EV, CK>(x2[r], ownA[r], ownD[r], t, ahA2, alA2, da2, acc[r]);
       }
 #pragma unroll
       for (int r = 0; r < R; ++r)
@@ -143,38 +143,38 @@ k_pts_direct(const float* __restrict__ P_out, const float* __restrict__ P_in, in
   }
 }
 
-template <int MODE, int D, int WC, int CK>
+template <int MODE, int D, int EV, int CK>
 static cudaError_t launch_direct_d(const float* Pout, const float* Pin, int64_t nout, int64_t nin, const Work& w,
                                    double* part, int splits, const Consts& k, cudaStream_t st) {
   int64_t tin = cdiv(nin, kDTile);
   int tps = (int)cdiv(tin, splits);
   dim3 grid((unsigned)cdiv(nout, kThreads * DirectCfg<D>::R), (unsigned)splits);
-  return launch_kernel(k_pts_direct<MODE, D, WC, CK>, grid, kThreads, 0, st, Pout, Pin, nout, nin, w, part, tps, k);
+  return launch_kernel(k_pts_direct<MODE, D, EV, CK>, grid, kThreads, 0, st, Pout, Pin, nout, nin, w, part, tps, k);
 }
 
-template <int MODE, int WC, int CK>
+template <int MODE, int EV, int CK>
 static cudaError_t launch_direct_ck(const float* Pout, const float* Pin, int64_t nout, int64_t nin, const Work& w,
                                     double* part, int splits, const Consts& k, cudaStream_t st) {
   switch (k.d) {
-    case 1: return launch_direct_d<MODE, 1, WC, CK>(Pout, Pin, nout, nin, w, part, splits, k, st);
-    case 2: return launch_direct_d<MODE, 2, WC, CK>(Pout, Pin, nout, nin, w, part, splits, k, st);
-    case 3: return launch_direct_d<MODE, 3, WC, CK>(Pout, Pin, nout, nin, w, part, splits, k, st);
-    case 4: return launch_direct_d<MODE, 4, WC, CK>(Pout, Pin, nout, nin, w, part, splits, k, st);
-    case 5: return launch_direct_d<MODE, 5, WC, CK>(Pout, Pin, nout, nin, w, part, splits, k, st);
-    case 6: return launch_direct_d<MODE, 6, WC, CK>(Pout, Pin, nout, nin, w, part, splits, k, st);
-    case 7: return launch_direct_d<MODE, 7, WC, CK>(Pout, Pin, nout, nin, w, part, splits, k, st);
-    case 8: return launch_direct_d<MODE, 8, WC, CK>(Pout, Pin, nout, nin, w, part, splits, k, st);
+    case 1: return launch_direct_d<MODE, 1, EV, CK>(Pout, Pin, nout, nin, w, part, splits, k, st);
+    case 2: return launch_direct_d<MODE, 2, EV, CK>(Pout, Pin, nout, nin, w, part, splits, k, st);
+    case 3: return launch_direct_d<MODE, 3, EV, CK>(Pout, Pin, nout, nin, w, part, splits, k, st);
+    case 4: return launch_direct_d<MODE, 4, EV, CK>(Pout, Pin, nout, nin, w, part, splits, k, st);
+    case 5: return launch_direct_d<MODE, 5, EV, CK>(Pout, Pin, nout, nin, w, part, splits, k, st);
+    case 6: return launch_direct_d<MODE, 6, EV, CK>(Pout, Pin, nout, nin, w, part, splits, k, st);
+    case 7: return launch_direct_d<MODE, 7, EV, CK>(Pout, Pin, nout, nin, w, part, splits, k, st);
+    case 8: return launch_direct_d<MODE, 8, EV, CK>(Pout, Pin, nout, nin, w, part, splits, k, st);
     default: return cudaErrorNotSupported;
   }
 }
 
-template <int MODE, int WC>
+template <int MODE, int EV>
 static cudaError_t launch_direct(const float* Pout, const float* Pin, int64_t nout, int64_t nin, const Work& w,
                                  double* part, int splits, const Consts& k, cudaStream_t st) {
   switch (k.cost_op) {
-    case 0: return launch_direct_ck<MODE, WC, 0>(Pout, Pin, nout, nin, w, part, splits, k, st);
-    case 1: return launch_direct_ck<MODE, WC, 1>(Pout, Pin, nout, nin, w, part, splits, k, st);
-    case 2: return launch_direct_ck<MODE, WC, 2>(Pout, Pin, nout, nin, w, part, splits, k, st);
+    case 0: return launch_direct_ck<MODE, EV, 0>(Pout, Pin, nout, nin, w, part, splits, k, st);
+    case 1: return launch_direct_ck<MODE, EV, 1>(Pout, Pin, nout, nin, w, part, splits, k, st);
+    case 2: return launch_direct_ck<MODE, EV, 2>(Pout, Pin, nout, nin, w, part, splits, k, st);
     default: return cudaErrorNotSupported;
   }
 }
@@ -185,16 +185,16 @@ static cudaError_t launch_direct(const float* Pout, const float* Pin, int64_t no
 int direct_outer(int d) { return kThreads * (d <= 4 ? DirectCfg<4>::R : DirectCfg<8>::R); }
 
 int direct_blocks_per_sm() {
-  // every instantiation is declared with __launch_bounds__(kThreads, 2) and static shared memory
-  int nb = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_pts_direct<M_COLSUM, 8, 1, 0>, kThreads, 0);
-  return nb > 0 ? nb : 1;
+  // two CTAs per SM (__launch_bounds__ of every instantiation); a constant, because the splits that
+  // follow from it decide how the float32 partial sums are grouped
+  return 2;
 }
 
 cudaError_t launch_direct_sweep(bool rows, int eval, const Inputs& in, const Consts& k, const Work& w,
                                 const Geometry& g, cudaStream_t st) {
   if (direct_small_serves(rows ? k.n : k.m, rows ? k.m : k.n, k.d, rows ? g.rows_split : g.cols_split, g.sms))
     return launch_direct_small(rows, eval, in, k, w, g, st);
+  if (rows && eval) return launch_direct<M_ROWSUM, 1>(in.x, in.y, k.n, k.m, w, w.rowpart, g.rows_split, k, st);
   if (rows) return launch_direct<M_ROWSUM, 0>(in.x, in.y, k.n, k.m, w, w.rowpart, g.rows_split, k, st);
   if (eval) return launch_direct<M_COLSUM, 1>(in.y, in.x, k.m, k.n, w, w.colpart, g.cols_split, k, st);
   return launch_direct<M_COLSUM, 0>(in.y, in.x, k.m, k.n, w, w.colpart, g.cols_split, k, st);

@@ -87,11 +87,15 @@ struct DirectPair {
   }
 };
 
-// the two entries (outer point, pair) added to the packed sums acc = {A, B, cost-weighted A}:
-// MODE = M_ROWSUM, or M_COLSUM with WC = 1 (evaluation pass) or 0; CK = the ground cost
-// (Consts::cost_op): 0 |x - y|^2, 1 l1, 2 l-inf.  own, ownD: -offset of the outer point, and a
-// column's dB = BqA - BcolB
-template <int MODE, int D, int WC, int CK, int NACC>
+// sums per outer point
+template <int MODE, int EV>
+constexpr int kDirectSums = MODE == M_ROWSUM && EV ? 1 : 2;
+
+// the two entries (outer point, pair) added to the packed sums acc: {A, B}, or in an evaluation
+// pass (EV) stream A alone, {A} (rows) or {A, cost-weighted A} (columns).  MODE = M_ROWSUM or
+// M_COLSUM; CK = the ground cost (Consts::cost_op): 0 |x - y|^2, 1 l1, 2 l-inf.  own, ownD:
+// -offset of the outer point, and a column's dB = BqA - BcolB
+template <int MODE, int D, int EV, int CK, int NACC>
 __device__ __forceinline__ void direct_pair(const uint64_t (&x2)[D], uint64_t own, uint64_t ownD,
                                             const DirectPair<D>& t, uint64_t ahA2, uint64_t alA2, uint64_t da2,
                                             uint64_t (&acc)[NACC]) {
@@ -113,20 +117,22 @@ __device__ __forceinline__ void direct_pair(const uint64_t (&x2)[D], uint64_t ow
     }
   }
   const uint64_t vA = f2fma(alA2, z2, f2fma(ahA2, z2, f2add(own, t.oA2)));
-  const uint64_t vB = f2fma(da2, z2, f2add(vA, MODE == M_ROWSUM ? t.dC2 : ownD));
-  const float2 vAf = upk(vA), vBf = upk(vB);
+  const float2 vAf = upk(vA);
   const uint64_t eA = pk(ex2(vAf.x), ex2(vAf.y));
-  const uint64_t eB = pk(ex2(vBf.x), ex2(vBf.y));
-  if constexpr (WC) {
+  if constexpr (EV && MODE == M_COLSUM) {
     const uint64_t pA = f2mul(eA, t.wA2);
     acc[0] = f2add(acc[0], pA);
-    acc[2] = f2fma(z2, pA, acc[2]);
+    acc[1] = f2fma(z2, pA, acc[1]);
   } else {
     acc[0] = f2fma(eA, t.wA2, acc[0]);
   }
-  // row sums of stream B carry no weight (it is inside dB_j); column sums weight by q^B_i
-  if constexpr (MODE == M_ROWSUM) acc[1] = f2add(acc[1], eB);
-  else acc[1] = f2fma(eB, t.wB2, acc[1]);
+  if constexpr (!EV) {
+    const float2 vBf = upk(f2fma(da2, z2, f2add(vA, MODE == M_ROWSUM ? t.dC2 : ownD)));
+    const uint64_t eB = pk(ex2(vBf.x), ex2(vBf.y));
+    // row sums of stream B carry no weight (it is inside dB_j); column sums weight by q^B_i
+    if constexpr (MODE == M_ROWSUM) acc[1] = f2add(acc[1], eB);
+    else acc[1] = f2fma(eB, t.wB2, acc[1]);
+  }
 }
 
 }  // namespace lamp

@@ -22,13 +22,13 @@ constexpr int kMaxTiles = 8;  // tiles of a split: 16 groups
 
 inline int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
-template <int MODE, int D, int WC, int CK, int R>
+template <int MODE, int D, int EV, int CK, int R>
 __global__ void __launch_bounds__(128, R == 1 ? 5 : 4)
 k_direct_small(const float* __restrict__ P_out, const float* __restrict__ P_in, int64_t n_out, int64_t n_in,
                const Work w, double* __restrict__ part, int tiles_per_split, const Consts k) {
   using C = DirectCfg<D>;
   constexpr int REC = C::REC;
-  constexpr int NACC = WC ? 3 : 2;
+  constexpr int NACC = kDirectSums<MODE, EV>;
   constexpr int kPts = 32 * R;
   const DevState* __restrict__ dev = w.dev;
   if (dev->done) return;
@@ -89,7 +89,7 @@ k_direct_small(const float* __restrict__ P_out, const float* __restrict__ P_in, 
       t.load(rp + p * REC);
 #pragma unroll
       for (int r = 0; r < R; ++r)
-        direct_pair<MODE, D, WC, CK>(x2[r], ownA[r], ownD[r], t, ahA2, alA2, da2, acc[r]);
+        direct_pair<MODE, D, EV, CK>(x2[r], ownA[r], ownD[r], t, ahA2, alA2, da2, acc[r]);
     }
 #pragma unroll
     for (int r = 0; r < R; ++r)
@@ -117,44 +117,44 @@ struct Launch {
   bool wide;  // R = 4 (d <= 4) or 2 outer points per lane, else 1
 };
 
-template <int MODE, int D, int WC, int CK, int R>
+template <int MODE, int D, int EV, int CK, int R>
 cudaError_t go(const Launch& l, const Work& w, const Consts& k, cudaStream_t st) {
-  constexpr int NACC = WC ? 3 : 2;
+  constexpr int NACC = kDirectSums<MODE, EV>;
   const int groups = l.tps * (kDPairs / kDFold);
   const unsigned threads = 32u * (unsigned)(groups < 4 ? groups : 4);
   const size_t smem = ((size_t)l.tps * kDPairs * DirectCfg<D>::REC + (size_t)groups * NACC * 32 * R) * sizeof(float);
-  static_assert(((size_t)kMaxTiles * kDPairs * DirectCfg<8>::REC + (size_t)2 * kMaxTiles * 3 * 128) * 4 <= 100 * 1024, "");
+  static_assert(((size_t)kMaxTiles * kDPairs * DirectCfg<8>::REC + (size_t)2 * kMaxTiles * 2 * 128) * 4 <= 100 * 1024, "");
   if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(k_direct_small<MODE, D, WC, CK, R>,
+    cudaError_t e = cudaFuncSetAttribute(k_direct_small<MODE, D, EV, CK, R>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
     if (e != cudaSuccess) return e;
   }
-  return launch_kernel(k_direct_small<MODE, D, WC, CK, R>, dim3((unsigned)cdiv(l.nout, 32 * R), (unsigned)l.splits), threads,
+  return launch_kernel(k_direct_small<MODE, D, EV, CK, R>, dim3((unsigned)cdiv(l.nout, 32 * R), (unsigned)l.splits), threads,
                     smem, st, l.Pout, l.Pin, l.nout, l.nin, w, l.part, l.tps, k);
 }
 
-template <int MODE, int D, int WC>
+template <int MODE, int D, int EV>
 cudaError_t go_cost(const Launch& l, const Work& w, const Consts& k, cudaStream_t st) {
   constexpr int RW = DirectCfg<D>::R;
   switch (k.cost_op) {
-    case 0: return l.wide ? go<MODE, D, WC, 0, RW>(l, w, k, st) : go<MODE, D, WC, 0, 1>(l, w, k, st);
-    case 1: return l.wide ? go<MODE, D, WC, 1, RW>(l, w, k, st) : go<MODE, D, WC, 1, 1>(l, w, k, st);
-    case 2: return l.wide ? go<MODE, D, WC, 2, RW>(l, w, k, st) : go<MODE, D, WC, 2, 1>(l, w, k, st);
+    case 0: return l.wide ? go<MODE, D, EV, 0, RW>(l, w, k, st) : go<MODE, D, EV, 0, 1>(l, w, k, st);
+    case 1: return l.wide ? go<MODE, D, EV, 1, RW>(l, w, k, st) : go<MODE, D, EV, 1, 1>(l, w, k, st);
+    case 2: return l.wide ? go<MODE, D, EV, 2, RW>(l, w, k, st) : go<MODE, D, EV, 2, 1>(l, w, k, st);
     default: return cudaErrorNotSupported;
   }
 }
 
-template <int MODE, int WC>
+template <int MODE, int EV>
 cudaError_t go_dim(const Launch& l, const Work& w, const Consts& k, cudaStream_t st) {
   switch (k.d) {
-    case 1: return go_cost<MODE, 1, WC>(l, w, k, st);
-    case 2: return go_cost<MODE, 2, WC>(l, w, k, st);
-    case 3: return go_cost<MODE, 3, WC>(l, w, k, st);
-    case 4: return go_cost<MODE, 4, WC>(l, w, k, st);
-    case 5: return go_cost<MODE, 5, WC>(l, w, k, st);
-    case 6: return go_cost<MODE, 6, WC>(l, w, k, st);
-    case 7: return go_cost<MODE, 7, WC>(l, w, k, st);
-    case 8: return go_cost<MODE, 8, WC>(l, w, k, st);
+    case 1: return go_cost<MODE, 1, EV>(l, w, k, st);
+    case 2: return go_cost<MODE, 2, EV>(l, w, k, st);
+    case 3: return go_cost<MODE, 3, EV>(l, w, k, st);
+    case 4: return go_cost<MODE, 4, EV>(l, w, k, st);
+    case 5: return go_cost<MODE, 5, EV>(l, w, k, st);
+    case 6: return go_cost<MODE, 6, EV>(l, w, k, st);
+    case 7: return go_cost<MODE, 7, EV>(l, w, k, st);
+    case 8: return go_cost<MODE, 8, EV>(l, w, k, st);
     default: return cudaErrorNotSupported;
   }
 }
@@ -181,6 +181,7 @@ cudaError_t launch_direct_small(bool rows, int eval, const Inputs& in, const Con
   // several outer points per lane share each record load (a 16-byte broadcast load fills the
   // same 512 bytes of registers as any other): the wide form once it gives two CTAs per SM
   l.wide = cdiv(l.nout, 32 * (k.d <= 4 ? 4 : 2)) * l.splits >= 2 * (int64_t)g.sms;
+  if (rows && eval) return go_dim<M_ROWSUM, 1>(l, w, k, st);
   if (rows) return go_dim<M_ROWSUM, 0>(l, w, k, st);
   if (eval) return go_dim<M_COLSUM, 1>(l, w, k, st);
   return go_dim<M_COLSUM, 0>(l, w, k, st);

@@ -28,7 +28,8 @@ constexpr int kIn = 128;      // inner points of a tile: the unit of the splits 
 constexpr int kStage = 256;   // inner points of a stage (two tiles)
 constexpr int kThreads = 256;
 
-enum Mode : int { kRowSum = 0, kColSum = 1, kColSumCost = 2, kMax = 3, kMax2 = 4, kKmax = 5 };
+// kRowEval, kColEval: evaluation passes (stream A alone; columns also weighted by the cost)
+enum Mode : int { kRowSum = 0, kColSum = 1, kRowEval = 2, kColEval = 3, kMax = 4, kMax2 = 5, kKmax = 6 };
 
 __device__ __forceinline__ void cp16(void* dst, const void* src) {
   const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
@@ -90,7 +91,7 @@ __device__ __forceinline__ void load_outer(float* so, float4* soff, const Args& 
   if (MODE != kMax && tid < kOut) {
     int64_t go = t.o * kOut + tid;
     if (go >= a.n_out) go = a.n_out - 1;
-    if (MODE == kColSum || MODE == kColSumCost)
+    if (MODE == kColSum || MODE == kColEval)
       cp16(soff + tid, (cur ? a.off4[1] : a.off4[0]) + go);
     else
       cp8(soff + tid, (cur ? a.off2[1] : a.off2[0]) + go);
@@ -111,8 +112,8 @@ __device__ __forceinline__ void load_stage(float* si, float4* sd, const Args& a,
 
 template <int MODE>
 struct Acc {
-  static constexpr bool kSums = MODE <= kColSumCost;
-  static constexpr int N = MODE == kColSumCost ? 3 : 2;
+  static constexpr bool kSums = MODE <= kColEval;
+  static constexpr int N = MODE == kRowEval ? 1 : 2;
   float hi[8][N], lo[8][N];  // kSums: float-float sums; else hi = the running maxima
   __device__ __forceinline__ void reset() {
 #pragma unroll
@@ -179,7 +180,7 @@ __device__ __forceinline__ void tile_sums(const float* __restrict__ so, const fl
     for (int r = 0; r < 8; ++r) {
       const int ro = (r < 4) ? (ty * 4 + r) : (64 + ty * 4 + r - 4);
       float oA = 0.f, oB = 0.f;
-      if (MODE == kColSum || MODE == kColSumCost) {
+      if (MODE == kColSum || MODE == kColEval) {
         const float4 o = soff[ro];
         oA = o.x;
         oB = o.z;
@@ -190,28 +191,29 @@ __device__ __forceinline__ void tile_sums(const float* __restrict__ so, const fl
       }
       if constexpr (Acc<MODE>::kSums) {
         const uint64_t oA2 = pk(-oA, -oA), oB2 = pk(-oB, -oB);
-        float sA = 0.f, sB = 0.f, sC = 0.f;
+        float sA = 0.f, sB = 0.f;
 #pragma unroll
         for (int p = 0; p < 4; ++p) {
           const uint64_t z = z2[r][4 * u + p];
           const float4 d0 = dat[2 * p], d1 = dat[2 * p + 1];
           const float2 eA = upk(exp2_pair(ahA2, alA2, z, f2sub(oA2, pk(d0.x, d1.x))));
-          const float2 eB = upk(exp2_pair(ahB2, alB2, z, f2sub(oB2, pk(d0.z, d1.z))));
-          if (MODE == kRowSum) {
+          if (MODE == kRowSum || MODE == kRowEval) {
             sA = __fmaf_rn(eA.y, d1.y, __fmaf_rn(eA.x, d0.y, sA));
           } else {
             const float p0 = __fmul_rn(eA.x, d0.y), p1 = __fmul_rn(eA.y, d1.y);
             sA = __fadd_rn(__fadd_rn(sA, p0), p1);
-            if (MODE == kColSumCost) {
+            if (MODE == kColEval) {
               const float2 zf = upk(z);
-              sC = __fmaf_rn(zf.y, p1, __fmaf_rn(zf.x, p0, sC));
+              sB = __fmaf_rn(zf.y, p1, __fmaf_rn(zf.x, p0, sB));
             }
           }
-          sB = __fmaf_rn(eB.y, d1.w, __fmaf_rn(eB.x, d0.w, sB));
+          if (MODE == kRowSum || MODE == kColSum) {
+            const float2 eB = upk(exp2_pair(ahB2, alB2, z, f2sub(oB2, pk(d0.z, d1.z))));
+            sB = __fmaf_rn(eB.y, d1.w, __fmaf_rn(eB.x, d0.w, sB));
+          }
         }
         ff_add(acc.hi[r][0], acc.lo[r][0], sA);
-        ff_add(acc.hi[r][1], acc.lo[r][1], sB);
-        if (MODE == kColSumCost) ff_add(acc.hi[r][Acc<MODE>::N - 1], acc.lo[r][Acc<MODE>::N - 1], sC);
+        if (Acc<MODE>::N > 1) ff_add(acc.hi[r][Acc<MODE>::N - 1], acc.lo[r][Acc<MODE>::N - 1], sB);
       } else {
 #pragma unroll
         for (int p = 0; p < 4; ++p) {
@@ -266,25 +268,16 @@ template <int MODE>
 __device__ __forceinline__ void write_item(const Args& a, const Item& t, Acc<MODE>& acc, int tx, int ty) {
   constexpr int NACC = Acc<MODE>::N;
   if constexpr (Acc<MODE>::kSums) {
+    // value 8 q + r: sum q of outer point r (evaluation row sums have q = 0 alone)
     double v[16];
 #pragma unroll
     for (int r = 0; r < 8; ++r)
 #pragma unroll
-      for (int q = 0; q < 2; ++q) v[2 * r + q] = (double)acc.hi[r][q] + (double)acc.lo[r][q];
-    const double s = halfwarp_sum16(v, tx);  // value index tx: outer point tx >> 1, stream tx & 1
-    const int r = tx >> 1;
+      for (int q = 0; q < 2; ++q) v[8 * q + r] = q < NACC ? (double)acc.hi[r][q % NACC] + (double)acc.lo[r][q % NACC] : 0.0;
+    const double s = halfwarp_sum16(v, tx);
+    const int r = tx & 7, q = tx >> 3;
     const int64_t go = t.o * kOut + ((r < 4) ? (ty * 4 + r) : (64 + ty * 4 + r - 4));
-    if (go < a.n_out) a.part[((int64_t)t.split * NACC + (tx & 1)) * a.n_out + go] = s;
-    if (NACC == 3) {
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        v[q] = (double)acc.hi[q][NACC - 1] + (double)acc.lo[q][NACC - 1];
-        v[8 + q] = 0.0;
-      }
-      const double c = halfwarp_sum16(v, tx);
-      const int64_t gc = t.o * kOut + ((tx < 4) ? (ty * 4 + tx) : (64 + ty * 4 + tx - 4));
-      if (tx < 8 && gc < a.n_out) a.part[((int64_t)t.split * NACC + 2) * a.n_out + gc] = c;
-    }
+    if (go < a.n_out && q < NACC) a.part[((int64_t)t.split * NACC + q) * a.n_out + go] = s;
   } else {
 #pragma unroll
     for (int r = 0; r < 8; ++r) {
@@ -652,7 +645,8 @@ void set_smem() {
 void dot_prepare() {
   set_smem<dot::kRowSum>();
   set_smem<dot::kColSum>();
-  set_smem<dot::kColSumCost>();
+  set_smem<dot::kRowEval>();
+  set_smem<dot::kColEval>();
   set_smem<dot::kMax>();
   set_smem<dot::kMax2>();
   set_smem<dot::kKmax>();
@@ -715,7 +709,7 @@ cudaError_t dot_grad(bool rows, const Inputs& in, const Work& w, const Consts& k
 }
 
 cudaError_t dot_launch(int mode, const Work& w, const Consts& k, const Geometry& g, cudaStream_t st) {
-  const bool cols = mode == kDotColSum || mode == kDotColSumCost;
+  const bool cols = mode == kDotColSum || mode == kDotColEval;
   dot::Args a{};
   a.out_t = cols ? w.yt : w.xt;
   a.in_t = cols ? w.xt : w.yt;
@@ -738,7 +732,8 @@ cudaError_t dot_launch(int mode, const Work& w, const Consts& k, const Geometry&
   switch (mode) {
     case kDotRowSum: return launch_mode<dot::kRowSum>(a, w, k, g.sms, st);
     case kDotColSum: return launch_mode<dot::kColSum>(a, w, k, g.sms, st);
-    case kDotColSumCost: return launch_mode<dot::kColSumCost>(a, w, k, g.sms, st);
+    case kDotRowEval: return launch_mode<dot::kRowEval>(a, w, k, g.sms, st);
+    case kDotColEval: return launch_mode<dot::kColEval>(a, w, k, g.sms, st);
     case kDotMax: return launch_mode<dot::kMax>(a, w, k, g.sms, st);
     case kDotMax2: return launch_mode<dot::kMax2>(a, w, k, g.sms, st);
     default: return launch_mode<dot::kKmax>(a, w, k, g.sms, st);

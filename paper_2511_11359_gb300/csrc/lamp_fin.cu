@@ -159,10 +159,10 @@ __device__ __forceinline__ void store_pair_field(float4* __restrict__ a, int64_t
   reinterpret_cast<float*>(a + (e >> 1) * 2)[2 * field + (int)(e & 1)] = v;
 }
 
-// RF: row finalize of iteration t.  The warps of stream A give q^A (and, in evaluation passes,
-// log Z); those of stream B q^B and the row shifts of iteration t + 1, where stream A has
+// RF: row finalize of iteration t.  The warps of stream A give q^A; those of stream B q^B and the row shifts of iteration t + 1, where stream A has
 // kappa_{t+1} (stream B here) and stream B is extrapolated linearly in t.  Block `rowblocks`
-// prepares make_sweep_params of kappa_{t+2} for CF.
+// prepares make_sweep_params of kappa_{t+2} for CF.  Evaluation passes have stream A alone, and
+// the second warps form log Z.
 template <bool EVAL>
 __global__ void __launch_bounds__(kThreads)
 k_row_fin(const Work w, int splits, const double* __restrict__ r, int rowblocks, const Consts k) {
@@ -194,9 +194,11 @@ k_row_fin(const Work w, int splits, const double* __restrict__ r, int rowblocks,
     ri = r[i];
     if (k.zdot && (EVAL || !k.shared_shift)) snx = k.s * w.nx[i];
     // the partials' loads are independent and in flight together; the sums keep the split order
-    const double* __restrict__ part = w.rowpart + (int64_t)role * k.n + i;
+    // (evaluation passes sweep stream A alone: one sum per split, read by both warps)
+    constexpr int na = EVAL ? 1 : 2;
+    const double* __restrict__ part = w.rowpart + (int64_t)(EVAL ? 0 : role) * k.n + i;
 #pragma unroll 8
-    for (int s = 0; s < splits; ++s) S += part[(int64_t)s * 2 * k.n];
+    for (int s = 0; s < splits; ++s) S += part[(int64_t)s * na * k.n];
     if (!in_range(S)) {
       atomicExch(&dev->status, 5 /* LAMP_E_NUMERIC */);
       S = 1.0;
@@ -216,14 +218,13 @@ k_row_fin(const Work w, int splits, const double* __restrict__ r, int rowblocks,
         store_pair_field(w.g2row2, i, 0, -rq.x);
         store_pair_field(w.g2row2, i, 1, q);
       }
-      if (EVAL) {
-        ls = log2(S);
-        const double lz = kLn2 * ((double)rq.x - sp.lamA * snx + ls);  // log Z of X^t
-        w.logZ[i] = lz;
-        contrib = ri * lz;
-      } else if (!k.shared_shift) {
+      if (!EVAL && !k.shared_shift) {
         sx[p] = (double)rq.x - sp.lamA * snx + log2_table(S, stab);
       }
+    } else if (EVAL) {
+      const double lz = kLn2 * ((double)rq.x - sp.lamA * snx + log2(S));  // log Z of X^t
+      w.logZ[i] = lz;
+      contrib = ri * lz;
     } else {
       const float q = (float)div_seeded(ri, S);
       reinterpret_cast<float2*>(w.g2row + i)[1] = make_float2(rq.y, q);
@@ -231,13 +232,13 @@ k_row_fin(const Work w, int splits, const double* __restrict__ r, int rowblocks,
         store_pair_field(w.g2row2, i, 2, k.shared_shift ? 0.f : -rq.y);
         store_pair_field(w.g2row2, i, 3, q);
       }
-      if (!EVAL) ls = log2_table(S, stab);
+      ls = log2_table(S, stab);
     }
   }
   if (EVAL) {
-    if (role == 0) {
+    if (role == 1) {
       contrib = warp_sum_d(contrib);
-      if ((threadIdx.x & 31) == 0) sred[threadIdx.x >> 5] = contrib;
+      if ((threadIdx.x & 31) == 0) sred[p >> 5] = contrib;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -283,8 +284,9 @@ k_col_fin(const Work w, int splits, const double* __restrict__ cvec, int rowbloc
   SweepParams sp, spn;
   iteration_params_of(dev, k, sp, spn);
   if (valid) {
-    // partials of split s: [s][3][m] with the cost-weighted sums (evaluation passes), else [s][2][m]
-    constexpr int na = EVAL ? 3 : 2;
+    // partials of split s: [s][2][m], the streams' sums; evaluation passes: stream A's sums and
+    // the cost-weighted ones, which the second warps take
+    constexpr int na = 2;
     const float4 cq = w.colq[cur][j];
     const double cj = cvec[j];
     const double nuj = w.nu[cur][j], thj = EVAL ? 0.0 : w.theta[cur][j];
@@ -293,8 +295,6 @@ k_col_fin(const Work w, int splits, const double* __restrict__ cvec, int rowbloc
     if (k.zdot) sny = k.s * w.ny[j];
     double a = 0.0;
     // the partials' loads are independent and in flight together; the sums keep the split order
-    // evaluation passes: the second warps take the cost-weighted sums instead of stream B's
-    if (EVAL && role) part += k.m;
 #pragma unroll 8
     for (int s = 0; s < splits; ++s) a += part[(int64_t)s * na * k.m];
     if (EVAL && role) zsum = (double)cq.y * a;

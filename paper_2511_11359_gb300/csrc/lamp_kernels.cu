@@ -83,7 +83,8 @@ struct SweepIO {
   const float4* indat[2];
 };
 
-// M_COLSUM: DG = 1 also accumulates the cost-weighted sums (evaluation passes).
+// M_ROWSUM, M_COLSUM: DG = 1 is an evaluation pass (stream A alone, column sums also weighted by
+// the cost).
 // M_GRAD accumulates sum_b 2^{v_ab} weight_b V_b[0:DG], V = Vin (n_in x DG, row-major): the
 // transport map of costs that the packed kernels do not serve (l1, l-inf with d > 8)
 template <int MODE, int DG>
@@ -145,8 +146,9 @@ k_pts_sweep(const float* __restrict__ P_out, const float* __restrict__ P_in, int
 
   const float ahA = sp.ahA, alA = sp.alA, ahB = sp.ahB, alB = sp.alB;
 
-  constexpr bool WC = MODE == M_COLSUM && DG > 0;
-  constexpr int NACC = WC ? 3 : 2;
+  constexpr bool EV = MODE <= M_COLSUM && DG > 0;  // evaluation pass: stream A alone
+  constexpr bool WC = MODE == M_COLSUM && EV;      // ... and the cost-weighted sums
+  constexpr int NACC = EV && !WC ? 1 : 2;
   float hi[8][NACC], lo[8][NACC];
   float mx[8][2];
   double gacc[8][DG > 0 ? DG : 1];
@@ -229,26 +231,25 @@ k_pts_sweep(const float* __restrict__ P_out, const float* __restrict__ P_in, int
     if (MODE == M_ROWSUM || MODE == M_COLSUM) {
 #pragma unroll
       for (int a = 0; a < 8; ++a) {
-        float sA = 0.f, sB = 0.f, sC = 0.f;
+        float sA = 0.f, sB = 0.f;
 #pragma unroll
         for (int b = 0; b < 8; ++b) {
           const float zz = z[a][b];
-          const float vA = __fmaf_rn(alA, zz, __fmaf_rn(ahA, zz, -(oA[a] + dat[b].x)));
-          const float vB = __fmaf_rn(alB, zz, __fmaf_rn(ahB, zz, -(oB[a] + dat[b].z)));
-          const float eA = ex2(vA);
-          const float eB = ex2(vB);
+          const float eA = ex2(__fmaf_rn(alA, zz, __fmaf_rn(ahA, zz, -(oA[a] + dat[b].x))));
           if (MODE == M_ROWSUM) {
             sA = __fmaf_rn(eA, dat[b].y, sA);
           } else {
             const float pA = __fmul_rn(eA, dat[b].y);
             sA = __fadd_rn(sA, pA);
-            if (WC) sC = __fmaf_rn(zz, pA, sC);
+            if (WC) sB = __fmaf_rn(zz, pA, sB);
           }
-          sB = __fmaf_rn(eB, dat[b].w, sB);
+          if (!EV) {
+            const float eB = ex2(__fmaf_rn(alB, zz, __fmaf_rn(ahB, zz, -(oB[a] + dat[b].z))));
+            sB = __fmaf_rn(eB, dat[b].w, sB);
+          }
         }
         ff_add(hi[a][0], lo[a][0], sA);
-        ff_add(hi[a][1], lo[a][1], sB);
-        if (WC) ff_add(hi[a][NACC - 1], lo[a][NACC - 1], sC);
+        if (NACC > 1) ff_add(hi[a][NACC - 1], lo[a][NACC - 1], sB);
       }
     } else if (MODE == M_MAX) {
 #pragma unroll
@@ -357,7 +358,8 @@ constexpr int kDR = 4;          // rows per CTA in the row sweep
 constexpr int kDSplitRows = 8;  // rows per tile in the choice of its splits
 constexpr int kDChunk = 1024;   // columns per CTA step (4 per thread, stride 256)
 
-template <int MODE>  // M_ROWSUM, M_MAX or M_MAX2
+// MODE = M_ROWSUM, M_MAX or M_MAX2; EV = 1: row sums of an evaluation pass (stream A alone)
+template <int MODE, int EV = 0>
 __global__ void __launch_bounds__(kThreads, 3)
 k_dense_rows(const float* __restrict__ C, int64_t ldc, int64_t n, int64_t m, const Work w,
              int chunks_per_split, const Consts k) {
@@ -429,9 +431,11 @@ k_dense_rows(const float* __restrict__ C, int64_t ldc, int64_t n, int64_t m, con
         const uint64_t z2 = pk(cv[a][2 * p], cv[a][2 * p + 1]);
         if (MODE == M_ROWSUM) {
           const float2 eA = upk(exp2_pair(ahA2, alA2, z2, f2sub(pk(oA[a], oA[a]), pk(d0.x, d1.x))));
-          const float2 eB = upk(exp2_pair(ahB2, alB2, z2, f2sub(pk(oB[a], oB[a]), pk(d0.z, d1.z))));
           sA = __fmaf_rn(eA.y, d1.y, __fmaf_rn(eA.x, d0.y, sA));
-          sB = __fmaf_rn(eB.y, d1.w, __fmaf_rn(eB.x, d0.w, sB));
+          if (!EV) {
+            const float2 eB = upk(exp2_pair(ahB2, alB2, z2, f2sub(pk(oB[a], oB[a]), pk(d0.z, d1.z))));
+            sB = __fmaf_rn(eB.y, d1.w, __fmaf_rn(eB.x, d0.w, sB));
+          }
         } else if (MODE == M_MAX2) {
           // refinement pass of the eta = 0 dual bound (see k_pts_sweep, M_MAX2)
           const float2 u = upk(f2sub(f2fma(alA2, z2, f2fma(ahA2, z2, f2sub(pk(oA[a], oA[a]), pk(d0.x, d1.x)))),
@@ -459,7 +463,7 @@ k_dense_rows(const float* __restrict__ C, int64_t ldc, int64_t n, int64_t m, con
       double v = 0.0;
       for (int u = 0; u < kThreads / 32; ++u) v += sred[u][tid];
       const int a = tid >> 1, s = tid & 1;
-      if (r0 + a < n) w.rowpart[((int64_t)split * 2 + s) * n + r0 + a] = v;
+      if (r0 + a < n && s < 2 - EV) w.rowpart[((int64_t)split * (2 - EV) + s) * n + r0 + a] = v;
     }
   } else {
     __shared__ float fred[kThreads / 32][NV];
@@ -482,7 +486,7 @@ constexpr int kDColRows = 16;      // rows per group: the unit of the column sum
 constexpr int kDColThreads = 128;  // two columns per thread
 constexpr int kDCols = 2 * kDColThreads;
 
-template <int WC>  // 1: an evaluation pass, with the cost-weighted sums
+template <int WC>  // 1: an evaluation pass: stream A's sums and the cost-weighted ones
 __global__ void __launch_bounds__(kDColThreads, 6)
 k_dense_cols(const float* __restrict__ C, int64_t ldc, int64_t n, int64_t m, const Work w, int64_t rows_per_split,
              const Consts k) {
@@ -535,30 +539,30 @@ k_dense_cols(const float* __restrict__ C, int64_t ldc, int64_t n, int64_t m, con
       const float4 rd = __ldg(g2row + ib + a);
       const uint64_t z2 = pk(cv[a][0], cv[a][1]);
       const float2 eA = upk(exp2_pair(ahA2, alA2, z2, f2sub(oA2, pk(rd.x, rd.x))));
-      const float2 eB = upk(exp2_pair(ahB2, alB2, z2, f2sub(oB2, pk(rd.z, rd.z))));
       const float pA[2] = {__fmul_rn(eA.x, rd.y), __fmul_rn(eA.y, rd.y)};
 #pragma unroll
       for (int q = 0; q < 2; ++q) {
         sA[q] = __fadd_rn(sA[q], pA[q]);
         if (WC) sC[q] = __fmaf_rn(cv[a][q], pA[q], sC[q]);
       }
-      sB[0] = __fmaf_rn(eB.x, rd.w, sB[0]);
-      sB[1] = __fmaf_rn(eB.y, rd.w, sB[1]);
+      if (!WC) {
+        const float2 eB = upk(exp2_pair(ahB2, alB2, z2, f2sub(oB2, pk(rd.z, rd.z))));
+        sB[0] = __fmaf_rn(eB.x, rd.w, sB[0]);
+        sB[1] = __fmaf_rn(eB.y, rd.w, sB[1]);
+      }
     }
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
       ff_add(hiA[q], loA[q], sA[q]);
-      ff_add(hiB[q], loB[q], sB[q]);
       if (WC) ff_add(hiC[q], loC[q], sC[q]);
+      else ff_add(hiB[q], loB[q], sB[q]);
     }
   }
 #pragma unroll
   for (int q = 0; q < 2; ++q) {
     if (!ok[q]) continue;
-    constexpr int na = WC ? 3 : 2;  // the layout k_col_fin reads for this pass
-    part[((int64_t)split * na + 0) * m + jj[q]] = (double)hiA[q] + (double)loA[q];
-    part[((int64_t)split * na + 1) * m + jj[q]] = (double)hiB[q] + (double)loB[q];
-    if (WC) part[((int64_t)split * na + 2) * m + jj[q]] = (double)hiC[q] + (double)loC[q];
+    part[((int64_t)split * 2 + 0) * m + jj[q]] = (double)hiA[q] + (double)loA[q];
+    part[((int64_t)split * 2 + 1) * m + jj[q]] = WC ? (double)hiC[q] + (double)loC[q] : (double)hiB[q] + (double)loB[q];
   }
 }
 
@@ -824,24 +828,27 @@ cudaError_t launch_init_state(const Inputs& in, const Consts& k, const Work& w, 
 }
 
 static cudaError_t launch_row_sweep(const Inputs& in, const Consts& k, const Work& w, const Geometry& g, int mode,
-                                    cudaStream_t st) {
-  if (k.kind == COST_DENSE && g.map_c && mode == M_ROWSUM) return dense_launch_sweep(true, 0, g, w, k, g.rows_split, st);
+                                    int eval, cudaStream_t st) {
+  if (k.kind == COST_DENSE && g.map_c && mode == M_ROWSUM) return dense_launch_sweep(true, eval, g, w, k, g.rows_split, st);
   if (k.kind == COST_DENSE) {
     int64_t nch = cdiv(k.m, kDChunk);
     int cps = (int)cdiv(nch, g.rows_split);
     dim3 grid((unsigned)cdiv(k.n, kDR), (unsigned)g.rows_split);
-    const auto kern = mode == M_ROWSUM ? k_dense_rows<M_ROWSUM> : mode == M_MAX2 ? k_dense_rows<M_MAX2> : k_dense_rows<M_MAX>;
+    const auto kern = mode == M_ROWSUM ? (eval ? k_dense_rows<M_ROWSUM, 1> : k_dense_rows<M_ROWSUM>) : mode == M_MAX2 ? k_dense_rows<M_MAX2> : k_dense_rows<M_MAX>;
     return launch_kernel(kern, grid, kThreads, 0, st, in.C, in.ldc, k.n, k.m, w, cps, k);
   }
-  if (mode == M_ROWSUM && k.shared_shift) return launch_direct_sweep(true, 0, in, k, w, g, st);
+  if (mode == M_ROWSUM && k.shared_shift) return launch_direct_sweep(true, eval, in, k, w, g, st);
   if (k.shared_shift) return direct_max(mode == M_MAX2 ? kDirectMax2 : kDirectMax, in, w, k, g.rows_split, st);
-  if (k.zdot) return dot_launch(mode == M_ROWSUM ? kDotRowSum : mode == M_MAX2 ? kDotMax2 : kDotMax, w, k, g, st);
+  if (k.zdot)
+    return dot_launch(mode == M_ROWSUM ? (eval ? kDotRowEval : kDotRowSum) : mode == M_MAX2 ? kDotMax2 : kDotMax, w, k, g, st);
   SweepIO io;
   for (int b = 0; b < 2; ++b) {
     io.off2[b] = w.rowshift[b];
     io.off4[b] = nullptr;
     io.indat[b] = w.colq[b];
   }
+  if (mode == M_ROWSUM && eval)
+    return launch_pts<M_ROWSUM, 1>(in.x, in.y, k.n, k.m, k.d, io, w.rowpart, nullptr, g.rows_split, w.dev, k, st);
   if (mode == M_ROWSUM)
     return launch_pts<M_ROWSUM, 0>(in.x, in.y, k.n, k.m, k.d, io, w.rowpart, nullptr, g.rows_split, w.dev, k, st);
   if (mode == M_MAX2)
@@ -859,7 +866,7 @@ static cudaError_t launch_col_sweep(const Inputs& in, const Consts& k, const Wor
     return launch_kernel(eval ? k_dense_cols<1> : k_dense_cols<0>, grid, kDColThreads, 0, st, in.C, in.ldc, k.n, k.m, w, rps, k);
   }
   if (k.shared_shift) return launch_direct_sweep(false, eval, in, k, w, g, st);
-  if (k.zdot) return dot_launch(eval ? kDotColSumCost : kDotColSum, w, k, g, st);
+  if (k.zdot) return dot_launch(eval ? kDotColEval : kDotColSum, w, k, g, st);
   SweepIO io;
   for (int b = 0; b < 2; ++b) {
     io.off2[b] = nullptr;
@@ -876,7 +883,7 @@ cudaError_t launch_prime(const Inputs& in, const Consts& k, const Work& w, const
   // the tensor-core context takes its row maxima from the tensor-core sweep (the cost its
   // iteration uses)
   cudaError_t e = prec == 1 /* LAMP_PREC_BF16_TC */ && g.map_x ? tc_launch_rowmax(1, g, w, k, g.rows_split, st)
-                                                                : launch_row_sweep(in, k, w, g, M_MAX, st);
+                                                                : launch_row_sweep(in, k, w, g, M_MAX, 0, st);
   if (e != cudaSuccess) return e;
   k_prime_fin<<<(unsigned)cdiv(k.n, 256), 256, 0, st>>>(w, g.rows_split, k);
   return cudaGetLastError();
@@ -885,7 +892,7 @@ cudaError_t launch_prime(const Inputs& in, const Consts& k, const Work& w, const
 cudaError_t launch_rowmax_refined(const Inputs& in, const Consts& k, const Work& w, const Geometry& g, int prec,
                                   cudaStream_t st) {
   if (prec == 1 /* LAMP_PREC_BF16_TC */ && g.map_x) return tc_launch_rowmax(2, g, w, k, g.rows_split, st);
-  return launch_row_sweep(in, k, w, g, M_MAX2, st);
+  return launch_row_sweep(in, k, w, g, M_MAX2, 0, st);
 }
 
 cudaError_t launch_iteration_part(const Inputs& in, const Consts& k, const Work& w, const Geometry& g, int prec,
@@ -893,8 +900,8 @@ cudaError_t launch_iteration_part(const Inputs& in, const Consts& k, const Work&
   const bool tcpath = prec == 1 /* LAMP_PREC_BF16_TC */;
   switch (part) {
     case 0:
-      if (tcpath) return tc_launch_sweep(true, 0, g, w, k, g.rows_split, st);
-      return launch_row_sweep(in, k, w, g, M_ROWSUM, st);
+      if (tcpath) return tc_launch_sweep(true, eval, g, w, k, g.rows_split, st);
+      return launch_row_sweep(in, k, w, g, M_ROWSUM, eval, st);
     case 1:
       return launch_row_fin(in, k, w, g, eval, st);
     case 2:
@@ -927,6 +934,7 @@ void prepare_kernels() {
   static bool done = false;
   if (done) return;
   set_attr<M_ROWSUM, 0>();
+  set_attr<M_ROWSUM, 1>();
   set_attr<M_COLSUM, 0>();
   set_attr<M_COLSUM, 1>();
   set_attr<M_MAX, 0>();

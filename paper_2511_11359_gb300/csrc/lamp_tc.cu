@@ -137,7 +137,8 @@ __device__ __forceinline__ void epi_bar() { asm volatile("bar.sync 1, %0;" ::"n"
 
 // ROWS = true: G1 (fixed x tile, streamed y tiles, per-row sums of both streams)
 // ROWS = false: G2 (fixed y tile, streamed x tiles, per-column sums of both streams)
-// WC: column sweep of an evaluation pass (also accumulates sum_i z_ij X_ij for <C, X^t>)
+// WC: an evaluation pass: stream A alone (the column sweep also accumulates sum_i z_ij X_ij for
+// <C, X^t>)
 // map_fixed: 128-row boxes of the fixed operand; map_stream: 64-row boxes of the streamed one
 // MODE (row sweeps only): kSums, the iteration's sums; kMax, the row maxima of stream A's
 // exponent without row shift, a z_ij - Bq_j (the prime pass that sets the row shifts);
@@ -352,18 +353,19 @@ k_tc_sweep(const __grid_constant__ CUtensorMap map_fixed, const __grid_constant_
           for (int r = 0; r < 2; ++r) {
             const uint64_t z2 = pk(__uint_as_float(v[8 * r + 2 * p]), __uint_as_float(v[8 * r + 2 * p + 1]));
             const uint64_t vA = f2fma(ahA2, z2, f2add(ownA2[r], offA2));
-            // G1: the inner column's dB from the pair data; G2: the own column's
-            const uint64_t vB = f2fma(da2, z2, f2add(vA, ROWS ? pk(qb.x, qb.y) : ownD2[r]));
-            const float2 vAf = upk(vA), vBf = upk(vB);
+            const float2 vAf = upk(vA);
             const uint64_t eA = pk(ex2(vAf.x), ex2(vAf.y));
-            const uint64_t eB = pk(ex2(vBf.x), ex2(vBf.y));
-            if (WC) {
+            if (WC && !ROWS) {
               const uint64_t pA = f2mul(eA, wA2);
               accA[r] = f2add(accA[r], pA);
               accC[r] = f2fma(z2, pA, accC[r]);
             } else {
               accA[r] = f2fma(eA, wA2, accA[r]);
             }
+            if (WC) continue;
+            // G1: the inner column's dB from the pair data; G2: the own column's
+            const float2 vBf = upk(f2fma(da2, z2, f2add(vA, ROWS ? pk(qb.x, qb.y) : ownD2[r])));
+            const uint64_t eB = pk(ex2(vBf.x), ex2(vBf.y));
             // G1: stream B's column weight is inside dB; G2: weight by the row's q^B
             if (ROWS) accB[r] = f2add(accB[r], eB);
             else accB[r] = f2fma(eB, pk(qb.z, qb.w), accB[r]);
@@ -375,8 +377,8 @@ k_tc_sweep(const __grid_constant__ CUtensorMap map_fixed, const __grid_constant_
       for (int r = 0; r < 2 && MODE == kSums; ++r) {
         const float2 a2 = upk(accA[r]), b2 = upk(accB[r]);
         ff_add(hiA[r], loA[r], a2.x + a2.y);
-        ff_add(hiB[r], loB[r], b2.x + b2.y);
-        if (WC) {
+        if (!WC) ff_add(hiB[r], loB[r], b2.x + b2.y);
+        if (WC && !ROWS) {
           const float2 c2 = upk(accC[r]);
           ff_add(hiC[r], loC[r], c2.x + c2.y);
         }
@@ -436,14 +438,12 @@ k_tc_sweep(const __grid_constant__ CUtensorMap map_fixed, const __grid_constant_
         }
         if (ROWS) {
           if (own[r] < n) {
-            w.rowpart[((int64_t)blockIdx.y * 2 + 0) * n + own[r]] = sA;
-            w.rowpart[((int64_t)blockIdx.y * 2 + 1) * n + own[r]] = sB;
+            w.rowpart[(int64_t)blockIdx.y * (2 - WC) * n + own[r]] = sA;
+            if (!WC) w.rowpart[((int64_t)blockIdx.y * 2 + 1) * n + own[r]] = sB;
           }
         } else if (own[r] < m) {
-          constexpr int na = WC ? 3 : 2;  // the layout k_col_fin reads for this pass
-          w.colpart[((int64_t)blockIdx.y * na + 0) * m + own[r]] = sA;
-          w.colpart[((int64_t)blockIdx.y * na + 1) * m + own[r]] = sB;
-          if (WC) w.colpart[((int64_t)blockIdx.y * na + 2) * m + own[r]] = sC;
+          w.colpart[((int64_t)blockIdx.y * 2 + 0) * m + own[r]] = sA;
+          w.colpart[((int64_t)blockIdx.y * 2 + 1) * m + own[r]] = WC ? sC : sB;
         }
       }
     }
@@ -578,7 +578,8 @@ cudaError_t tc_make_map2(void* map_out, const void* base, int64_t inner, int64_t
 cudaError_t tc_prepare() {
   const int sm = (int)tc_smem_bytes();
   cudaError_t e = cudaSuccess;
-  for (const void* f : {(const void*)tc::k_tc_sweep<true, 0>, (const void*)tc::k_tc_sweep<false, 0>,
+  for (const void* f : {(const void*)tc::k_tc_sweep<true, 0>, (const void*)tc::k_tc_sweep<true, 1>,
+                        (const void*)tc::k_tc_sweep<false, 0>,
                         (const void*)tc::k_tc_sweep<false, 1>, (const void*)tc::k_tc_sweep<true, 0, tc::kMax>,
                         (const void*)tc::k_tc_sweep<true, 0, tc::kMax2>,
                         (const void*)tc::k_tc_sweep<true, 0, tc::kKmax>}) {
@@ -622,7 +623,7 @@ cudaError_t tc_launch_sweep(bool rows, int eval, const Geometry& g, const Work& 
   // G1: x fixed (128-row boxes), y streamed (64-row boxes); G2: the reverse
   const CUtensorMap& mf = *reinterpret_cast<const CUtensorMap*>(rows ? g.map_x : g.map_y);
   const CUtensorMap& ms = *reinterpret_cast<const CUtensorMap*>(rows ? g.map_y64 : g.map_x64);
-  const auto kern = rows ? tc::k_tc_sweep<true, 0> : eval ? tc::k_tc_sweep<false, 1> : tc::k_tc_sweep<false, 0>;
+  const auto kern = rows ? (eval ? tc::k_tc_sweep<true, 1> : tc::k_tc_sweep<true, 0>) : eval ? tc::k_tc_sweep<false, 1> : tc::k_tc_sweep<false, 0>;
   return launch_kernel(kern, grid, tc::kThreads, tc_smem_bytes(), st, mf, ms, w, k.n, k.m, tps, k);
 }
 
