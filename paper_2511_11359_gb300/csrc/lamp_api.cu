@@ -42,6 +42,7 @@ struct lamp_ctx {
   DevState* host_dev = &host_mirror;
   int64_t t_host = 0;    // the state's iteration index as far as the host knows (errors stop it short)
   int64_t launched = 0;  // passes launched so far, see run_passes
+  bool on_chip = false;  // iterations run in one launch (lamp_cluster.cu)
   // LAMP_PREC_BF16_TC: bf16 copies (zero padded to 128-row multiples x 64 coordinates),
   // float32 copies of the rounded points, and their TMA descriptors
   void* xb = nullptr;
@@ -625,6 +626,7 @@ static int create_impl(lamp_ctx** out, const lamp_problem* prob, const lamp_para
     k.rnx = k.s * rnx;
   }
 
+  ctx->on_chip = cluster_serves(k, g);
   {
     cudaError_t e = launch_mirror_gain(in, k, w, ctx->stream);
     if (e != cudaSuccess) return bail(fail(ctx, LAMP_E_CUDA, "mirror gain: %s", cudaGetErrorString(e)));
@@ -653,6 +655,10 @@ extern "C" int lamp_create_owned(lamp_ctx** out, const lamp_problem* prob, const
 // longer.  Later ones are graphs of check_every iterations, or of one.
 constexpr int64_t kDirectPasses = 256;
 static int run_passes(lamp_ctx* ctx, int64_t passes) {
+  if (ctx->on_chip && passes > 0) {
+    CK(launch_cluster(ctx->in, ctx->k, ctx->w, ctx->g, passes, ctx->stream));
+    return LAMP_OK;
+  }
   const int64_t L = ctx->params.check_every;
   while (passes > 0) {
     if (ctx->launched < kDirectPasses) {

@@ -546,6 +546,10 @@ bool uses_direct_sweeps(const Consts& k, int prec);
 constexpr int kDirectTile = 128;
 int direct_outer(int d);
 int direct_blocks_per_sm();
+// whole iterations of small low-dimensional problems in one launch (lamp_cluster.cu)
+bool cluster_serves(const Consts& k, const Geometry& g);
+cudaError_t launch_cluster(const Inputs& in, const Consts& k, const Work& w, const Geometry& g, int64_t passes,
+                           cudaStream_t st);
 // the same sweeps for grids below one wave (lamp_direct_small.cu)
 bool direct_small_serves(int64_t nout, int64_t nin, int d, int splits, int sms);
 cudaError_t launch_direct_small(bool rows, int eval, const Inputs& in, const Consts& k, const Work& w,
