@@ -113,7 +113,7 @@ k_pts_direct(const float* __restrict__ P_out, const float* __restrict__ P_in, in
     const float* rec = srec[buf];
 #pragma unroll 1
     for (int p0 = 0; p0 < kDPairs; p0 += kDFold) {
-#pragma unroll 2
+#pragma unroll 8
       for (int p = p0; p < p0 + kDFold; ++p) {
         DirectPair<D> t;
         t.load(rec + p * REC);

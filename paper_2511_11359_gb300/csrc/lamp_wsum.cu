@@ -177,7 +177,7 @@ k_direct_wsum(const Args a, const DevState* __restrict__ dev, const Consts k) {
     __syncthreads();
 #pragma unroll 1
     for (int p0 = 0; p0 < kPairs; p0 += kFold) {
-#pragma unroll 2
+#pragma unroll 4
       for (int p = p0; p < p0 + kFold; ++p) {
         const float* rp = srec[buf] + p * REC;
         uint64_t y2[C::DP], v2[C::VP + 1];
