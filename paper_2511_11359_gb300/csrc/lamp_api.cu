@@ -35,7 +35,7 @@ struct lamp_ctx {
   float* own_b = nullptr;  // y
   double* own_r = nullptr;
   double* own_c = nullptr;
-  // graph slots: 0 = one iteration, 1 = check_every iterations (see run_passes)
+  // graph slots: 0 = kUnitPasses iterations, 1 = check_every iterations (see run_passes)
   cudaGraphExec_t gexec[2] = {nullptr, nullptr};
   int64_t glen[2] = {0, 0};
   DevState host_mirror{};        // host copy of the control block, filled by poll()
@@ -649,11 +649,12 @@ extern "C" int lamp_create_owned(lamp_ctx** out, const lamp_problem* prob, const
   return create_impl(out, prob, params, stream, true);
 }
 
-// `passes` iterations' kernels on the context's stream.  A context's first kDirectPasses are
-// launched one by one: a graph of 50 iterations takes 0.17 ms to instantiate and 0.07 ms to
-// release, with the GPU idle, while the launches (about 2 us each) run ahead of kernels that take
-// longer.  Later ones are graphs of check_every iterations, or of one.
-constexpr int64_t kDirectPasses = 256;
+// `passes` iterations' kernels on the context's stream, as CUDA graphs: launched one by one the
+// kernels of a small problem wait for the host (2.5 us between kernels against 0.7 us in a graph;
+// 1024 points: 35 us per iteration of which 25 us are work).  A graph of 50 iterations takes 0.17
+// ms to instantiate and 0.07 ms to release, so a context starts with graphs of kUnitPasses and
+// makes one of check_every when it has run kLongRun passes.
+constexpr int64_t kUnitPasses = 10, kLongRun = 150;
 static int run_passes(lamp_ctx* ctx, int64_t passes) {
   if (ctx->on_chip && passes > 0) {
     CK(launch_cluster(ctx->in, ctx->k, ctx->w, ctx->g, passes, ctx->stream));
@@ -661,20 +662,20 @@ static int run_passes(lamp_ctx* ctx, int64_t passes) {
   }
   const int64_t L = ctx->params.check_every;
   while (passes > 0) {
-    if (ctx->launched < kDirectPasses) {
+    const int slot = ctx->launched >= kLongRun && passes >= L && L > kUnitPasses ? 1 : 0;
+    const int64_t len = slot ? L : kUnitPasses;
+    if (passes >= len) {
+      int rc = build_graph(ctx, slot, len);
+      if (rc) return rc;
+      CK(cudaGraphLaunch(ctx->gexec[slot], ctx->stream));
+      passes -= len;
+      ctx->launched += len;
+    } else {
       cudaError_t e = launch_iteration(ctx->in, ctx->k, ctx->w, ctx->g, ctx->prec, 0, ctx->stream);
       if (e != cudaSuccess) return fail(ctx, LAMP_E_CUDA, "launching an iteration: %s", cudaGetErrorString(e));
       --passes;
       ++ctx->launched;
-      continue;
     }
-    const int slot = passes >= L ? 1 : 0;
-    const int64_t len = slot ? L : 1;
-    int rc = build_graph(ctx, slot, len);
-    if (rc) return rc;
-    CK(cudaGraphLaunch(ctx->gexec[slot], ctx->stream));
-    passes -= len;
-    ctx->launched += len;
   }
   return LAMP_OK;
 }
