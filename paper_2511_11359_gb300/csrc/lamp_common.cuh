@@ -41,6 +41,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <stddef.h>
 #include <stdint.h>
 
 namespace lamp {
@@ -329,6 +330,8 @@ struct DevState {
   SweepParams spq;  // make_sweep_params of kappa_{t+2}, from the row finalize to the column finalize
 };
 
+static_assert(offsetof(DevState, cur) % 16 == 0, "read_control's 16-byte load");
+
 __host__ __device__ inline SweepF sweep_floats(const SweepParams& p) {
   SweepF f;
   f.ahA = p.ahA;
@@ -341,6 +344,13 @@ __host__ __device__ inline SweepF sweep_floats(const SweepParams& p) {
 }
 
 #ifdef __CUDACC__
+// {cur, done, status, eval_only} of the control block in one load: a kernel's first accesses are a
+// chain of L2 latencies, so the flag it may return on and the parity that the next loads need come
+// together
+__device__ __forceinline__ int4 read_control(const DevState* dev) {
+  return *reinterpret_cast<const int4*>(&dev->cur);
+}
+
 // the sweeps' constants at the current kappa: from the control block when the column
 // finalize of the previous iteration computed them for this kappa, else (first iteration
 // after a state change, evaluation passes with a kappa override) derived here in float64

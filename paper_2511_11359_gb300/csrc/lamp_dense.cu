@@ -55,7 +55,8 @@ __global__ void __launch_bounds__(kThreads, 2)
 k_dense_tma(const __grid_constant__ CUtensorMap map_c, const Work w, int64_t n, int64_t m, int tiles_per_split,
             const Consts k) {
   DevState* __restrict__ dev = w.dev;
-  if (dev->done) return;
+  const int4 ctl = read_control(dev);
+  if (ctl.y) return;  // done
   extern __shared__ __align__(128) unsigned char smem_raw[];
   unsigned char* smem =
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
@@ -65,7 +66,7 @@ k_dense_tma(const __grid_constant__ CUtensorMap map_c, const Work w, int64_t n, 
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
-  const int cur = dev->cur;
+  const int cur = ctl.x;
   const int64_t ntiles_all = ROWS ? (m + kTC - 1) / kTC : (n + kTR - 1) / kTR;
   const int64_t it0 = (int64_t)blockIdx.y * tiles_per_split;
   int64_t it1 = it0 + tiles_per_split;

@@ -44,8 +44,9 @@ k_pts_direct(const float* __restrict__ P_out, const float* __restrict__ P_in, in
   constexpr int R = C::R, DP = C::DP, REC = C::REC;
   constexpr int NACC = kDirectSums<MODE, EV>;
   const DevState* __restrict__ dev = w.dev;
-  if (dev->done) return;
-  const int cur = dev->cur;
+  const int4 ctl = read_control(dev);
+  if (ctl.y) return;  // done
+  const int cur = ctl.x;
   // row sweep: inner = columns (colq2 of the current state); column sweep: inner = rows (g2row2)
   const float4* __restrict__ pairs = MODE == M_ROWSUM ? w.colq2[cur] : w.g2row2;
   __shared__ __align__(16) float srec[2][kDPairs * REC];

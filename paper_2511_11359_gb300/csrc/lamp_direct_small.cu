@@ -31,8 +31,9 @@ k_direct_small(const float* __restrict__ P_out, const float* __restrict__ P_in, 
   constexpr int NACC = kDirectSums<MODE, EV>;
   constexpr int kPts = 32 * R;
   const DevState* __restrict__ dev = w.dev;
-  if (dev->done) return;
-  const int cur = dev->cur;
+  const int4 ctl = read_control(dev);
+  if (ctl.y) return;  // done
+  const int cur = ctl.x;
   const float4* __restrict__ pairs = MODE == M_ROWSUM ? w.colq2[cur] : w.g2row2;
   extern __shared__ __align__(16) float smem[];
   float* rec = smem;                                                   // [tiles][64 pairs][REC]

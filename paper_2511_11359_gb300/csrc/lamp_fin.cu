@@ -37,7 +37,8 @@ template <bool EVAL>
 __global__ void __launch_bounds__(kThreads)
 k_row_fin(const Work w, int splits, const double* __restrict__ r, int rowblocks, const Consts k) {
   DevState* __restrict__ dev = w.dev;
-  if (dev->done) return;
+  const int4 ctl = read_control(dev);
+  if (ctl.y) return;  // done
   if (!EVAL && (int)blockIdx.x == rowblocks) {
     if (threadIdx.x == 0) {
       SweepParams sp, spn;
@@ -53,7 +54,7 @@ k_row_fin(const Work w, int splits, const double* __restrict__ r, int rowblocks,
   const int p = threadIdx.x - role * kPts;
   const int64_t i = (int64_t)blockIdx.x * kPts + p;
   if (threadIdx.x < 128) stab[threadIdx.x] = kLogTab[threadIdx.x];
-  const int cur = dev->cur;
+  const int cur = ctl.x;
   const bool valid = i < k.n;
   double S = 0.0, ri = 0.0, snx = 0.0;
   float2 rq = make_float2(0.f, 0.f);
@@ -139,8 +140,9 @@ template <bool EVAL>
 __global__ void __launch_bounds__(kThreads)
 k_col_fin(const Work w, int splits, const double* __restrict__ cvec, int rowblocks, const Consts k) {
   DevState* __restrict__ dev = w.dev;
-  if (dev->done) return;
-  const int cur = dev->cur;
+  const int4 ctl = read_control(dev);
+  if (ctl.y) return;  // done
+  const int cur = ctl.x;
   __shared__ double snu[kPts], sq[kPts];
   __shared__ double sred[4][kThreads / 32];
   __shared__ bool amLast;
@@ -153,6 +155,9 @@ k_col_fin(const Work w, int splits, const double* __restrict__ cvec, int rowbloc
   double nun = 0.0, thn = 0.0, sny = 0.0;
   SweepParams sp, spn;
   iteration_params_of(dev, k, sp, spn);
+  // what the deciding thread needs, loaded with everything else instead of behind the last barrier
+  const long long t = dev->t, tmax = dev->tmax;
+  const double kappa = dev->kappa, tol = dev->tol;
   if (valid) {
     // partials of split s: [s][2][m], the streams' sums; evaluation passes: stream A's sums and
     // the cost-weighted ones, which the second warps take
@@ -299,22 +304,20 @@ k_col_fin(const Work w, int splits, const double* __restrict__ cvec, int rowbloc
     dev->colnu = EVAL ? Cn : NAN;
     dev->rlogZ = EVAL ? RL : NAN;
     if (EVAL) {
-      dev->t_eval = dev->t;
-      dev->kappa_eval = dev->kappa;
+      dev->t_eval = t;
+      dev->kappa_eval = kappa;
     }
-    if (dev->status != 0 || !isfinite(R)) {
-      if (dev->status == 0) dev->status = 5;
+    if (ctl.z != 0 || !isfinite(R)) {  // status: RF has completed, and CF does not set it before this point
+      if (ctl.z == 0) dev->status = 5;
       dev->done = 1;
     } else if (EVAL) {
       dev->done = 1;
-    } else if ((dev->t >= 1 && R <= dev->tol &&
-                (k.eta == 0.0 || k.infeas_only || 1.0 - dev->kappa * k.eta <= dev->tol)) ||
-               dev->t >= dev->tmax) {
+    } else if ((t >= 1 && R <= tol && (k.eta == 0.0 || k.infeas_only || 1.0 - kappa * k.eta <= tol)) || t >= tmax) {
       dev->done = 1;
     } else {
-      dev->t = dev->t + 1;
+      dev->t = t + 1;
       dev->kappa = sp.kapB;
-      dev->cur ^= 1;
+      dev->cur = cur ^ 1;
       // the next iteration's parameters, once per iteration instead of once per thread
       // (make_sweep_params of kappa_{t+2} comes from RF)
       dev->spc = spn;
@@ -322,7 +325,6 @@ k_col_fin(const Work w, int splits, const double* __restrict__ cvec, int rowbloc
       dev->swf = sweep_floats(spn);
       dev->swf_kap = spn.kapA;
     }
-    __threadfence();
   }
 }
 

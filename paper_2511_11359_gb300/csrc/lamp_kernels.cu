@@ -364,8 +364,9 @@ __global__ void __launch_bounds__(kThreads, 3)
 k_dense_rows(const float* __restrict__ C, int64_t ldc, int64_t n, int64_t m, const Work w,
              int chunks_per_split, const Consts k) {
   const DevState* __restrict__ dev = w.dev;
-  if (MODE == M_ROWSUM && dev->done) return;
-  const int cur = dev->cur;
+  const int4 ctl = read_control(dev);
+  if (MODE == M_ROWSUM && ctl.y) return;  // done
+  const int cur = ctl.x;
   const float2* __restrict__ rowshift = w.rowshift[cur];
   const float4* __restrict__ colq = w.colq[cur];
   constexpr int NV = 2 * kDR;  // values per thread: both streams of kDR rows
@@ -491,9 +492,10 @@ __global__ void __launch_bounds__(kDColThreads, 6)
 k_dense_cols(const float* __restrict__ C, int64_t ldc, int64_t n, int64_t m, const Work w, int64_t rows_per_split,
              const Consts k) {
   const DevState* __restrict__ dev = w.dev;
-  if (dev->done) return;
+  const int4 ctl = read_control(dev);
+  if (ctl.y) return;  // done
   const float4* __restrict__ g2row = w.g2row;
-  const float4* __restrict__ colq = w.colq[dev->cur];
+  const float4* __restrict__ colq = w.colq[ctl.x];
   double* __restrict__ part = w.colpart;
   const int tid = threadIdx.x;
   const int split = blockIdx.y;

@@ -152,7 +152,8 @@ __global__ void __launch_bounds__(kThreads, 2)
 k_tc_sweep(const __grid_constant__ CUtensorMap map_fixed, const __grid_constant__ CUtensorMap map_stream,
            const Work w, int64_t n, int64_t m, int tiles_per_split, const Consts k) {
   DevState* __restrict__ dev = w.dev;
-  if (dev->done) return;
+  const int4 ctl = read_control(dev);
+  if (ctl.y) return;  // done
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   // 1024-byte alignment for the swizzled tiles
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -166,7 +167,7 @@ k_tc_sweep(const __grid_constant__ CUtensorMap map_fixed, const __grid_constant_
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
-  const int cur = dev->cur;
+  const int cur = ctl.x;
   const int64_t fixed0 = (int64_t)blockIdx.x * kFixed;  // first row (G1) / column (G2) of the fixed tile
   const int64_t nstream = ROWS ? m : n;
   const int64_t ntiles_all = (nstream + kStream - 1) / kStream;
