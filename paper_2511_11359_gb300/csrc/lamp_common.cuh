@@ -537,6 +537,9 @@ cudaError_t direct_grad(bool rows, const Inputs& in, const Work& w, const Consts
 // (splits_cols) with `pairs` as the rows' data.  Writes log Z.
 cudaError_t direct_map(int side, const Inputs& in, const Work& w, const Consts& k, const float* V, int nv,
                        int splits_rows, int splits_cols, double* part, float4* pairs, float* out, cudaStream_t st);
+// rowterm_i = dr_i sum_j C_ij dc_j (dc in float32); pairs: the columns' data (scratch), part: splits x n
+cudaError_t direct_bilinear(const Inputs& in, const Work& w, const Consts& k, int splits, const double* dr,
+                            const double* dc, float4* pairs, double* part, double* rowterm, cudaStream_t st);
 cudaError_t direct_max(int mode, const Inputs& in, const Work& w, const Consts& k, int splits, cudaStream_t st);
 // finalize kernels (lamp_fin.cu)
 cudaError_t launch_mirror_gain(const Inputs& in, const Consts& k, const Work& w, cudaStream_t st);

@@ -156,8 +156,8 @@ k_round_dense_bilinear(const float* __restrict__ C, int64_t ldc, int64_t n, int6
   if (lane == 0) rowterm[i] = acc * dr[i];
 }
 
-// delta_r^T C delta_c for a point-cloud cost without a closed form (l1, l-inf): one warp
-// per row, the cost recomputed in float32, float64 accumulation per lane
+// delta_r^T C delta_c for a point-cloud cost without a closed form (l1, l-inf) and d > 8 (below:
+// direct_bilinear): one warp per row, the cost recomputed in float32, float64 accumulation per lane
 __global__ void __launch_bounds__(kT)
 k_round_pts_bilinear(const float* __restrict__ x, const float* __restrict__ y, int d, int64_t n, int64_t m,
                      const double* __restrict__ dr, const double* __restrict__ dc, double* __restrict__ rowterm,
@@ -313,14 +313,23 @@ cudaError_t launch_round(const Inputs& in, const Consts& k, const Work& w, const
   if (e != cudaSuccess) return e;
   k_round_rows<<<(unsigned)rb, kT, 0, st>>>(w, g.rows_split, in.r, in.x, dm, dr, rowp, k);
   if (!moments) {
-    // delta_r is in rowpart[0, n) (k_round_rows); per-row terms go to rowpart[n, 2n)
-    if (k.kind == COST_DENSE)
-      k_round_dense_bilinear<<<(unsigned)cdiv(k.n, kT / 32), kT, 0, st>>>(in.C, in.ldc, k.n, k.m, w.rowpart,
-                                                                         dc_tmp, w.rowpart + k.n);
-    else
-      k_round_pts_bilinear<<<(unsigned)cdiv(k.n, kT / 32), kT, 0, st>>>(in.x, in.y, k.d, k.n, k.m, w.rowpart,
-                                                                        dc_tmp, w.rowpart + k.n, k);
-    k_fields<<<1, kT, 0, st>>>(w.rowpart + k.n, k.n, 1, densef);
+    // delta_r is in rowpart[0, n) (k_round_rows); per-row terms go behind it
+    double* rowterm = w.rowpart + k.n;
+    if (k.kind == COST_DENSE) {
+      k_round_dense_bilinear<<<(unsigned)cdiv(k.n, kT / 32), kT, 0, st>>>(in.C, in.ldc, k.n, k.m, w.rowpart, dc_tmp,
+                                                                         rowterm);
+    } else if (k.shared_shift) {
+      // the packed sweep (d <= 8): its partial sums, then the row terms, behind delta_r (rowpart has
+      // 3 rows_split n doubles); the columns' pair data reuse the scratch parity
+      double* part = w.rowpart + k.n;
+      rowterm = part + (int64_t)g.rows_split * k.n;
+      e = direct_bilinear(in, w, k, g.rows_split, w.rowpart, dc_tmp, w.colq2[nx], part, rowterm, st);
+      if (e != cudaSuccess) return e;
+    } else {
+      k_round_pts_bilinear<<<(unsigned)cdiv(k.n, kT / 32), kT, 0, st>>>(in.x, in.y, k.d, k.n, k.m, w.rowpart, dc_tmp,
+                                                                       rowterm, k);
+    }
+    k_fields<<<1, kT, 0, st>>>(rowterm, k.n, 1, densef);
   }
   k_fields<<<(unsigned)nf, kT, 0, st>>>(rowp, rb, nf, rowf);
   k_fields<<<(unsigned)nf, kT, 0, st>>>(colp, cb, nf, colf);

@@ -3,7 +3,8 @@
 //
 //   k_direct_wsum  sum_b 2^{v_ab} weight_b value_b of stream A over the inner points: the
 //                  envelope gradient (values = the points' coordinates), the transport map
-//                  (value columns), and the plain row sum next to it
+//                  (value columns), and the plain row sum next to it; or, without the exponential,
+//                  Round's C delta_c of an l1 or l-inf cost
 //   k_direct_max   row maxima: the K pass, the prime pass and the eta = 0 dual bound's second
 //                  pass (launch_dual)
 //
@@ -100,6 +101,7 @@ __device__ __forceinline__ void stage_points(float* buf, int rec, const Args& a,
 }
 
 // NV value columns (COORDS: the inner points' coordinates), SUM: also the sum of the weights alone
+// (BILIN: the weights times the unscaled cost, without the exponential)
 template <int D, int NV, bool COORDS, bool SUM>
 struct SumCfg {
   static constexpr int NA = NV + (SUM ? 1 : 0);           // sums per outer point
@@ -109,7 +111,7 @@ struct SumCfg {
   static constexpr int REC = 2 * DP + 4 + 2 * VP;         // floats per pair: coordinates, {-off, w}, values
 };
 
-template <int D, int NV, bool COORDS, bool SUM>
+template <int D, int NV, bool COORDS, bool SUM, bool BILIN = false>
 __global__ void __launch_bounds__(kThreads, 2)
 k_direct_wsum(const Args a, const DevState* __restrict__ dev, const Consts k) {
   using C = SumCfg<D, NV, COORDS, SUM>;
@@ -197,7 +199,7 @@ k_direct_wsum(const Args a, const DevState* __restrict__ dev, const Consts k) {
 #pragma unroll
         for (int r = 0; r < R; ++r) {
           const uint64_t z2 = pair_cost<D>(x2[r], y2, op);
-          const uint64_t e2 = exp2_pair(ah2, al2, z2, f2add(own[r], dA.x));
+          const uint64_t e2 = BILIN ? z2 : exp2_pair(ah2, al2, z2, f2add(own[r], dA.x));
           if (NV == 0) {
             acc[r][0] = f2fma(e2, dA.y, acc[r][0]);
           } else {
@@ -316,6 +318,25 @@ k_direct_max(const Args a, const DevState* __restrict__ dev, const Consts k) {
     a.pmax[((int64_t)blockIdx.y * 2 + 0) * a.n_out + go] = mx[r];
     a.pmax[((int64_t)blockIdx.y * 2 + 1) * a.n_out + go] = MODE == kDirectKmax ? mn[r] : mx[r];
   }
+}
+
+// the weights of stream A in pair data become the float32 values of v (padding entries keep theirs, 0)
+__global__ void __launch_bounds__(256)
+k_weight_pairs(const double* __restrict__ v, int64_t np, float4* __restrict__ pairs) {
+  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e < np) reinterpret_cast<float*>(pairs + (e >> 1) * 2)[2 + (e & 1)] = (float)v[e];
+}
+
+// rowterm_i = s dr_i sum_s part[s][i]
+__global__ void __launch_bounds__(256)
+k_bilinear_fin(const double* __restrict__ part, int splits, int64_t np, const double* __restrict__ dr, double s,
+               double* __restrict__ rowterm) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= np) return;
+  double acc = 0.0;
+#pragma unroll 8
+  for (int u = 0; u < splits; ++u) acc += part[(int64_t)u * np + i];
+  rowterm[i] = s * acc * dr[i];
 }
 
 // out_i = 2 s (mass_i p_i - weight_i sum_s part[s][i]), one thread per coordinate
@@ -505,6 +526,25 @@ cudaError_t direct_map(int side, const Inputs& in, const Work& w, const Consts& 
   e = wsum::by_dim(k.d, [&](auto dd) { return wsum::go_values<decltype(dd)::value, false>(a, splits_cols, w, k, st); });
   if (e != cudaSuccess) return e;
   wsum::k_wmap_cols_fin<<<(unsigned)wsum::cdiv(k.m * nv, 256), 256, 0, st>>>(part, splits_cols, k.m, nv, w, out);
+  return cudaGetLastError();
+}
+
+cudaError_t direct_bilinear(const Inputs& in, const Work& w, const Consts& k, int splits, const double* dr,
+                            const double* dc, float4* pairs, double* part, double* rowterm, cudaStream_t st) {
+  wsum::k_weight_pairs<<<(unsigned)wsum::cdiv(k.m, 256), 256, 0, st>>>(dc, k.m, pairs);
+  wsum::Args a = wsum::side(in, k, w, true);
+  a.pairs[0] = a.pairs[1] = pairs;
+  a.part = part;
+  a.tiles_per_split = (int)wsum::cdiv(wsum::cdiv(k.m, wsum::kTile), splits);
+  cudaError_t e = wsum::by_dim(k.d, [&](auto dd) {
+    constexpr int D = decltype(dd)::value;
+    const dim3 grid((unsigned)wsum::cdiv(k.n, (int64_t)wsum::kThreads * wsum::SumCfg<D, 0, false, true>::R),
+                    (unsigned)splits);
+    wsum::k_direct_wsum<D, 0, false, true, true><<<grid, wsum::kThreads, 0, st>>>(a, w.dev, k);
+    return cudaGetLastError();
+  });
+  if (e != cudaSuccess) return e;
+  wsum::k_bilinear_fin<<<(unsigned)wsum::cdiv(k.n, 256), 256, 0, st>>>(part, splits, k.n, dr, k.s, rowterm);
   return cudaGetLastError();
 }
 
