@@ -254,7 +254,7 @@ k_cluster_iterate(const Inputs in, const Work w, const Shape s, int64_t passes, 
       if (cok && role < 2) {
         const double a = fold_sums(gs, s.groups_rows, s.tps_cols, s.own_cols, role, p);
         if (role == 0) {
-          const double A = (double)cw[p] * a;
+          const double A = __dmul_rn((double)cw[p], a);  // rounded, as the column sum that k_col_fin stores
           srp[p] = fabs(A - cj);
           const double tA = tanh(gj * (A - cj));
           const double thbar = div_seeded(tA + thj, fma(tA, thj, 1.0));
