@@ -35,13 +35,10 @@ struct lamp_ctx {
   float* own_b = nullptr;  // y
   double* own_r = nullptr;
   double* own_c = nullptr;
-  // graph slots: 0 = kUnitPasses iterations, 1 = check_every iterations (see run_passes)
-  cudaGraphExec_t gexec[2] = {nullptr, nullptr};
-  int64_t glen[2] = {0, 0};
+  cudaGraphExec_t gexec = nullptr;  // kUnitPasses iterations (see run_passes)
   DevState host_mirror{};        // host copy of the control block, filled by poll()
   DevState* host_dev = &host_mirror;
   int64_t t_host = 0;    // the state's iteration index as far as the host knows (errors stop it short)
-  int64_t launched = 0;  // passes launched so far, see run_passes
   bool on_chip = false;  // iterations run in one launch (lamp_cluster.cu)
   // LAMP_PREC_BF16_TC: bf16 copies (zero padded to 128-row multiples x 64 coordinates),
   // float32 copies of the rounded points, and their TMA descriptors
@@ -210,13 +207,9 @@ static int choose_split(int64_t tout, int64_t tin, int64_t wave, int64_t min_inn
   return best;
 }
 
-static int build_graph(lamp_ctx* ctx, int slot, int64_t len) {
-  if (ctx->gexec[slot] && ctx->glen[slot] == len) return LAMP_OK;
+static int build_graph(lamp_ctx* ctx, int64_t len) {
+  if (ctx->gexec) return LAMP_OK;
   if (!ctx->cap) CK(cudaStreamCreateWithFlags(&ctx->cap, cudaStreamNonBlocking));
-  if (ctx->gexec[slot]) {
-    cudaGraphExecDestroy(ctx->gexec[slot]);
-    ctx->gexec[slot] = nullptr;
-  }
   CK(cudaStreamBeginCapture(ctx->cap, cudaStreamCaptureModeThreadLocal));
   for (int64_t i = 0; i < len; ++i) {
     cudaError_t e = launch_iteration(ctx->in, ctx->k, ctx->w, ctx->g, ctx->prec, 0, ctx->cap);
@@ -229,10 +222,12 @@ static int build_graph(lamp_ctx* ctx, int slot, int64_t len) {
   }
   cudaGraph_t graph = nullptr;
   CK(cudaStreamEndCapture(ctx->cap, &graph));
-  cudaError_t e = cudaGraphInstantiate(&ctx->gexec[slot], graph, 0);
+  cudaError_t e = cudaGraphInstantiate(&ctx->gexec, graph, 0);
   cudaGraphDestroy(graph);
-  if (e != cudaSuccess) return fail(ctx, LAMP_E_CUDA, "cudaGraphInstantiate: %s", cudaGetErrorString(e));
-  ctx->glen[slot] = len;
+  if (e != cudaSuccess) {
+    ctx->gexec = nullptr;
+    return fail(ctx, LAMP_E_CUDA, "cudaGraphInstantiate: %s", cudaGetErrorString(e));
+  }
   return LAMP_OK;
 }
 
@@ -649,33 +644,25 @@ extern "C" int lamp_create_owned(lamp_ctx** out, const lamp_problem* prob, const
   return create_impl(out, prob, params, stream, true);
 }
 
-// `passes` iterations' kernels on the context's stream, as CUDA graphs: launched one by one the
-// kernels of a small problem wait for the host (2.5 us between kernels against 0.7 us in a graph;
-// 1024 points: 35 us per iteration of which 25 us are work).  A graph of 50 iterations takes 0.17
-// ms to instantiate and 0.07 ms to release, so a context starts with graphs of kUnitPasses and
-// makes one of check_every when it has run kLongRun passes.
-constexpr int64_t kUnitPasses = 10, kLongRun = 150;
+// `passes` iterations' kernels on the context's stream, as graphs of kUnitPasses iterations:
+// launched one by one the kernels of a small problem wait for the host (2.5 us between kernels
+// against 0.7 us in a graph; 1024 points: 35 us per iteration of which 25 us are work).  Longer
+// graphs gain nothing (1500 points, 3000 iterations: 66.0 ms with graphs of 100, 65.9 ms with
+// these) and take 5 us per iteration to make and release.
+constexpr int64_t kUnitPasses = 10;
 static int run_passes(lamp_ctx* ctx, int64_t passes) {
   if (ctx->on_chip && passes > 0) {
     CK(launch_cluster(ctx->in, ctx->k, ctx->w, ctx->g, passes, ctx->stream));
     return LAMP_OK;
   }
-  const int64_t L = ctx->params.check_every;
-  while (passes > 0) {
-    const int slot = ctx->launched >= kLongRun && passes >= L && L > kUnitPasses ? 1 : 0;
-    const int64_t len = slot ? L : kUnitPasses;
-    if (passes >= len) {
-      int rc = build_graph(ctx, slot, len);
-      if (rc) return rc;
-      CK(cudaGraphLaunch(ctx->gexec[slot], ctx->stream));
-      passes -= len;
-      ctx->launched += len;
-    } else {
-      cudaError_t e = launch_iteration(ctx->in, ctx->k, ctx->w, ctx->g, ctx->prec, 0, ctx->stream);
-      if (e != cudaSuccess) return fail(ctx, LAMP_E_CUDA, "launching an iteration: %s", cudaGetErrorString(e));
-      --passes;
-      ++ctx->launched;
-    }
+  for (; passes >= kUnitPasses; passes -= kUnitPasses) {
+    int rc = build_graph(ctx, kUnitPasses);
+    if (rc) return rc;
+    CK(cudaGraphLaunch(ctx->gexec, ctx->stream));
+  }
+  for (; passes > 0; --passes) {
+    cudaError_t e = launch_iteration(ctx->in, ctx->k, ctx->w, ctx->g, ctx->prec, 0, ctx->stream);
+    if (e != cudaSuccess) return fail(ctx, LAMP_E_CUDA, "launching an iteration: %s", cudaGetErrorString(e));
   }
   return LAMP_OK;
 }
@@ -819,11 +806,8 @@ static int ensure_part_width(lamp_ctx* ctx, int width) {
     ctx->allocs.erase(it);
     cudaFree(old);
   }
-  for (int s = 0; s < 2; ++s) {
-    if (ctx->gexec[s]) cudaGraphExecDestroy(ctx->gexec[s]);
-    ctx->gexec[s] = nullptr;
-    ctx->glen[s] = 0;
-  }
+  if (ctx->gexec) cudaGraphExecDestroy(ctx->gexec);
+  ctx->gexec = nullptr;
   int rc = dalloc(ctx, &ctx->w.rowpart, (size_t)ctx->g.rows_split * width * ctx->k.n);
   if (!rc) rc = dalloc(ctx, &ctx->w.colpart, (size_t)ctx->g.cols_split * width * ctx->k.m);
   if (rc) return rc;
@@ -1232,8 +1216,7 @@ extern "C" const char* lamp_last_error(const lamp_ctx* ctx) { return ctx ? ctx->
 extern "C" void lamp_destroy(lamp_ctx* ctx) {
   if (!ctx) return;
   if (ctx->stream) cudaStreamSynchronize(ctx->stream);
-  for (int s = 0; s < 2; ++s)
-    if (ctx->gexec[s]) cudaGraphExecDestroy(ctx->gexec[s]);
+  if (ctx->gexec) cudaGraphExecDestroy(ctx->gexec);
   for (void* p : ctx->allocs) cudaFree(p);
   if (ctx->cap) cudaStreamDestroy(ctx->cap);
   if (ctx->gside) {
