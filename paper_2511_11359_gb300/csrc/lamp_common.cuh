@@ -476,6 +476,8 @@ int dense_tile_cols();
 int dense_blocks_per_sm();
 cudaError_t dense_launch_sweep(bool rows, int eval, const Geometry& g, const Work& w, const Consts& k, int splits,
                                cudaStream_t st);
+cudaError_t dense_launch_rowmax(int mode, const Geometry& g, const Work& w, const Consts& k, int splits,
+                                cudaStream_t st);
 // tensor-core gradient pass (lamp_tc_grad.cu): transposed bf16 copies (64 x np_pad), one side
 // of the pass (float32 partials [splits][np][64]) and its finalize
 size_t tcg_smem_bytes();

@@ -50,13 +50,15 @@ struct __align__(8) Bars {
 constexpr size_t kSmemBytes = (size_t)kStages * kTileBytes + (size_t)kStages * kAuxMax * sizeof(float4) + 128 + 128;
 
 // WC = 1: an evaluation pass (stream A alone; the column sums also weighted by the cost)
-template <bool ROWS, int WC>
+// MX (row sweeps): 0 sums; 1 row maxima of both streams' exponents without row shift (the prime
+// pass); 2 of stream A's with the row shifts and the column remainders subtracted (launch_dual)
+template <bool ROWS, int WC, int MX = 0>
 __global__ void __launch_bounds__(kThreads, 2)
 k_dense_tma(const __grid_constant__ CUtensorMap map_c, const Work w, int64_t n, int64_t m, int tiles_per_split,
             const Consts k) {
   DevState* __restrict__ dev = w.dev;
   const int4 ctl = read_control(dev);
-  if (ctl.y) return;  // done
+  if (MX == 0 && ctl.y) return;  // done
   extern __shared__ __align__(128) unsigned char smem_raw[];
   unsigned char* smem =
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
@@ -120,13 +122,16 @@ k_dense_tma(const __grid_constant__ CUtensorMap map_c, const Work w, int64_t n, 
       uint64_t oA2[4], oB2[4];
 #pragma unroll
       for (int a = 0; a < 4; ++a) {
-        const float2 q = w.rowshift[cur][g0 + a < n ? g0 + a : n - 1];
+        const float2 q = MX == 1 ? make_float2(0.f, 0.f) : w.rowshift[cur][g0 + a < n ? g0 + a : n - 1];
         oA2[a] = pk(-q.x, -q.x);
         oB2[a] = pk(-q.y, -q.y);
       }
-      float hi[8], lo[8];  // float-float sums [2 row + stream]
+      float hi[8], lo[8];  // float-float sums [2 row + stream], or the maxima in hi
 #pragma unroll
-      for (int q = 0; q < 8; ++q) hi[q] = lo[q] = 0.f;
+      for (int q = 0; q < 8; ++q) {
+        hi[q] = MX ? -INFINITY : 0.f;
+        lo[q] = 0.f;
+      }
       bool ok = true;
       for (int i = 0; i < ntiles; ++i) {
         const int s = i % kStages;
@@ -147,6 +152,18 @@ k_dense_tma(const __grid_constant__ CUtensorMap map_c, const Work w, int64_t n, 
 #pragma unroll
           for (int a = 0; a < 4; ++a) {
             const uint64_t z2 = pk(tC[a * kTC + c0], tC[a * kTC + c1]);
+            if constexpr (MX == 1) {
+              const float2 uA = upk(f2fma(ahA2, z2, f2sub(0ull, xA2))), uB = upk(f2fma(ahB2, z2, f2sub(0ull, xB2)));
+              hi[2 * a] = fmaxf(hi[2 * a], fmaxf(uA.x, uA.y));
+              hi[2 * a + 1] = fmaxf(hi[2 * a + 1], fmaxf(uB.x, uB.y));
+              continue;
+            }
+            if constexpr (MX == 2) {
+              const float2 u =
+                  upk(f2sub(f2fma(alA2, z2, f2fma(ahA2, z2, f2sub(oA2[a], xA2))), pk(d0.y, d1.y)));
+              hi[2 * a] = fmaxf(hi[2 * a], fmaxf(u.x, u.y));
+              continue;
+            }
             const float2 eA = upk(exp2_pair(ahA2, alA2, z2, f2sub(oA2[a], xA2)));
             sA[a] = __fmaf_rn(eA.y, d1.y, __fmaf_rn(eA.x, d0.y, sA[a]));
             if (!WC) {
@@ -156,7 +173,7 @@ k_dense_tma(const __grid_constant__ CUtensorMap map_c, const Work w, int64_t n, 
           }
         }
 #pragma unroll
-        for (int a = 0; a < 4; ++a) {
+        for (int a = 0; a < 4 && !MX; ++a) {
           ff_add(hi[2 * a], lo[2 * a], sA[a]);
           ff_add(hi[2 * a + 1], lo[2 * a + 1], sB[a]);
         }
@@ -167,11 +184,22 @@ k_dense_tma(const __grid_constant__ CUtensorMap map_c, const Work w, int64_t n, 
       }
       // warp-uniform: the reduction below needs every lane
       if (__all_sync(0xffffffffu, ok && !*(volatile int*)&B->err)) {
-        warp_sums_ff<8>(hi, lo, lane);  // value lane / 4: row (lane / 8), stream (lane / 4) % 2
-        const int64_t gi = g0 + (lane >> 3);
-        const int q = (lane >> 2) & 1;
-        if ((lane & 3) == 0 && gi < n && q < 2 - WC)
-          w.rowpart[((int64_t)blockIdx.y * (2 - WC) + q) * n + gi] = (double)hi[0] + (double)lo[0];
+        if constexpr (MX != 0) {
+#pragma unroll
+          for (int q = 0; q < 8; ++q) {
+            float v = hi[q];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+            const int64_t gi = g0 + (q >> 1);
+            if (lane == 0 && gi < n) w.rowmax[((int64_t)blockIdx.y * 2 + (q & 1)) * n + gi] = v;
+          }
+        } else {
+          warp_sums_ff<8>(hi, lo, lane);  // value lane / 4: row (lane / 8), stream (lane / 4) % 2
+          const int64_t gi = g0 + (lane >> 3);
+          const int q = (lane >> 2) & 1;
+          if ((lane & 3) == 0 && gi < n && q < 2 - WC)
+            w.rowpart[((int64_t)blockIdx.y * (2 - WC) + q) * n + gi] = (double)hi[0] + (double)lo[0];
+        }
       }
     } else {
       // ---------------- G2: column 32 warp + lane of this column block ----------------
@@ -252,6 +280,7 @@ cudaError_t dense_make_map(void* map_out, const float* C, int64_t n, int64_t m, 
 cudaError_t dense_prepare() {
   cudaError_t e = cudaSuccess;
   for (const void* f : {(const void*)dense::k_dense_tma<true, 0>, (const void*)dense::k_dense_tma<true, 1>,
+                        (const void*)dense::k_dense_tma<true, 0, 1>, (const void*)dense::k_dense_tma<true, 0, 2>,
                         (const void*)dense::k_dense_tma<false, 0>,
                         (const void*)dense::k_dense_tma<false, 1>}) {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dense::kSmemBytes);
@@ -279,6 +308,17 @@ cudaError_t dense_launch_sweep(bool rows, int eval, const Geometry& g, const Wor
   const CUtensorMap& map = *reinterpret_cast<const CUtensorMap*>(g.map_c);
   const auto kern = rows ? (eval ? dense::k_dense_tma<true, 1> : dense::k_dense_tma<true, 0>) : eval ? dense::k_dense_tma<false, 1> : dense::k_dense_tma<false, 0>;
   return launch_kernel(kern, grid, dense::kThreads, dense::kSmemBytes, st, map, w, k.n, k.m, tps, k);
+}
+
+// Row maxima per split into w.rowmax: mode 1 the prime pass, 2 the refined pass of the dual bound.
+// Bound by HBM as the sweeps are; a kernel of plain loads took 237 us at 16384 x 16384.
+cudaError_t dense_launch_rowmax(int mode, const Geometry& g, const Work& w, const Consts& k, int splits,
+                                cudaStream_t st) {
+  const int64_t ntiles = (k.m + dense::kTC - 1) / dense::kTC;
+  const int tps = (int)((ntiles + splits - 1) / splits);
+  const dim3 grid((unsigned)((k.n + dense::kTR - 1) / dense::kTR), (unsigned)splits);
+  return launch_kernel(mode == 1 ? dense::k_dense_tma<true, 0, 1> : dense::k_dense_tma<true, 0, 2>, grid, dense::kThreads,
+                       dense::kSmemBytes, st, *reinterpret_cast<const CUtensorMap*>(g.map_c), w, k.n, k.m, tps, k);
 }
 
 }  // namespace lamp

@@ -349,10 +349,9 @@ k_pts_sweep(const float* __restrict__ P_out, const float* __restrict__ P_in, int
 // Row sweep: a CTA of 256 threads owns kDR rows and steps over chunks of 1024 columns (thread t
 // takes columns t + 256 q); column sweep: a CTA of 128 threads owns 256 columns (two per thread)
 // and walks a split's rows in groups of 16.  These serve stored costs whose rows are not a
-// multiple of 16 bytes apart (lamp_dense.cu streams the others) and the row-max passes of all
-// stored costs.  Bound by the latency of the loads at the sizes that fit the L2 and by HBM above:
-// the next chunk's (group's) entries are loaded while the current one is evaluated, and the grid
-// is fine enough to fill the SMs.  3001 x 2777: 19.9 -> 12.3 us (rows; 8 rows per CTA, no load
+// multiple of 16 bytes apart (lamp_dense.cu streams the others).  Bound by the latency of the
+// loads at the sizes that fit the L2 and by HBM above: the next chunk's (group's) entries are
+// loaded while the current one is evaluated, and the grid is fine enough to fill the SMs.  3001 x 2777: 19.9 -> 12.3 us (rows; 8 rows per CTA, no load
 // ahead, a butterfly of five steps per sum), 20.4 -> 13.9 us (columns; 1024 columns per CTA).
 constexpr int kDR = 4;          // rows per CTA in the row sweep
 constexpr int kDSplitRows = 8;  // rows per tile in the choice of its splits
@@ -831,7 +830,9 @@ cudaError_t launch_init_state(const Inputs& in, const Consts& k, const Work& w, 
 
 static cudaError_t launch_row_sweep(const Inputs& in, const Consts& k, const Work& w, const Geometry& g, int mode,
                                     int eval, cudaStream_t st) {
-  if (k.kind == COST_DENSE && g.map_c && mode == M_ROWSUM) return dense_launch_sweep(true, eval, g, w, k, g.rows_split, st);
+  if (k.kind == COST_DENSE && g.map_c)
+    return mode == M_ROWSUM ? dense_launch_sweep(true, eval, g, w, k, g.rows_split, st)
+                            : dense_launch_rowmax(mode == M_MAX2 ? 2 : 1, g, w, k, g.rows_split, st);
   if (k.kind == COST_DENSE) {
     int64_t nch = cdiv(k.m, kDChunk);
     int cps = (int)cdiv(nch, g.rows_split);

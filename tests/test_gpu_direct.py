@@ -78,6 +78,25 @@ def test_stored_cost_unaligned_rows(n, m):
     sol.close()
 
 
+@pytest.mark.parametrize("n,m", [(1, 4), (31, 260), (33, 1028), (300, 2052)])
+def test_stored_cost_row_maxima(n, m):
+    """Row maxima of stored costs read by tensor copies (32 x 256 tiles): the shifts of a run that
+    resumes from a given state, and the dual bound's refined maxima."""
+    w = W.dense_problem(f"mx{n}", n, m, seed=n + m)
+    C, s, K = oracle_cost(w)
+    P = O.LampParams(K=K)
+    mid, ref = O.lamp_run(C, w.r, w.c, P, 20), O.lamp_run(C, w.r, w.c, P, 30)
+    sol, _, _ = gpu_solver(w, K=K, check_every=7)
+    sol.set_state(mid.nu, mid.theta, mid.kappa, mid.t)
+    dual = max(O.saddle_dual(C, w.r, w.c, K, mid.theta), O.saddle_dual(C, w.r, w.c, K, mid.nu))
+    assert abs(sol.objective()["dual"] - dual) <= 1e-9 * K
+    sol.iterate(10)
+    st = sol.get_state()
+    tol = cost_slack(w, ref.kappa)
+    assert np.abs(st["nu"] - ref.nu).max() <= tol and np.abs(st["theta"] - ref.theta).max() <= tol
+    sol.close()
+
+
 @pytest.mark.parametrize("n,m,d,cost,eta", [(1, 1, 1, "sqeuclid", 0.0), (2, 1024, 8, "sqeuclid", 0.0),
                                             (1024, 129, 3, "l1", 0.0), (97, 130, 2, "linf", 0.0),
                                             (256, 256, 2, "sqeuclid", 0.0), (500, 641, 4, "sqeuclid", 1e-2)])
