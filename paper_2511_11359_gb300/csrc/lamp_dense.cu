@@ -92,11 +92,7 @@ k_dense_tma(const __grid_constant__ CUtensorMap map_c, const Work w, int64_t n, 
       int issued = 0;
       for (int i = 0; i < ntiles; ++i) {
         const int s = i % kStages;
-        if (i >= kStages) {
-          if (!async::mbar_wait(&B->empty[s], ((i / kStages) & 1) ^ 1, &B->err, dev)) break;
-          // the slot was read through the generic proxy; the copies below are async-proxy writes
-          async::fence_proxy_async_smem();
-        }
+        if (i >= kStages && !async::mbar_wait(&B->empty[s], ((i / kStages) & 1) ^ 1, &B->err, dev)) break;
         const int64_t t = it0 + i;
         async::mbar_expect_tx(&B->full[s], kTileBytes + kAux * (uint32_t)sizeof(float4));
         if (ROWS) {
@@ -181,6 +177,9 @@ k_dense_tma(const __grid_constant__ CUtensorMap map_c, const Work w, int64_t n, 
           ff_add(hi[2 * a], lo[2 * a], sA[a]);
           ff_add(hi[2 * a + 1], lo[2 * a + 1], sB[a]);
         }
+        // the tile was read through the generic proxy; the next tensor copy into it is an
+        // async-proxy write
+        async::fence_proxy_async_smem();
         async::mbar_arrive(&B->empty[s]);
       }
       // warp-uniform: the reduction below needs every lane
@@ -239,6 +238,7 @@ k_dense_tma(const __grid_constant__ CUtensorMap map_c, const Work w, int64_t n, 
         ff_add(hA, lA, sA);
         if (WC) ff_add(hC, lC, sCx);
         else ff_add(hB, lB, sB);
+        async::fence_proxy_async_smem();
         async::mbar_arrive(&B->empty[s]);
       }
       if (ok && !*(volatile int*)&B->err && gj < m) {
