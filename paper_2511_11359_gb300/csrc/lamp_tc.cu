@@ -114,25 +114,6 @@ __device__ __forceinline__ void tmem_wait_ld(uint32_t (&v)[16]) {
                : "memory");
 }
 
-
-
-// barrier over the epilogue threads (named barrier 1) returning the OR of `v`
-// across them, so that every epilogue warp takes the same branch
-__device__ __forceinline__ bool epi_bar_or(bool v) {
-  uint32_t r;
-  asm volatile(
-      "{\n"
-      ".reg .pred p, q;\n"
-      "setp.ne.u32 p, %1, 0;\n"
-      "bar.red.or.pred q, 1, %2, p;\n"
-      "selp.u32 %0, 1, 0, q;\n"
-      "}\n"
-      : "=r"(r)
-      : "r"((uint32_t)v), "n"(kEpiThreads)
-      : "memory");
-  return r != 0;
-}
-
 __device__ __forceinline__ void epi_bar() { asm volatile("bar.sync 1, %0;" ::"n"(kEpiThreads) : "memory"); }
 
 // ROWS = true: G1 (fixed x tile, streamed y tiles, per-row sums of both streams)

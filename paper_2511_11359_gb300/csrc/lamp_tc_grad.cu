@@ -242,7 +242,8 @@ k_tc_grad(const __grid_constant__ CUtensorMap map_fixed, const __grid_constant__
           umma_commit(&B->s_full[b]);
           any = true;
           // the slot of tile i - kBufs is free: its offsets and weights were read through the generic
-          // proxy, and the copies are async-proxy writes
+          // proxy (into P, which the epilogue had stored before it released the tile), and the copies
+          // are async-proxy writes
           if (i >= kBufs && issued < ntiles) {
             fence_proxy_async_smem();
             load();
