@@ -200,11 +200,12 @@ LAMP_API int lamp_objective(lamp_ctx* ctx, double out[LAMP_OBJECTIVE_SLOTS]);
  *   side 0: out = p V      (V: device m x k float32 row-major; out: device n x k)
  *   side 1: out = p^T U    (U: device n x k float32 row-major; out: device m x k)
  * 1 <= k <= 8 value columns (colour channels, coordinates: p y is the barycentric map).
- * One evaluation pass, then one recompute sweep of X^t over all n m entries with
- * float32 exponents as in the iteration and float64 accumulation across tiles.
- * The first call with k larger than the context's partial-sum width (3, or d for
- * |x - y|^2 with d <= 8) widens two O(k (n + m) splits) buffers (LAMP_E_NOMEM if that
- * fails).  Asynchronous on the context's stream after the evaluation pass. */
+ * Point clouds with d <= 8: one recompute sweep of X^t that forms the row sums on the way
+ * (side 1: a row-sum sweep and one recompute sweep); it leaves log Z of X^t, not col(X^t).
+ * Others: one evaluation pass, then one recompute sweep.  float32 exponents as in the
+ * iteration.  The first call, and one with a larger k, may allocate O(k (n + m) splits)
+ * partial sums (LAMP_E_NOMEM if that fails).  Asynchronous on the context's stream, for d > 8
+ * and stored costs after the evaluation pass. */
 LAMP_API int lamp_apply_map(lamp_ctx* ctx, const float* V, int64_t k, float* out, int side);
 
 /* Dual function of the saddle problem (App. B, Eqs. def:dual_spp, def:dual_spp_e)
@@ -240,7 +241,7 @@ LAMP_API int lamp_round(lamp_ctx* ctx, double out[4], double* y, double* delta_r
  * dx: device n x d float32, dy: device m x d float32 (either may be NULL).
  * One evaluation pass (skipped when the state's X^t was the last one evaluated, e.g. after
  * lamp_solve or lamp_objective), then per side one recompute pass (X never stored):
- *   LAMP_PREC_FP32: ceil(d / 8) float32 sweeps per side (chunks of 8 coordinates);
+ *   LAMP_PREC_FP32: one float32 sweep per side (the first call allocates its partial sums);
  *   LAMP_PREC_BF16_TC: one tensor-core pass per side on the bf16-rounded points the
  *   context solves with: S = x.y^T by tcgen05, the coupling's entries formed in the
  *   epilogue and split into two bf16 parts (16 significant bits), sum_j X_ij y_j by a
@@ -302,7 +303,9 @@ LAMP_API int lamp_measure_ex2_rate(double* ex2_per_clk_per_sm);
  * LAMP_E_CUDA.  The device stays usable afterwards.  Synchronises. */
 LAMP_API int lamp_selftest_wait_timeout(int64_t polls, int* status);
 
-/* Number of kernel launches one iteration issues (for launch accounting). */
+/* Number of kernel launches one iteration issues when its kernels are launched one by one
+ * (lamp_time_kernels; for launch accounting).  lamp_iterate and lamp_solve launch the same kernels
+ * from graphs, and run small point clouds (d <= 8, n and m <= 1024) several iterations to a launch. */
 LAMP_API int64_t lamp_launches_per_iteration(const lamp_ctx* ctx);
 
 LAMP_API const char* lamp_last_error(const lamp_ctx* ctx);
