@@ -64,12 +64,10 @@ k_row_fin(const Work w, int splits, const double* __restrict__ r, int rowblocks,
     rq = w.rowshift[cur][i];
     ri = r[i];
     if (k.zdot && (EVAL || !k.shared_shift)) snx = k.s * w.nx[i];
-    // the partials' loads are independent and in flight together; the sums keep the split order
-    // (evaluation passes sweep stream A alone: one sum per split, read by both warps)
+    // evaluation passes sweep stream A alone: one sum per split, read by both warps
     constexpr int na = EVAL ? 1 : 2;
     const double* __restrict__ part = w.rowpart + (int64_t)(EVAL ? 0 : role) * k.n + i;
-#pragma unroll 8
-    for (int s = 0; s < splits; ++s) S += part[(int64_t)s * na * k.n];
+    S = split_sum(part, (int64_t)na * k.n, splits);
     if (!in_range(S)) {
       atomicExch(&dev->status, 5 /* LAMP_E_NUMERIC */);
       S = 1.0;
@@ -168,10 +166,7 @@ k_col_fin(const Work w, int splits, const double* __restrict__ cvec, int rowbloc
     const double gj = EVAL ? 0.0 : w.gj[j];
     const double* __restrict__ part = w.colpart + (int64_t)role * k.m + j;
     if (k.zdot) sny = k.s * w.ny[j];
-    double a = 0.0;
-    // the partials' loads are independent and in flight together; the sums keep the split order
-#pragma unroll 8
-    for (int s = 0; s < splits; ++s) a += part[(int64_t)s * na * k.m];
+    double a = split_sum(part, (int64_t)na * k.m, splits);
     if (EVAL && role) zsum = (double)cq.y * a;
     if (role == 0) {
       const double A = (double)cq.y * a;  // col(X^t)_j
