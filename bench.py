@@ -59,13 +59,13 @@ NCU_TRAFFIC = {
     ("highdim", "bf16_tc", 32768, 64): {
         "sources": ["paper_2511_11359_gb300/csrc/lamp_tc.cu", "paper_2511_11359_gb300/csrc/lamp_tc.cuh",
                     "paper_2511_11359_gb300/csrc/lamp_async.cuh", "paper_2511_11359_gb300/csrc/lamp_common.cuh"],
-        "sha256": "7c3a6dc1c18d6bdc294b81a37c05316fd98c0753effa207139a19e8aa6b02602",
-        "row_sweep": 9203712, "col_sweep": 9990144},
+        "sha256": "92caa86dd35da0e2d36fd75273dd237ead316436807c81fe48e7d6238dcd74ba",
+        "row_sweep": 9203712, "col_sweep": 9990400},
     ("image_grid", "fp32", 4096, 0): {
         "sources": ["paper_2511_11359_gb300/csrc/lamp_dense.cu", "paper_2511_11359_gb300/csrc/lamp_async.cuh",
                     "paper_2511_11359_gb300/csrc/lamp_common.cuh"],
-        "sha256": "61d2c461514d13861b82ae999b5ce9986d3999b359c1fba50280d88da1925b2a",
-        "row_sweep": 67246848 + 244224, "col_sweep": 67254016 + 358912},
+        "sha256": "71a85ed497bf04eabc18e41ca97860370dae675b4a09e98565429335bee8906b",
+        "row_sweep": 67231488 + 82688, "col_sweep": 67252736 + 100864},
 }
 
 

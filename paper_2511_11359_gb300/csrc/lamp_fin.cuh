@@ -144,7 +144,7 @@ __device__ __forceinline__ void add_group(double& a, const double* __restrict__ 
 
 // 0 + p[0] + p[stride] + ... in split order.  The adds are one dependent chain of float64 (64 cycles
 // each) and the loads of a group of 8 take as long as its adds, so the next group is loaded while
-// one is added: column finalize of 3001 x 2777 (41 splits) 18.4 -> 15.4 us between events, of
+// one is added: column finalize of 3001 x 2777 (41 splits) 18.4 -> 14.3 us between events, 50
 // iterations there 2.25 -> 2.08 ms, on 4096 x 4096 2.15 -> 2.11.  No guarded adds: one that is
 // predicated off takes its 64 cycles too.
 __device__ __forceinline__ double split_sum(const double* __restrict__ p, int64_t stride, int splits) {
