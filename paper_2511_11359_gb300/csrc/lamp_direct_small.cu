@@ -84,6 +84,7 @@ k_direct_small(const float* __restrict__ P_out, const float* __restrict__ P_in, 
 #pragma unroll
       for (int q = 0; q < NACC; ++q) acc[r][q] = 0ull;
     const float* rp = rec + (size_t)g * kDFold * REC;
+    // 40.5 -> 38.5 us at 8192 points against an unroll of 2
 #pragma unroll 4
     for (int p = 0; p < kDFold; ++p) {
       DirectPair<D> t;

@@ -15,7 +15,7 @@
 // gain is kept per column, divisions start from a float32 reciprocal, the row shift's log2
 // comes from a table, and the parameters of the next iteration are prepared by a block of RF
 // instead of by CF's last thread.  RF + CF together, against one thread per point doing all of
-// it in blocks of 128: 22.9 -> 12.8 us at 4096 points (16 splits), 37.5 -> 24.4 us at 2^15 (19
+// it in blocks of 128: 22.9 -> 12.0 us at 4096 points (16 splits), 37.5 -> 23.1 us at 2^15 (19
 // splits).
 #include <cmath>
 

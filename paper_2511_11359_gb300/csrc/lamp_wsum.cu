@@ -179,6 +179,7 @@ k_direct_wsum(const Args a, const DevState* __restrict__ dev, const Consts k) {
     __syncthreads();
 #pragma unroll 1
     for (int p0 = 0; p0 < kPairs; p0 += kFold) {
+      // transport map of 65536 x 16384: 605 -> 582 us against an unroll of 2
 #pragma unroll 4
       for (int p = p0; p < p0 + kFold; ++p) {
         const float* rp = srec[buf] + p * REC;
