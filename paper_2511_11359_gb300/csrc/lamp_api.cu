@@ -115,6 +115,7 @@ static int ensure_dot_copies(lamp_ctx* ctx) {
   const Consts& k = ctx->k;
   int rc;
   if (!ctx->w.xt) {
+    CK(dot_prepare());  // a tensor-core context's first transport map
     if ((rc = dalloc(ctx, &ctx->w.xt, (size_t)dot_pad(k.n) * k.d))) return rc;
     if ((rc = dalloc(ctx, &ctx->w.yt, (size_t)dot_pad(k.m) * k.d))) return rc;
     ctx->dot_fresh = false;
@@ -286,6 +287,7 @@ static int create_impl(lamp_ctx** out, const lamp_problem* prob, const lamp_para
   ctx->prec = params->prec;
   ctx->stream = (cudaStream_t)stream;
   auto bail = [&](int code) {
+    if (!ctx->err.empty()) g_err = ctx->err;  // the context goes: its message stays readable
     lamp_destroy(ctx);
     return code;
   };
@@ -297,7 +299,6 @@ static int create_impl(lamp_ctx** out, const lamp_problem* prob, const lamp_para
       return LAMP_E_CUDA;
     }
   }
-  prepare_kernels();
   if (params->prec == LAMP_PREC_BF16_TC) {
     cudaError_t e = tc_prepare();
     if (e != cudaSuccess) {
@@ -326,6 +327,10 @@ static int create_impl(lamp_ctx** out, const lamp_problem* prob, const lamp_para
   k.alpha_m = params->alpha / (double)prob->m;
   k.clipb = std::tanh(params->beta / 2.0);
   ctx->log_m = std::log((double)k.m);
+  {
+    cudaError_t e = prepare_kernels(k, ctx->prec);
+    if (e != cudaSuccess) return bail(fail(ctx, LAMP_E_CUDA, "kernel setup: %s", cudaGetErrorString(e)));
+  }
 
   // inputs
   Inputs& in = ctx->in;

@@ -460,7 +460,7 @@ cudaError_t launch_rowmax_refined(const Inputs& in, const Consts& k, const Work&
 // of every row and the column sweep also accumulates <C, X^t>
 cudaError_t launch_iteration(const Inputs& in, const Consts& k, const Work& w, const Geometry& g, int prec,
                              int eval, cudaStream_t st);
-void prepare_kernels();
+cudaError_t prepare_kernels(const Consts& k, int prec);
 // tcgen05 path (lamp_tc.cu)
 size_t tc_smem_bytes();
 int64_t tc_pad(int64_t v);
@@ -522,7 +522,7 @@ cudaError_t launch_dual(const Inputs& in, const Consts& k, const Work& w, const 
 enum DotMode : int { kDotRowSum, kDotColSum, kDotRowEval, kDotColEval, kDotMax, kDotMax2, kDotKmax };
 int64_t dot_pad(int64_t np);
 cudaError_t dot_transpose(const float* P, int64_t np, int d, float* out, cudaStream_t st);
-void dot_prepare();
+cudaError_t dot_prepare();
 int dot_tile();
 cudaError_t dot_launch(int mode, const Work& w, const Consts& k, const Geometry& g, cudaStream_t st);
 cudaError_t dot_weighted(bool rows, const Work& w, const Consts& k, const float* values, int dv, const float4* off,

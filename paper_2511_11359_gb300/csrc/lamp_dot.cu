@@ -634,30 +634,27 @@ cudaError_t launch_mode(const dot::Args& a, const Work& w, const Consts& k, int 
   return launch_kernel(dot::k_dot_sweep<MODE>, grid, dot::kThreads, dot::smem_floats(a.d) * sizeof(float), st, a, w.dev, k);
 }
 
-template <int MODE>
-void set_smem() {
-  cudaFuncSetAttribute(dot::k_dot_sweep<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)(dot::smem_floats(64) * sizeof(float)));
+template <class K>
+cudaError_t set_smem(K kern, size_t floats) {
+  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(floats * sizeof(float)));
 }
 
 }  // namespace
 
-void dot_prepare() {
-  set_smem<dot::kRowSum>();
-  set_smem<dot::kColSum>();
-  set_smem<dot::kRowEval>();
-  set_smem<dot::kColEval>();
-  set_smem<dot::kMax>();
-  set_smem<dot::kMax2>();
-  set_smem<dot::kKmax>();
-  cudaFuncSetAttribute(dot::k_dot_grad<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)(dot::grad_smem_floats<2>(64) * sizeof(float)));
-  cudaFuncSetAttribute(dot::k_dot_grad<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)(dot::grad_smem_floats<4>(64) * sizeof(float)));
-  cudaFuncSetAttribute(dot::k_dot_grad<6>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)(dot::grad_smem_floats<6>(64) * sizeof(float)));
-  cudaFuncSetAttribute(dot::k_dot_grad<8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)(dot::grad_smem_floats<8>(64) * sizeof(float)));
+// the shared-memory limits of these kernels on the current device
+cudaError_t dot_prepare() {
+  const size_t sweep = dot::smem_floats(64);
+  for (const auto kern : {dot::k_dot_sweep<dot::kRowSum>, dot::k_dot_sweep<dot::kColSum>, dot::k_dot_sweep<dot::kRowEval>,
+                          dot::k_dot_sweep<dot::kColEval>, dot::k_dot_sweep<dot::kMax>, dot::k_dot_sweep<dot::kMax2>,
+                          dot::k_dot_sweep<dot::kKmax>}) {
+    const cudaError_t e = set_smem(kern, sweep);
+    if (e != cudaSuccess) return e;
+  }
+  cudaError_t e = set_smem(dot::k_dot_grad<2>, dot::grad_smem_floats<2>(64));
+  if (e == cudaSuccess) e = set_smem(dot::k_dot_grad<4>, dot::grad_smem_floats<4>(64));
+  if (e == cudaSuccess) e = set_smem(dot::k_dot_grad<6>, dot::grad_smem_floats<6>(64));
+  if (e == cudaSuccess) e = set_smem(dot::k_dot_grad<8>, dot::grad_smem_floats<8>(64));
+  return e;
 }
 
 int dot_tile() { return dot::kOut; }

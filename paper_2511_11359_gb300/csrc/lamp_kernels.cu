@@ -927,32 +927,26 @@ cudaError_t launch_iteration(const Inputs& in, const Consts& k, const Work& w, c
 int launches_per_iteration(const Consts& k, int prec) { return 4; }
 
 template <int MODE, int DG>
-static void set_attr() {
+static cudaError_t set_attr() {
   const int sm = (int)pts_smem(64, DG);
-  cudaFuncSetAttribute(k_pts_sweep<MODE, DG>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+  return cudaFuncSetAttribute(k_pts_sweep<MODE, DG>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
 }
 
-// raise the dynamic shared-memory limit of every sweep instantiation once, before any capture
-void prepare_kernels() {
-  static bool done = false;
-  if (done) return;
-  set_attr<M_ROWSUM, 0>();
-  set_attr<M_ROWSUM, 1>();
-  set_attr<M_COLSUM, 0>();
-  set_attr<M_COLSUM, 1>();
-  set_attr<M_MAX, 0>();
-  set_attr<M_MAX2, 0>();
-  set_attr<M_KMAX, 0>();
-  set_attr<M_GRAD, 1>();
-  set_attr<M_GRAD, 2>();
-  set_attr<M_GRAD, 3>();
-  set_attr<M_GRAD, 4>();
-  set_attr<M_GRAD, 5>();
-  set_attr<M_GRAD, 6>();
-  set_attr<M_GRAD, 7>();
-  set_attr<M_GRAD, 8>();
-  dot_prepare();
-  done = true;
+// Raise the dynamic shared-memory limits of the sweeps that serve this problem, before any capture.
+// The limits belong to the current device (and end with cudaDeviceReset), so every context sets those
+// of its own kernels: a flag per process left the second device's launches without them.  The packed
+// sweeps (d <= 8) and the stored-cost ones of this file need none.
+cudaError_t prepare_kernels(const Consts& k, int prec) {
+  if (k.kind != COST_SQEUCLID || prec == 1 /* LAMP_PREC_BF16_TC */ || uses_direct_sweeps(k, prec)) return cudaSuccess;
+  if (k.zdot) return dot_prepare();
+  for (const auto set : {set_attr<M_ROWSUM, 0>, set_attr<M_ROWSUM, 1>, set_attr<M_COLSUM, 0>, set_attr<M_COLSUM, 1>,
+                         set_attr<M_MAX, 0>, set_attr<M_MAX2, 0>, set_attr<M_KMAX, 0>, set_attr<M_GRAD, 1>,
+                         set_attr<M_GRAD, 2>, set_attr<M_GRAD, 3>, set_attr<M_GRAD, 4>, set_attr<M_GRAD, 5>,
+                         set_attr<M_GRAD, 6>, set_attr<M_GRAD, 7>, set_attr<M_GRAD, 8>}) {
+    const cudaError_t e = set();
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 int sweep_blocks_per_sm(const Consts& k, int prec, int which) {

@@ -173,7 +173,6 @@ extern "C" int lamp_marginals_noalloc(const lamp_problem* prob, double K, double
   k.W = 5.0 * K;
   k.rnx = 0.0;
 
-  prepare_kernels();
   Geometry g{};
   {
     int sms = 0;
