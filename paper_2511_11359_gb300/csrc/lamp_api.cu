@@ -102,8 +102,10 @@ template <class T>
 static int dalloc(lamp_ctx* ctx, T** p, size_t count) {
   void* q = nullptr;
   cudaError_t e = cudaMalloc(&q, std::max<size_t>(count, 1) * sizeof(T));
-  if (e != cudaSuccess) return fail(ctx, LAMP_E_NOMEM, "cudaMalloc(%zu bytes): %s", count * sizeof(T),
-                                    cudaGetErrorString(e));
+  if (e != cudaSuccess) {
+    (void)cudaGetLastError();  // reported here: the next launch's check must not find it
+    return fail(ctx, LAMP_E_NOMEM, "cudaMalloc(%zu bytes): %s", count * sizeof(T), cudaGetErrorString(e));
+  }
   ctx->allocs.push_back(q);
   *p = reinterpret_cast<T*>(q);
   return LAMP_OK;

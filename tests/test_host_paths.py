@@ -87,3 +87,12 @@ def test_failure_to_raise_a_limit_is_reported(fake, make, kind, d):
     code, h = make(getattr(fake.L, "COST_" + kind), 300, 200, d)
     assert code == fake.L.LAMP_E_CUDA and not h.value
     assert b"fake error" in fake.lamp_last_error(None)
+
+
+def test_a_failed_allocation_is_reported_once(fake, make):
+    code, h = make(fake.L.COST_SQEUCLID, 500, 400, 3)
+    fake.fake_fail_alloc(0)
+    assert code == 0 and fake.lamp_grad(h, BUF, BUF) == fake.L.LAMP_E_NOMEM
+    fake.fake_fail_alloc(-1)
+    assert fake.lamp_iterate(h, 2) == 0, fake.lamp_last_error(h)
+    assert fake.lamp_grad(h, BUF, BUF) == 0
