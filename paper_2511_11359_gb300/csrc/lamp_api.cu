@@ -118,8 +118,11 @@ static int ensure_dot_copies(lamp_ctx* ctx) {
   int rc;
   if (!ctx->w.xt) {
     CK(dot_prepare());  // a tensor-core context's first transport map
-    if ((rc = dalloc(ctx, &ctx->w.xt, (size_t)dot_pad(k.n) * k.d))) return rc;
-    if ((rc = dalloc(ctx, &ctx->w.yt, (size_t)dot_pad(k.m) * k.d))) return rc;
+    // both in one allocation: a failure leaves neither
+    float* t = nullptr;
+    if ((rc = dalloc(ctx, &t, (size_t)(dot_pad(k.n) + dot_pad(k.m)) * k.d))) return rc;
+    ctx->w.xt = t;
+    ctx->w.yt = t + (size_t)dot_pad(k.n) * k.d;
     ctx->dot_fresh = false;
   }
   if (!ctx->dot_fresh) {
@@ -802,22 +805,25 @@ static int end_passes(lamp_ctx* ctx) {
 }
 
 // widen rowpart / colpart to `width` values per point (per split); the captured graphs hold
-// the old pointers, so they are dropped and rebuilt on their next use
+// the old pointers, so they are dropped and rebuilt on their next use.  The new buffers (one
+// allocation) come first: without memory for them the context keeps the old ones
 static int ensure_part_width(lamp_ctx* ctx, int width) {
   if (width <= ctx->part_width) return LAMP_OK;
   CK(cudaStreamSynchronize(ctx->stream));
-  // the first ones are part of the context's one allocation
-  for (double* old : {ctx->w.rowpart, ctx->w.colpart}) {
-    auto it = std::find(ctx->allocs.begin(), ctx->allocs.end(), (void*)old);
-    if (it == ctx->allocs.end()) continue;
+  const size_t rows = (size_t)ctx->g.rows_split * width * ctx->k.n;
+  double* p = nullptr;
+  int rc = dalloc(ctx, &p, rows + (size_t)ctx->g.cols_split * width * ctx->k.m);
+  if (rc) return rc;
+  // the first buffers are part of the context's one allocation, later ones begin with rowpart
+  auto it = std::find(ctx->allocs.begin(), ctx->allocs.end(), (void*)ctx->w.rowpart);
+  if (it != ctx->allocs.end()) {
+    cudaFree(*it);
     ctx->allocs.erase(it);
-    cudaFree(old);
   }
   if (ctx->gexec) cudaGraphExecDestroy(ctx->gexec);
   ctx->gexec = nullptr;
-  int rc = dalloc(ctx, &ctx->w.rowpart, (size_t)ctx->g.rows_split * width * ctx->k.n);
-  if (!rc) rc = dalloc(ctx, &ctx->w.colpart, (size_t)ctx->g.cols_split * width * ctx->k.m);
-  if (rc) return rc;
+  ctx->w.rowpart = p;
+  ctx->w.colpart = p + rows;
   ctx->part_width = width;
   return LAMP_OK;
 }
@@ -974,22 +980,23 @@ static int grad_tc(lamp_ctx* ctx, float* dx, float* dy) {
   int rc;
   if (!ctx->xT) {
     CK(tcg_prepare());
-    if ((rc = dalloc(ctx, reinterpret_cast<uint16_t**>(&ctx->xT), (size_t)n_pad * 64))) return rc;
-    if ((rc = dalloc(ctx, reinterpret_cast<uint16_t**>(&ctx->yT), (size_t)m_pad * 64))) return rc;
-    CK(tc_make_map2(ctx->map_xT, ctx->xT, n_pad, 64, 64, 64));
-    CK(tc_make_map2(ctx->map_yT, ctx->yT, m_pad, 64, 64, 64));
+    // both in one allocation, and kept once their maps are made: a failure leaves neither
+    uint16_t* t = nullptr;
+    if ((rc = dalloc(ctx, &t, (size_t)(n_pad + m_pad) * 64))) return rc;
+    uint16_t* ty = t + (size_t)n_pad * 64;
+    CK(tc_make_map2(ctx->map_xT, t, n_pad, 64, 64, 64));
+    CK(tc_make_map2(ctx->map_yT, ty, m_pad, 64, 64, 64));
+    ctx->xT = t;
+    ctx->yT = ty;
     ctx->tcg_fresh = false;
   }
   // the two sides run concurrently (dx on the context's stream, dy on a side stream), each
   // with partials of its own: one side's tail overlaps the other side's start
   const size_t need_x = (size_t)sx * k.n * 64, need_y = (size_t)sy * k.m * 64;
   const size_t need = need_x + need_y;
-  if (!ctx->gside) {
-    if (cudaStreamCreateWithFlags(&ctx->gside, cudaStreamNonBlocking) != cudaSuccess ||
-        cudaEventCreateWithFlags(&ctx->gfork, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&ctx->gjoin, cudaEventDisableTiming) != cudaSuccess)
-      return fail(ctx, LAMP_E_CUDA, "lamp_grad: stream / event creation failed");
-  }
+  if (!ctx->gside) CK(cudaStreamCreateWithFlags(&ctx->gside, cudaStreamNonBlocking));
+  if (!ctx->gfork) CK(cudaEventCreateWithFlags(&ctx->gfork, cudaEventDisableTiming));
+  if (!ctx->gjoin) CK(cudaEventCreateWithFlags(&ctx->gjoin, cudaEventDisableTiming));
   if (need > ctx->tcg_part_floats) {
     if (ctx->tcg_part) {
       CK(cudaStreamSynchronize(ctx->stream));

@@ -96,3 +96,31 @@ def test_a_failed_allocation_is_reported_once(fake, make):
     fake.fake_fail_alloc(-1)
     assert fake.lamp_iterate(h, 2) == 0, fake.lamp_last_error(h)
     assert fake.lamp_grad(h, BUF, BUF) == 0
+
+
+@pytest.mark.parametrize("kind,d,prec,call,watch,after", [
+    # a tensor-core context's transposed points for the transport map, and those of its gradient
+    ("SQEUCLID", 64, 1, "map", ("k_transpose_points", 3), 0), ("SQEUCLID", 64, 1, "map", ("k_transpose_points", 3), 1),
+    ("SQEUCLID", 64, 1, "grad", ("k_transpose_bf16", 2), 0), ("SQEUCLID", 64, 1, "grad", ("k_transpose_bf16", 2), 1),
+    # l1 with d > 8: wider partial sums, which the iteration's sweeps write too
+    ("L1", 20, 0, "map", ("k_pts_sweep", 6), 0)])
+def test_context_survives_a_failed_allocation(fake, make, kind, d, prec, call, watch, after):
+    """LAMP_E_NOMEM leaves the context as it was: no later launch gets memory that was released or
+    never allocated, and the call works once there is memory."""
+    code, h = make(getattr(fake.L, "COST_" + kind), 500, 400, d, prec)
+    assert code == 0
+    if call == "map" and kind == "L1":
+        assert fake.lamp_apply_map(h, BUF, 4, BUF, 0) == 0  # widened once already
+
+    def run():
+        return fake.lamp_grad(h, BUF, BUF) if call == "grad" else fake.lamp_apply_map(h, BUF, 8, BUF, 0)
+
+    fake.fake_watch(watch[0].encode(), watch[1])
+    before = fake.fake_bytes()
+    fake.fake_fail_alloc(after)
+    code = run()
+    fake.fake_fail_alloc(-1)
+    assert code == fake.L.LAMP_E_NOMEM
+    assert fake.lamp_iterate(h, 2) == 0 and fake.fake_bad() == 0
+    assert run() == 0 and fake.lamp_iterate(h, 2) == 0, fake.lamp_last_error(h)
+    assert fake.fake_bad() == 0 and fake.fake_bytes() >= before
