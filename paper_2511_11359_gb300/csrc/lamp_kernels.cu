@@ -37,17 +37,19 @@ __device__ __forceinline__ float warp_min_f(float v) {
 
 // stage a tile of 128 points (rows base.., np valid) x d coordinates into s[kk * 128 + p]:
 // thread (p = idx % 128, coordinate quad) reads up to 4 consecutive coordinates of one
-// point (one 16-byte load when d % 4 == 0) and consecutive threads write consecutive p,
-// so the transposed shared stores are free of bank conflicts
+// point (one 16-byte load when d % 4 == 0 and the points are 16-byte aligned, which a caller's
+// need not be) and consecutive threads write consecutive p, so the transposed shared stores are
+// free of bank conflicts
 __device__ __forceinline__ void stage_points(float* __restrict__ s, const float* __restrict__ P, int64_t base,
                                              int64_t np, int d, int tid, int nthreads) {
   const int dq = (d + 3) >> 2;
+  const bool vec = (d & 3) == 0 && (reinterpret_cast<uintptr_t>(P) & 15) == 0;
   for (int idx = tid; idx < 128 * dq; idx += nthreads) {
     const int p = idx & 127, kq = (idx >> 7) << 2;
     const int64_t g = base + p;
     float v[4] = {0.f, 0.f, 0.f, 0.f};
     if (g < np) {
-      if ((d & 3) == 0) {
+      if (vec) {
         const float4 t = *reinterpret_cast<const float4*>(P + g * d + kq);
         v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
       } else {
