@@ -90,6 +90,26 @@ def ncu_traffic(workload, prec, n, d, which):
     return rec[which] if sources_digest(rec["sources"]) == rec["sha256"] else None
 
 
+def iteration_kernels(solver, iters: int, span_ms):
+    """Mean device milliseconds of the kernels that solver.iterate(1) runs, by name, and their number
+    per iteration: the four kernels of an iteration, or the one launch of a problem whose iterations
+    run on chip (Lamp.on_chip; lamp_time_kernels would time four kernels that iterate() does not
+    launch).  span_ms(f): device milliseconds of f()."""
+    if solver.on_chip():
+        return {"on_chip_iteration": span_ms(lambda: solver.iterate(10 * iters)) / (10 * iters)}, 1
+    return dict(zip(("row_sweep", "row_fin", "col_sweep", "col_fin"), solver.time_kernels(iters))), \
+        solver.launches_per_iteration()
+
+
+def dominant_sweep(kern: dict):
+    """(name, milliseconds, description) of the sweep that the roofline is taken on: the longer of the
+    two; on chip the average of the two with their finalizes, half an iteration."""
+    if "on_chip_iteration" in kern:
+        return None, kern["on_chip_iteration"] / 2, "average (finalizes included, on chip)"
+    name = "row_sweep" if kern["row_sweep"] >= kern["col_sweep"] else "col_sweep"
+    return name, kern[name], "row" if name == "row_sweep" else "column"
+
+
 def load_peaks():
     p = os.path.join(ROOT, "MEASURED_PEAKS.json")
     if os.path.exists(p):
@@ -401,7 +421,6 @@ def run_gpu(args, rank, world):
         flops_per_entry = 2 * w.d
         bytes_per_entry = 0
     stream = torch.cuda.current_stream()
-    launches = solver.launches_per_iteration()
 
     # L2 flush buffer (larger than the 129 MB L2), written between timed steps
     flush = torch.empty(256 * 1024 * 1024 // 4, dtype=torch.float32, device=devc)
@@ -428,7 +447,15 @@ def run_gpu(args, rank, world):
         dist.barrier()
     total_ms = sum(a.elapsed_time(b) for a, b in evs)
     # per-kernel device times, measured with events between the launches
-    kern_ms = solver.time_kernels(max(3, min(args.steps, 10)))
+    def span_ms(f):
+        e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        e0.record(stream)
+        f()
+        e1.record(stream)
+        torch.cuda.synchronize()
+        return e0.elapsed_time(e1)
+
+    kern_ms, launches = iteration_kernels(solver, max(3, min(args.steps, 10)), span_ms)
     value, total_s = job_throughput(n * m * args.steps, total_ms / 1e3, dist, devc)
     total_ms = total_s * 1e3
 
@@ -576,25 +603,24 @@ def run_gpu(args, rank, world):
             dist.destroy_process_group()
         return
     peaks, src = load_peaks()
-    dom = 0 if kern_ms[0] >= kern_ms[2] else 2
+    dom, dom_ms, dom_what = dominant_sweep(kern_ms)
     mhz = float(peaks.get("sm_max_mhz", 2070.0))
     sms = torch.cuda.get_device_properties(local).multi_processor_count
     if bytes_per_entry:
-        achieved = n * m * bytes_per_entry / (kern_ms[dom] / 1e3) / 1e9
+        achieved = n * m * bytes_per_entry / (dom_ms / 1e3) / 1e9
         roof = {"bound": "hbm", "achieved": achieved, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                 "frac": achieved / peaks["hbm_gbs"],
-                "traffic": ncu_traffic(args.workload, args.prec, n, w.d, "row_sweep" if dom == 0 else "col_sweep"),
+                "traffic": ncu_traffic(args.workload, args.prec, n, w.d, dom),
                 "traffic_unit": "bytes per launch (ncu dram read + write)",
-                "what": "stored C bytes of the " + ("row" if dom == 0 else "column") + " sweep"}
+                "what": f"stored C bytes of the {dom_what} sweep"}
     elif args.prec == "bf16_tc" or w.d <= 8:
         # tensor-core sweeps, and the packed f32x2 direct-form sweeps (d <= 8): two ex2 per entry
         rate = L.measure_ex2_rate()
         peak = sms * rate * mhz * 1e6 / 1e12
-        achieved = n * m * 2 / (kern_ms[dom] / 1e3) / 1e12
+        achieved = n * m * 2 / (dom_ms / 1e3) / 1e12
         form = "tcgen05 x.y" if args.prec == "bf16_tc" else "f32x2 direct |x - y|^2"
         mufu = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "Tex2/s", "frac": achieved / peak,
-                "what": "MUFU ex2 of the " + ("row" if dom == 0 else "column") + f" sweep ({form}; 2 ex2 per entry: "
-                        "streams A, B)",
+                "what": f"MUFU ex2 of the {dom_what} sweep ({form}; 2 ex2 per entry: streams A, B)",
                 "peak_source": f"{sms} SMs x {rate:.2f} ex2/clk/SM (measured, lamp_measure_ex2_rate) x {mhz:.0f} MHz"}
         if args.prec == "bf16_tc":
             # MUFU binds: 16 entries / clk / SM, against ~21 for the FP32 pipe at 6 lane-ops per entry
@@ -606,21 +632,19 @@ def run_gpu(args, rank, world):
             # that is 13 lane-ops, 9.8 entries / clk / SM, against 16 for MUFU
             lanes = 2 * w.d + 7
             fpeak = sms * 128 * mhz * 1e6 / 1e12
-            fach = n * m * lanes / (kern_ms[dom] / 1e3) / 1e12
+            fach = n * m * lanes / (dom_ms / 1e3) / 1e12
             roof = {"bound": "alu", "achieved": fach, "peak": fpeak, "unit": "Tlane-op/s", "frac": fach / fpeak,
-                    "what": "FP32-pipe lane operations of the " + ("row" if dom == 0 else "column") +
-                            f" sweep ({form}; {lanes} lane-ops per entry)",
+                    "what": f"FP32-pipe lane operations of the {dom_what} sweep ({form}; {lanes} lane-ops per entry)",
                     "peak_source": f"{sms} SMs x 128 FP32 lanes x {mhz:.0f} MHz", "mufu": mufu}
-        roof["traffic"] = ncu_traffic(args.workload, args.prec, n, w.d, "row_sweep" if dom == 0 else "col_sweep")
+        roof["traffic"] = ncu_traffic(args.workload, args.prec, n, w.d, dom)
         roof["traffic_unit"] = "bytes per launch (ncu dram read + write)"
     else:
         peak = sms * 128 * 2 * mhz * 1e6 / 1e12  # FP32 FMA lanes x 2 flop x max SM clock
-        achieved = n * m * flops_per_entry / (kern_ms[dom] / 1e3) / 1e12
+        achieved = n * m * flops_per_entry / (dom_ms / 1e3) / 1e12
         roof = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
-                "traffic": None, "what": "fp32 x.y FMA of the " + ("row" if dom == 0 else "column") + " sweep",
+                "traffic": None, "what": f"fp32 x.y FMA of the {dom_what} sweep",
                 "peak_source": f"{sms} SMs x 128 FP32 lanes x 2 flop x {mhz:.0f} MHz"}
-    roof["kernel_ms"] = {"row_sweep": kern_ms[0], "row_fin": kern_ms[1], "col_sweep": kern_ms[2],
-                         "col_fin": kern_ms[3]}
+    roof["kernel_ms"] = kern_ms
     roof["peak_of"] = src
     if not bytes_per_entry and (args.prec == "bf16_tc" or w.d <= 8):
         # the whole iteration against the MUFU rate, counting 2 ex2 per entry per iteration

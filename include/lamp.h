@@ -304,9 +304,15 @@ LAMP_API int lamp_measure_ex2_rate(double* ex2_per_clk_per_sm);
 LAMP_API int lamp_selftest_wait_timeout(int64_t polls, int* status);
 
 /* Number of kernel launches one iteration issues when its kernels are launched one by one
- * (lamp_time_kernels; for launch accounting).  lamp_iterate and lamp_solve launch the same kernels
- * from graphs, and run small point clouds (d <= 8, n and m <= 1024) several iterations to a launch. */
+ * (lamp_time_kernels; for launch accounting).  lamp_iterate and lamp_solve launch the same kernels,
+ * ten iterations to a graph, unless the context runs on chip (lamp_on_chip). */
 LAMP_API int64_t lamp_launches_per_iteration(const lamp_ctx* ctx);
+
+/* 1 if lamp_iterate and lamp_solve run whole iterations of this context in one launch (all those of a
+ * lamp_iterate call, check_every of them in lamp_solve), else 0.  The served problems: point clouds
+ * with d <= 8 in LAMP_PREC_FP32, n and m <= 1024 and n m (2 d + 7) <= 1.1e7, where the device can
+ * schedule a cluster of 16 thread blocks. */
+LAMP_API int lamp_on_chip(const lamp_ctx* ctx);
 
 LAMP_API const char* lamp_last_error(const lamp_ctx* ctx);
 

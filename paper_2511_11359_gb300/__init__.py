@@ -60,7 +60,7 @@ EXPORTED_SYMBOLS = [
     "lamp_get_state", "lamp_set_state", "lamp_step_host", "lamp_create_owned",
     "lamp_launches_per_iteration", "lamp_last_error", "lamp_destroy", "lamp_time_kernels",
     "lamp_marginals_noalloc", "lamp_measure_ex2_rate", "lamp_round", "lamp_dual", "lamp_selftest_wait_timeout",
-    "lamp_apply_map",
+    "lamp_apply_map", "lamp_on_chip",
 ]
 
 library_path = Path(__file__).resolve().parent / "liblamp.so"
@@ -121,6 +121,7 @@ def _load():
     L.lamp_time_kernels.argtypes = [vp, i64, ctypes.POINTER(dbl)]
     L.lamp_launches_per_iteration.argtypes = [vp]
     L.lamp_launches_per_iteration.restype = i64
+    L.lamp_on_chip.argtypes = [vp]
     L.lamp_last_error.argtypes = [vp]
     L.lamp_last_error.restype = ctypes.c_char_p
     L.lamp_destroy.argtypes = [vp]
@@ -355,6 +356,10 @@ class Lamp:
 
     def launches_per_iteration(self) -> int:
         return int(_get_lib().lamp_launches_per_iteration(self._h))
+
+    def on_chip(self) -> bool:
+        """Whether iterate() and solve() run whole iterations in one launch (lamp_on_chip)."""
+        return bool(_get_lib().lamp_on_chip(self._h))
 
 
 class LampHost:

@@ -1217,6 +1217,8 @@ extern "C" int64_t lamp_launches_per_iteration(const lamp_ctx* ctx) {
   return launches_per_iteration(ctx->k, ctx->prec);
 }
 
+extern "C" int lamp_on_chip(const lamp_ctx* ctx) { return ctx && ctx->on_chip ? 1 : 0; }
+
 extern "C" int lamp_selftest_wait_timeout(int64_t polls, int* status) {
   if (!status || polls < 1 || polls > (int64_t)1 << 30)
     return fail(nullptr, LAMP_E_INVALID, "lamp_selftest_wait_timeout: status must be non-NULL, 1 <= polls <= 2^30");
