@@ -14,7 +14,9 @@
 //   cluster barrier; every CTA adds the 16 partials and takes the same decision.
 // The arithmetic is that of the four kernels (lamp_direct.cuh, lamp_fin.cuh): a thread evaluates
 // one row (column) over a group of 64 points, the group sums are folded per split and the splits
-// added in the same order, so the results are the same to the bit.
+// added in the same order, so the states are the same to the bit.  The residual is not: it is added
+// per 1 / 16 of the columns here and per 64 columns there, so its last bits differ, and a tolerance
+// that lies between the two values stops one iteration apart.
 // n = m = 256, d = 2: 16.9 (graphs of the four kernels) -> 7.7 us per iteration: 2.1 us of sums, 3.9
 // of finalize chains, 1.7 of exchanges.
 #include <cmath>
@@ -164,6 +166,7 @@ k_cluster_iterate(const Inputs in, const Work w, const Shape s, int64_t passes, 
   const uint32_t rank = cluster_rank();
   const int r0 = (int)rank * s.own_rows, c0 = (int)rank * s.own_cols;
   const int cur0 = dev->cur;
+  const int status0 = dev->status;  // of an earlier call: the first decision is then to stop, as in k_col_fin
   const double tol = dev->tol;
   const long long tmax = dev->tmax;
   long long t = dev->t;
@@ -298,7 +301,7 @@ k_cluster_iterate(const Inputs in, const Work w, const Shape s, int64_t passes, 
       R = v;
       if (lane == 0) {
         const bool rule = t >= 1 && v <= tol && (k.eta == 0.0 || k.infeas_only || 1.0 - kap * k.eta <= tol);
-        verdict = !isfinite(v) ? 5 : rule || t >= tmax ? 1 : 0;
+        verdict = !isfinite(v) ? 5 : status0 != 0 || rule || t >= tmax ? 1 : 0;
       }
     }
     __syncthreads();
