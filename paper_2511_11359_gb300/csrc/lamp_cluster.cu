@@ -155,7 +155,8 @@ k_cluster_iterate(const Inputs in, const Work w, const Shape s, int64_t passes, 
   __shared__ float xs[kMaxOwn * D], ys[kMaxOwn * D];                  // own points
   __shared__ float roff[kMaxOwn], coff[kMaxOwn], cw[kMaxOwn], cdB[kMaxOwn];  // -RqA; -BqA, wA, dB
   __shared__ float4 rstage[kMaxOwn], cstage[kMaxOwn];                 // pair data of the own rows, columns
-  __shared__ double res[2][kCtas];                                    // residual partials of all CTAs, by parity
+  // residual partials of all CTAs, by parity of the iteration; the sign bit: a row sum out of range
+  __shared__ double res[2][kCtas];
   __shared__ double snu[kMaxOwn], sq[kMaxOwn], srp[kMaxOwn];
   __shared__ LogEntry stab[128];
   __shared__ SweepParams sp[3];                                       // of kappa_t, kappa_{t+1}, kappa_{t+2}
@@ -285,7 +286,7 @@ k_cluster_iterate(const Inputs in, const Work w, const Shape s, int64_t passes, 
         fc[6] = exp2f((float)(quantize_add(bBn, sp[1].g) - bBn));
       } else if (wid == 2) {
         const double rp = warp_sum_d(srp[lane] + srp[lane + 32]);
-        if (lane < kCtas) peer_store_d(peer(&res[par][rank], (uint32_t)lane), bad ? NAN : rp);
+        if (lane < kCtas) peer_store_d(peer(&res[par][rank], (uint32_t)lane), bad ? -rp : rp);
       }
       fin_bar();
       if (cok && role == 1) fc[4] = (float)(sq[p] - bBn);
@@ -295,13 +296,15 @@ k_cluster_iterate(const Inputs in, const Work w, const Shape s, int64_t passes, 
     cluster_sync();
     // ---- the decision, the same in every CTA: one warp's work, float64 is slow on this part ----
     if (wid == 0) {
-      double v = res[par][lane & (kCtas - 1)];
+      const double part = res[par][lane & (kCtas - 1)];
+      const bool range = __any_sync(0xffffffffu, signbit(part));
+      double v = fabs(part);
 #pragma unroll
       for (int o = kCtas / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
       R = v;
       if (lane == 0) {
         const bool rule = t >= 1 && v <= tol && (k.eta == 0.0 || k.infeas_only || 1.0 - kap * k.eta <= tol);
-        verdict = !isfinite(v) ? 5 : status0 != 0 || rule || t >= tmax ? 1 : 0;
+        verdict = range || !isfinite(v) ? 5 : status0 != 0 || rule || t >= tmax ? 1 : 0;
       }
     }
     __syncthreads();

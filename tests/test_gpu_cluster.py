@@ -1,5 +1,7 @@
 """Small point clouds run whole iterations in one launch of a cluster of 16 blocks (lamp_cluster.cu):
 which problems do, and that the launch takes the decisions of the four-kernel iteration."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -63,6 +65,24 @@ def test_an_earlier_numeric_failure_stops_the_iterations(n, chip):
     h.step(2, nu_out=again)
     assert not np.array_equal(again, nu)
     h.close()
+
+
+@pytest.mark.parametrize("n,chip", [(200, True), (1100, False)])
+def test_row_sums_out_of_range(n, chip):
+    """Row shifts far off leave row sums below the representable range: LAMP_E_NUMERIC, the state
+    stays, and the reported infeasibility is that of the column sums (about 0 against c)."""
+    import paper_2511_11359_gb300 as L
+
+    s = solver(n, n, 2, tol=1e-9, max_iter=50)
+    assert s.on_chip() == chip
+    s.iterate(5)
+    st = s.get_state()
+    s.set_state(st["nu"], st["theta"], st["kappa"], st["t"], st["row_shifts"] + np.float32(300.0))
+    out = L._Result()
+    assert L.lib.lamp_solve(s._h, ctypes.byref(out)) == L.LAMP_E_NUMERIC
+    assert out.status == L.LAMP_E_NUMERIC and out.iters == 5 and abs(out.infeas - 1.0) <= 1e-6
+    assert np.array_equal(s.get_state()["nu"], st["nu"])
+    s.close()
 
 
 def test_stops_inside_a_launch():
