@@ -11,11 +11,13 @@
 // Layout as in the iteration's sweeps (lamp_direct.cu): a thread owns R outer points, the inner
 // points stream through shared memory in tiles of 128 (cp.async, double-buffered) and every
 // thread reads the same pair of them, so that one f32x2 instruction serves two entries and
-// nothing is reduced across threads.  Bound by the FMA pipe: 2 d + 4 + NV lane operations and one
-// ex2 per entry (weighted sums), 2 d + 1 (maxima).  A block of 8 x 8 entries per thread with
-// float64 accumulators per tile took 2.78 ms for n = 65536, m = 16384, d = 3, three columns (the
-// float64 additions, at 1/64 of the float32 rate, bound it), after an evaluation pass of 1.06 ms;
-// the whole call, with the row sums in the same pass and no evaluation: 3.93 -> 0.60 ms.
+// nothing is reduced across threads.  Bound by the FMA pipe: 2 d + 4 + 3 NV lane operations (2 NV of
+// them the folds of the values' sums) and one ex2 per entry (weighted sums), 2 d + 1 (maxima).  A
+// block of 8 x 8 entries per thread with float64 accumulators per tile took 2.78 ms for n = 65536,
+// m = 16384, d = 3, three columns (the float64 additions, at 1/64 of the float32 rate, bound it),
+// after an evaluation pass of 1.06 ms; the whole call, with the row sums in the same pass and no
+// evaluation: 3.93 -> 0.65 ms (0.57 ms with folds every 32 pairs, whose sums of 64 float32 terms were
+// up to 8 u off, u = 2^-24, where 8 terms are within 4.5 u).
 #include <cmath>
 #include <cstdint>
 #include <type_traits>
@@ -29,7 +31,8 @@ namespace wsum {
 constexpr int kThreads = 256;
 constexpr int kTile = kDirectTile;   // inner points per tile
 constexpr int kPairs = kTile / 2;
-constexpr int kFold = 32;            // pairs between float-float folds of the packed sums
+constexpr int kFold = 32;            // pairs between float-float folds of the packed sums of weights
+constexpr int kFoldValues = 4;       // ... of the weighted values: 8 float32 terms
 
 __device__ __forceinline__ void cp4(void* dst, const void* src, bool valid) {
   const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
@@ -171,6 +174,23 @@ k_direct_wsum(const Args a, const DevState* __restrict__ dev, const Consts k) {
       hi[r][q] = lo[r][q] = 0.f;
       acc[r][q] = 0ull;
     }
+  // the sums [q0, q1) into their float-float pairs
+  const auto fold = [&](int q0, int q1) {
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+      for (int q = 0; q < NA; ++q) {
+        if (q < q0 || q >= q1) continue;
+        const float2 s = upk(acc[r][q]);
+        ff_add(hi[r][q], lo[r][q], s.x + s.y);
+        acc[r][q] = 0ull;
+      }
+  };
+  // Weighted values go into the float-float pairs after 8 float32 terms: the gradient and the map
+  // take differences of such sums, so their partial sums carry no more rounding than those of
+  // kernels that add 8 terms and go on in float64, and the pairs have 48 bits.  The sums of the
+  // weights alone (row sums) keep the groups of the iteration's sweeps.
+  constexpr int kStep = NV > 0 ? kFoldValues : kFold;
   for (int64_t it = it0; it < it1; ++it) {
     const int buf = (int)((it - it0) & 1);
     if (it + 1 < it1) stage(buf ^ 1, it + 1);
@@ -179,46 +199,42 @@ k_direct_wsum(const Args a, const DevState* __restrict__ dev, const Consts k) {
     __syncthreads();
 #pragma unroll 1
     for (int p0 = 0; p0 < kPairs; p0 += kFold) {
-      // transport map of 65536 x 16384: 605 -> 582 us against an unroll of 2
+#pragma unroll 1
+      for (int p1 = p0; p1 < p0 + kFold; p1 += kStep) {
 #pragma unroll 4
-      for (int p = p0; p < p0 + kFold; ++p) {
-        const float* rp = srec[buf] + p * REC;
-        uint64_t y2[C::DP], v2[C::VP + 1];
+        for (int p = p1; p < p1 + kStep; ++p) {
+          const float* rp = srec[buf] + p * REC;
+          uint64_t y2[C::DP], v2[C::VP + 1];
 #pragma unroll
-        for (int kk = 0; kk < C::DP; kk += 2) {
-          const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(rp + 2 * kk);
-          y2[kk] = t.x;
-          y2[kk + 1] = t.y;
-        }
-        const ulonglong2 dA = *reinterpret_cast<const ulonglong2*>(rp + 2 * C::DP);
+          for (int kk = 0; kk < C::DP; kk += 2) {
+            const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(rp + 2 * kk);
+            y2[kk] = t.x;
+            y2[kk + 1] = t.y;
+          }
+          const ulonglong2 dA = *reinterpret_cast<const ulonglong2*>(rp + 2 * C::DP);
 #pragma unroll
-        for (int q = 0; q < C::VP; q += 2) {
-          const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(rp + 2 * C::DP + 4 + 2 * q);
-          v2[q] = t.x;
-          v2[q + 1] = t.y;
-        }
+          for (int q = 0; q < C::VP; q += 2) {
+            const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(rp + 2 * C::DP + 4 + 2 * q);
+            v2[q] = t.x;
+            v2[q + 1] = t.y;
+          }
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-          const uint64_t z2 = pair_cost<D>(x2[r], y2, op);
-          const uint64_t e2 = BILIN ? z2 : exp2_pair(ah2, al2, z2, f2add(own[r], dA.x));
-          if (NV == 0) {
-            acc[r][0] = f2fma(e2, dA.y, acc[r][0]);
-          } else {
-            const uint64_t p2 = f2mul(e2, dA.y);
+          for (int r = 0; r < R; ++r) {
+            const uint64_t z2 = pair_cost<D>(x2[r], y2, op);
+            const uint64_t e2 = BILIN ? z2 : exp2_pair(ah2, al2, z2, f2add(own[r], dA.x));
+            if (NV == 0) {
+              acc[r][0] = f2fma(e2, dA.y, acc[r][0]);
+            } else {
+              const uint64_t p2 = f2mul(e2, dA.y);
 #pragma unroll
-            for (int q = 0; q < NV; ++q) acc[r][q] = f2fma(p2, COORDS ? y2[q] : v2[q], acc[r][q]);
-            if (SUM) acc[r][NA - 1] = f2add(acc[r][NA - 1], p2);
+              for (int q = 0; q < NV; ++q) acc[r][q] = f2fma(p2, COORDS ? y2[q] : v2[q], acc[r][q]);
+              if (SUM) acc[r][NA - 1] = f2add(acc[r][NA - 1], p2);
+            }
           }
         }
+        fold(0, NV);
       }
-#pragma unroll
-      for (int r = 0; r < R; ++r)
-#pragma unroll
-        for (int q = 0; q < NA; ++q) {
-          const float2 s = upk(acc[r][q]);
-          ff_add(hi[r][q], lo[r][q], s.x + s.y);
-          acc[r][q] = 0ull;
-        }
+      fold(NV, NA);
     }
     __syncthreads();  // every thread is done with srec[buf] before it is refilled
   }
