@@ -203,7 +203,8 @@ LAMP_API int lamp_objective(lamp_ctx* ctx, double out[LAMP_OBJECTIVE_SLOTS]);
  * Point clouds with d <= 8: one recompute sweep of X^t that forms the row sums on the way
  * (side 1: a row-sum sweep and one recompute sweep); it leaves log Z of X^t, not col(X^t).
  * Others: one evaluation pass, then one recompute sweep.  float32 exponents as in the
- * iteration.  The first call, and one with a larger k, may allocate O(k (n + m) splits)
+ * iteration; the sums of the value columns take 8 float32 terms (stored costs: 64) before they go on
+ * as float-float pairs (48 bits) or in float64.  The first call, and one with a larger k, may allocate O(k (n + m) splits)
  * partial sums (LAMP_E_NOMEM if that fails).  Asynchronous on the context's stream, for d > 8
  * and stored costs after the evaluation pass. */
 LAMP_API int lamp_apply_map(lamp_ctx* ctx, const float* V, int64_t k, float* out, int side);
@@ -241,7 +242,8 @@ LAMP_API int lamp_round(lamp_ctx* ctx, double out[4], double* y, double* delta_r
  * dx: device n x d float32, dy: device m x d float32 (either may be NULL).
  * One evaluation pass (skipped when the state's X^t was the last one evaluated, e.g. after
  * lamp_solve or lamp_objective), then per side one recompute pass (X never stored):
- *   LAMP_PREC_FP32: one float32 sweep per side (the first call allocates its partial sums);
+ *   LAMP_PREC_FP32: one float32 sweep per side, 8 float32 terms of a sum at a time as in
+ *   lamp_apply_map (the first call allocates its partial sums);
  *   LAMP_PREC_BF16_TC: one tensor-core pass per side on the bf16-rounded points the
  *   context solves with: S = x.y^T by tcgen05, the coupling's entries formed in the
  *   epilogue and split into two bf16 parts (16 significant bits), sum_j X_ij y_j by a

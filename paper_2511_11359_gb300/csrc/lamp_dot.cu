@@ -27,6 +27,7 @@ constexpr int kOut = 128;     // outer points of an item
 constexpr int kIn = 128;      // inner points of a tile: the unit of the splits and of the float32 sums
 constexpr int kStage = 256;   // inner points of a stage (two tiles)
 constexpr int kThreads = 256;
+constexpr int kGradFold = 8;  // float32 terms of the gradient's and the map's sums between folds
 
 // kRowEval, kColEval: evaluation passes (stream A alone; columns also weighted by the cost)
 enum Mode : int { kRowSum = 0, kColSum = 1, kRowEval = 2, kColEval = 3, kMax = 4, kMax2 = 5, kKmax = 6 };
@@ -386,11 +387,13 @@ k_transpose_points(const float* __restrict__ P, int64_t np, int d, float* __rest
 // coordinates (or value columns) p_b, P_ab = 2^{v_ab} weight_b with stream A's exponent (X never
 // stored).  Two contractions per tile of 128 x 128
 // entries: z = x.y as in the sweeps (8 x 8 block per thread), P to shared memory, then O += P p
-// with all coordinates at once: 0.49 ms a side at n = m = 8192, d = 64 (a pass per 8 coordinates
+// with all coordinates at once: 0.61 ms a side at n = m = 8192, d = 64 (a pass per 8 coordinates
 // computed every exponent and every product x.y d / 8 times, 8 x 0.67 ms a side).  In the second
 // contraction the halves of the CTA take 64 inner points each and thread (og, cg) the outer
-// points 4 og + {0..3}, 64 + 4 og + {0..3} and the CQ coordinates from CQ cg: 64 float32 terms
-// per output, then a fold into a float-float pair; the halves meet in float64.  P is stored
+// points 4 og + {0..3}, 64 + 4 og + {0..3} and the CQ coordinates from CQ cg: 8 float32 terms
+// per output, then a fold into a float-float pair (a fold per 64 terms: 0.49 ms a side, but chains
+// of 64 additions were up to 12 u off, u = 2^-24, and the gradient is a difference of such sums; 8
+// terms are within 4.5 u); the halves meet in float64.  P is stored
 // with its 16-byte chunks permuted by the row (chunk ^ (row / 4) % 8), which keeps both the
 // stores (one row per lane) and the loads (one row per warp) free of bank conflicts.
 
@@ -531,43 +534,46 @@ k_dot_grad(const GradArgs a, const DevState* __restrict__ dev, const Consts k) {
       load_dat(sd, a, it + 1, tid);
     }
     cp_commit();
-    uint64_t acc[4][CQ];
+#pragma unroll 1
+    for (int j0 = 64 * half; j0 < 64 * half + 64; j0 += kGradFold) {
+      uint64_t acc[4][CQ];
 #pragma unroll
-    for (int r = 0; r < 4; ++r)
+      for (int r = 0; r < 4; ++r)
 #pragma unroll
-      for (int q = 0; q < CQ; ++q) acc[r][q] = 0ull;
+        for (int q = 0; q < CQ; ++q) acc[r][q] = 0ull;
 #pragma unroll 2
-    for (int j = 64 * half; j < 64 * half + 64; ++j) {
-      const int sw = (j >> 2) & 7;
-      const ulonglong2* pr = reinterpret_cast<const ulonglong2*>(sP + j * kOut);
-      const ulonglong2 p0 = pr[og ^ sw], p1 = pr[(16 + og) ^ sw];
-      float y[CQ];
+      for (int j = j0; j < j0 + kGradFold; ++j) {
+        const int sw = (j >> 2) & 7;
+        const ulonglong2* pr = reinterpret_cast<const ulonglong2*>(sP + j * kOut);
+        const ulonglong2 p0 = pr[og ^ sw], p1 = pr[(16 + og) ^ sw];
+        float y[CQ];
 #pragma unroll
-      for (int q = 0; q < CQ; q += 2) {
-        const float2 t = *reinterpret_cast<const float2*>(sy + j * 8 * CQ + cg * CQ + q);
-        y[q] = t.x;
-        y[q + 1] = t.y;
-      }
+        for (int q = 0; q < CQ; q += 2) {
+          const float2 t = *reinterpret_cast<const float2*>(sy + j * 8 * CQ + cg * CQ + q);
+          y[q] = t.x;
+          y[q + 1] = t.y;
+        }
 #pragma unroll
-      for (int q = 0; q < CQ; ++q) {
-        const uint64_t yy = pk(y[q], y[q]);
-        acc[0][q] = f2fma(p0.x, yy, acc[0][q]);
-        acc[1][q] = f2fma(p0.y, yy, acc[1][q]);
-        acc[2][q] = f2fma(p1.x, yy, acc[2][q]);
-        acc[3][q] = f2fma(p1.y, yy, acc[3][q]);
+        for (int q = 0; q < CQ; ++q) {
+          const uint64_t yy = pk(y[q], y[q]);
+          acc[0][q] = f2fma(p0.x, yy, acc[0][q]);
+          acc[1][q] = f2fma(p0.y, yy, acc[1][q]);
+          acc[2][q] = f2fma(p1.x, yy, acc[2][q]);
+          acc[3][q] = f2fma(p1.y, yy, acc[3][q]);
+        }
       }
+      // TwoSum per lane (two_sum of the header), errors into the low parts
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int q = 0; q < CQ; ++q) {
+          const uint64_t s = f2add(hi[r][q], acc[r][q]);
+          const uint64_t bb = f2sub(s, hi[r][q]);
+          const uint64_t e = f2add(f2sub(hi[r][q], f2sub(s, bb)), f2sub(acc[r][q], bb));
+          hi[r][q] = s;
+          lo[r][q] = f2add(lo[r][q], e);
+        }
     }
-    // TwoSum per lane (two_sum of the header), errors into the low parts
-#pragma unroll
-    for (int r = 0; r < 4; ++r)
-#pragma unroll
-      for (int q = 0; q < CQ; ++q) {
-        const uint64_t s = f2add(hi[r][q], acc[r][q]);
-        const uint64_t bb = f2sub(s, hi[r][q]);
-        const uint64_t e = f2add(f2sub(hi[r][q], f2sub(s, bb)), f2sub(acc[r][q], bb));
-        hi[r][q] = s;
-        lo[r][q] = f2add(lo[r][q], e);
-      }
     __syncthreads();  // P and the row-major points may be overwritten
   }
   cp_wait<0>();

@@ -26,7 +26,8 @@ def context(x, y, **kw):
     return L.Lamp(dev(r), dev(c), x=dev(x), y=dev(y), **kw)
 
 
-@pytest.mark.parametrize("d,prec,k", [(1, "fp32", 1), (3, "fp32", 3), (3, "fp32", 4), (8, "fp32", 8), (2, "fp32", 6)])
+@pytest.mark.parametrize("d,prec,k", [(1, "fp32", 1), (3, "fp32", 3), (3, "fp32", 4), (8, "fp32", 8), (2, "fp32", 6),
+                                      (12, "fp32", 3), (64, "fp32", 8), (64, "bf16_tc", 4)])
 def test_transport_map(d, prec, k):
     rng = np.random.default_rng(d)
     s = context(rng.random((N, d), dtype=np.float32), rng.random((M, d), dtype=np.float32), prec=prec)
@@ -37,7 +38,7 @@ def test_transport_map(d, prec, k):
     s.close()
 
 
-@pytest.mark.parametrize("d", [1, 2, 3, 4, 5, 8])
+@pytest.mark.parametrize("d", [1, 2, 3, 4, 5, 8, 9, 17, 33, 64])
 def test_gradient(d):
     v, z = np.resize(VALUES, d), np.zeros
     for x, y, which in ((z((N, d), np.float32), np.tile(v, (M, 1)), 0), (np.tile(v, (N, 1)), z((M, d), np.float32), 1)):
