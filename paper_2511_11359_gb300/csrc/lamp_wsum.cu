@@ -190,7 +190,8 @@ k_direct_wsum(const Args a, const DevState* __restrict__ dev, const Consts k) {
   // take differences of such sums, so their partial sums carry no more rounding than those of
   // kernels that add 8 terms and go on in float64, and the pairs have 48 bits.  The sums of the
   // weights alone (row sums) keep the groups of the iteration's sweeps.
-  constexpr int kStep = NV > 0 ? kFoldValues : kFold;
+  // Round's C delta_c (BILIN): 32 terms.
+  constexpr int kGroup = BILIN ? kFold / 2 : kFold, kStep = NV > 0 ? kFoldValues : kGroup;
   for (int64_t it = it0; it < it1; ++it) {
     const int buf = (int)((it - it0) & 1);
     if (it + 1 < it1) stage(buf ^ 1, it + 1);
@@ -198,9 +199,9 @@ k_direct_wsum(const Args a, const DevState* __restrict__ dev, const Consts k) {
     cp_wait<1>();
     __syncthreads();
 #pragma unroll 1
-    for (int p0 = 0; p0 < kPairs; p0 += kFold) {
+    for (int p0 = 0; p0 < kPairs; p0 += kGroup) {
 #pragma unroll 1
-      for (int p1 = p0; p1 < p0 + kFold; p1 += kStep) {
+      for (int p1 = p0; p1 < p0 + kGroup; p1 += kStep) {
 #pragma unroll 4
         for (int p = p1; p < p1 + kStep; ++p) {
           const float* rp = srec[buf] + p * REC;

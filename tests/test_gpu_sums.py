@@ -19,11 +19,11 @@ VALUES = np.array([1.8835506439208984, 1.8873310089111328, 1.9065380096435547, 1
 N, M = 512, 1024
 
 
-def context(x, y, **kw):
+def context(x, y, c=None, **kw):
     import paper_2511_11359_gb300 as L
 
-    r, c = (np.full(k, 1.0 / k) for k in (N, M))
-    return L.Lamp(dev(r), dev(c), x=dev(x), y=dev(y), **kw)
+    c = np.full(M, 1.0 / M) if c is None else c
+    return L.Lamp(dev(np.full(N, 1.0 / N)), dev(c), x=dev(x), y=dev(y), **kw)
 
 
 @pytest.mark.parametrize("d,prec,k", [(1, "fp32", 1), (3, "fp32", 3), (3, "fp32", 4), (8, "fp32", 8), (2, "fp32", 6),
@@ -47,3 +47,21 @@ def test_gradient(d):
         want = -2.0 * v.astype(np.float64) / (N if which == 0 else M)
         assert np.abs(g / want - 1.0).max() <= 5.5 * U
         s.close()
+
+
+@pytest.mark.parametrize("cost,d", [("l1", 1), ("linf", 8)])
+def test_round(cost, d):
+    """delta_r^T C delta_c / ||delta_r|| = c ||delta_c|| for a cost of equal entries c, with a power of
+    two as delta_c of half the columns: 32 terms are added in float32, 16 to a lane of a pair, so the
+    error is that of 16 additions (emulated here) and one more."""
+    half = np.where(np.arange(M) < M // 2, 1.5, 0.5) / M
+    for v in VALUES:
+        s = context(np.zeros((N, d), np.float32), np.full((M, d), v, np.float32), half, cost=cost)
+        o = s.round()
+        s.close()
+        assert o["dc_l1"] == 0.25
+        a = np.float32(0.0)
+        for _ in range(16):
+            a += v
+        err = (o["cost"] - o["cost_scaled"]) / (0.25 * float(v)) - 1.0
+        assert abs(err) <= abs(float(a) / (16.0 * float(v)) - 1.0) + 1.0 * U
