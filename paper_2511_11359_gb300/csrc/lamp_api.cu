@@ -196,10 +196,11 @@ static int validate(const lamp_problem* pr, const lamp_params* pa, bool device_p
   return LAMP_OK;
 }
 
-static int choose_split(int64_t tout, int64_t tin, int64_t wave, int64_t min_inner, double per_split = 0.002) {
+static int choose_split(int64_t tout, int64_t tin, int64_t wave, int64_t min_inner, double per_split = 0.002,
+                        int64_t most = 128) {
   int best = 1;
   double best_score = -1.0;
-  int64_t smax = std::min<int64_t>(std::max<int64_t>(tin / std::max<int64_t>(min_inner, 1), 1), 128);
+  int64_t smax = std::min<int64_t>(std::max<int64_t>(tin / std::max<int64_t>(min_inner, 1), 1), most);
   for (int s = 1; s <= smax; ++s) {
     int64_t ctas = tout * s;
     int64_t waves = (ctas + wave - 1) / wave;
@@ -830,11 +831,27 @@ static int ensure_part_width(lamp_ctx* ctx, int width) {
 
 static inline int64_t cdiv64(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
-// inner splits of the dot-form gradient pass: one CTA per SM, and each split writes a partial
-// sum per output (1 % of a wave each)
-static int dot_splits(const lamp_ctx* ctx, bool rows) {
-  const int64_t out = cdiv64(rows ? ctx->k.n : ctx->k.m, dot_tile()), in = cdiv64(rows ? ctx->k.m : ctx->k.n, dot_tile());
-  return choose_split(out, in, ctx->g.sms, 4, 0.01);
+// room for the partial sums of the float32 gradient with d > 8: a value per point, split and
+// coordinate is 8 n d bytes a split (128 MiB at n = 2^18, d = 64).  Within kDotPart bytes the splits
+// are free (the most that fewer than 2^17 points take is 254 MiB); beyond that their number is limited
+// first, then the outer points are taken in parts.  Without memory for that, kDotPartLow do.
+constexpr int64_t kDotPart = int64_t(256) << 20, kDotPartLow = int64_t(32) << 20;
+
+// inner splits of a dot-form pass with dv sums per outer point: one CTA per SM, and each split writes
+// a partial sum per output (1 % of a wave each)
+static int dot_splits(const lamp_ctx* ctx, bool rows, int dv, int64_t room) {
+  const int64_t np = rows ? ctx->k.n : ctx->k.m;
+  const int64_t out = cdiv64(np, dot_tile()), in = cdiv64(rows ? ctx->k.m : ctx->k.n, dot_tile());
+  const int64_t most = std::min<int64_t>(std::max<int64_t>(room / 8 / (np * dv), 1), 128);
+  return choose_split(out, in, ctx->g.sms, 4, 0.01, most);
+}
+
+// outer points per launch: all, or as many whole waves of tiles as fit (what does not fit has one
+// split, see dot_splits; a wave of 152 tiles is 9.5 MiB at d = 64)
+static int64_t dot_points(const lamp_ctx* ctx, bool rows, int dv, int splits, int64_t room) {
+  const int64_t np = rows ? ctx->k.n : ctx->k.m, fit = room / 8 / ((int64_t)splits * dv);
+  const int64_t wave = (int64_t)ctx->g.sms * dot_tile();
+  return np <= fit ? np : fit / wave * wave;
 }
 
 // inner splits of a low-dimensional weighted-sum pass with `sums` sums per point (lamp_wsum.cu)
@@ -881,7 +898,7 @@ extern "C" int lamp_apply_map(lamp_ctx* ctx, const float* V, int64_t k, float* o
   }
   if (ctx->k.zdot) {
     if ((rc = ensure_dot_copies(ctx))) return rc;
-    splits = dot_splits(ctx, side == 0);
+    splits = dot_splits(ctx, side == 0, (int)k, kDotPart);
     rc = ensure_gpart(ctx, (size_t)splits * (side == 0 ? ctx->k.n : ctx->k.m) * k);
   } else {
     rc = ensure_part_width(ctx, (int)k);
@@ -1040,15 +1057,34 @@ static int grad_tc(lamp_ctx* ctx, float* dx, float* dy) {
 // the envelope gradient in float32: one pass per side with all coordinates
 static int grad_fp32(lamp_ctx* ctx, float* dx, float* dy) {
   const Consts& k = ctx->k;
-  const int sx = k.zdot ? dot_splits(ctx, true) : wsum_splits(ctx, true, k.d);
-  const int sy = k.zdot ? dot_splits(ctx, false) : wsum_splits(ctx, false, k.d);
-  int rc = ensure_gpart(ctx, std::max(dx ? (size_t)sx * k.n : 0, dy ? (size_t)sy * k.m : 0) * k.d);
+  int splits[2], rc = LAMP_OK;
+  int64_t points[2];  // outer points per launch
+  for (const int64_t room : {kDotPart, kDotPartLow}) {
+    size_t part = 0;
+    for (int side = 0; side < 2; ++side) {
+      const bool rows = side == 0;
+      splits[side] = k.zdot ? dot_splits(ctx, rows, k.d, room) : wsum_splits(ctx, rows, k.d);
+      points[side] = k.zdot ? dot_points(ctx, rows, k.d, splits[side], room) : rows ? k.n : k.m;
+      if (rows ? dx : dy) part = std::max(part, (size_t)splits[side] * points[side] * k.d);
+    }
+    if ((rc = ensure_gpart(ctx, part)) != LAMP_E_NOMEM || !k.zdot) break;
+  }
   if (rc) return rc;
   if ((rc = evaluate_if_stale(ctx))) return rc;
   const int cur = ctx->host_dev->cur;
-  const auto pass = k.zdot ? dot_grad : direct_grad;
-  if (dx) CK(pass(true, ctx->in, ctx->w, k, cur, sx, ctx->gpart, dx, ctx->stream));
-  if (dy) CK(pass(false, ctx->in, ctx->w, k, cur, sy, ctx->gpart, dy, ctx->stream));
+  for (int side = 0; side < 2; ++side) {
+    const bool rows = side == 0;
+    float* out = rows ? dx : dy;
+    if (!out) continue;
+    if (!k.zdot) {
+      CK(direct_grad(rows, ctx->in, ctx->w, k, cur, splits[side], ctx->gpart, out, ctx->stream));
+      continue;
+    }
+    const int64_t np = rows ? k.n : k.m;
+    for (int64_t i = 0; i < np; i += points[side])
+      CK(dot_grad(rows, ctx->in, ctx->w, k, cur, i, std::min(points[side], np - i), splits[side], ctx->gpart, out,
+                  ctx->stream));
+  }
   return LAMP_OK;
 }
 

@@ -525,10 +525,10 @@ cudaError_t dot_transpose(const float* P, int64_t np, int d, float* out, cudaStr
 cudaError_t dot_prepare();
 int dot_tile();
 cudaError_t dot_launch(int mode, const Work& w, const Consts& k, const Geometry& g, cudaStream_t st);
-cudaError_t dot_weighted(bool rows, const Work& w, const Consts& k, const float* values, int dv, const float4* off,
-                         const float4* dat, int splits, double* part, cudaStream_t st);
-cudaError_t dot_grad(bool rows, const Inputs& in, const Work& w, const Consts& k, int cur, int splits, double* part,
-                     float* out, cudaStream_t st);
+cudaError_t dot_weighted(bool rows, const Work& w, const Consts& k, int64_t first, int64_t count, const float* values,
+                         int dv, const float4* off, const float4* dat, int splits, double* part, cudaStream_t st);
+cudaError_t dot_grad(bool rows, const Inputs& in, const Work& w, const Consts& k, int cur, int64_t first, int64_t count,
+                     int splits, double* part, float* out, cudaStream_t st);
 // weighted sums and maxima over low-dimensional point clouds (lamp_wsum.cu)
 enum DirectMaxMode : int { kDirectMax, kDirectMax2, kDirectKmax };
 int wsum_outer(int d, int sums);

@@ -665,23 +665,24 @@ cudaError_t dot_prepare() {
 
 int dot_tile() { return dot::kOut; }
 
-// one side's sums of P times dv value columns per inner point: part[splits][n_out][dv].
-// off / dat: outer and inner data (n_out and n_in entries)
-cudaError_t dot_weighted(bool rows, const Work& w, const Consts& k, const float* values, int dv, const float4* off,
-                         const float4* dat, int splits, double* part, cudaStream_t st) {
+// one side's sums of P times dv value columns per inner point, of the `count` outer points from
+// `first` (a multiple of 128) on: part[splits][count][dv].  off / dat: outer and inner data (n_out and
+// n_in entries)
+cudaError_t dot_weighted(bool rows, const Work& w, const Consts& k, int64_t first, int64_t count, const float* values,
+                         int dv, const float4* off, const float4* dat, int splits, double* part, cudaStream_t st) {
   dot::GradArgs a{};
-  a.out_t = rows ? w.xt : w.yt;
+  a.out_t = (rows ? w.xt : w.yt) + first;
   a.in_t = rows ? w.yt : w.xt;
   a.in_v = values;
-  a.n_out = rows ? k.n : k.m;
+  a.n_out = count;
   a.n_in = rows ? k.m : k.n;
-  a.ld_out = dot_pad(a.n_out);
+  a.ld_out = dot_pad(rows ? k.n : k.m);
   a.ld_in = dot_pad(a.n_in);
   a.d = k.d;
   a.dv = dv;
   a.ntiles = (int)((a.n_in + dot::kIn - 1) / dot::kIn);
   a.tiles_per_split = (a.ntiles + splits - 1) / splits;
-  a.off = off;
+  a.off = off + first;
   a.dat = dat;
   a.part = part;
   const dim3 grid((unsigned)((a.n_out + dot::kOut - 1) / dot::kOut), (unsigned)splits);
@@ -698,16 +699,17 @@ cudaError_t dot_weighted(bool rows, const Work& w, const Consts& k, const float*
   return cudaGetLastError();
 }
 
-cudaError_t dot_grad(bool rows, const Inputs& in, const Work& w, const Consts& k, int cur, int splits, double* part,
-                     float* out, cudaStream_t st) {
+// the gradient of the `count` outer points from `first` on
+cudaError_t dot_grad(bool rows, const Inputs& in, const Work& w, const Consts& k, int cur, int64_t first, int64_t count,
+                     int splits, double* part, float* out, cudaStream_t st) {
   // rows: weights w_j of the column data, outer offsets RqA; columns: weights q_i, offsets BqA
   const float4* off = rows ? w.g2row : w.colq[cur];
   const float4* dat = rows ? w.colq[cur] : w.g2row;
-  cudaError_t e = dot_weighted(rows, w, k, rows ? in.y : in.x, k.d, off, dat, splits, part, st);
+  cudaError_t e = dot_weighted(rows, w, k, first, count, rows ? in.y : in.x, k.d, off, dat, splits, part, st);
   if (e != cudaSuccess) return e;
-  const int64_t n_out = rows ? k.n : k.m;
-  dot::k_dot_grad_fin<<<(unsigned)((n_out * k.d + 255) / 256), 256, 0, st>>>(
-      part, splits, n_out, k.d, rows ? in.x : in.y, rows ? in.r : w.colA, off, k.s, out);
+  dot::k_dot_grad_fin<<<(unsigned)((count * k.d + 255) / 256), 256, 0, st>>>(
+      part, splits, count, k.d, (rows ? in.x : in.y) + first * k.d, (rows ? in.r : w.colA) + first, off + first, k.s,
+      out + first * k.d);
   return cudaGetLastError();
 }
 

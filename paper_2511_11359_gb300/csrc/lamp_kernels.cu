@@ -1109,7 +1109,7 @@ static cudaError_t launch_map_k(const Inputs& in, const Consts& k, const Work& w
     }
     const float4* outer = side == 0 ? w.g2row : w.colq[cur];
     const int64_t np = side == 0 ? k.n : k.m;
-    cudaError_t e = dot_weighted(side == 0, w, k, V, DK, outer, inner, splits, part, st);
+    cudaError_t e = dot_weighted(side == 0, w, k, 0, np, V, DK, outer, inner, splits, part, st);
     if (e != cudaSuccess) return e;
     k_map_fin<<<(unsigned)cdiv(np, 256), 256, 0, st>>>(part, splits, np, DK, outer, side == 0 ? in.r : nullptr, out);
     return cudaGetLastError();

@@ -3,8 +3,8 @@
 // held against the limits and the allocations that a device would hold it against.
 //   - cudaFuncSetAttribute holds for the current device alone, as the runtime documents it; a launch
 //     with more dynamic shared memory than its kernel's limit there (48 KiB unless raised) fails.
-//   - fake_fail_alloc(i): the allocation after the next i ones fails; fake_fail_attr(1): every
-//     cudaFuncSetAttribute does.
+//   - fake_fail_alloc(i): the allocation after the next i ones fails; fake_limit(b): those that would
+//     take the total above b bytes; fake_fail_attr(1): every cudaFuncSetAttribute.
 //   - fake_watch(name, arg): the pointer argument `arg` of every launch of a kernel whose name
 //     contains `name` has to lie inside a live allocation; fake_bad() counts those that do not.
 #include <cuda.h>
@@ -27,7 +27,7 @@ struct Config {
 };
 
 int g_device = 0, g_fail_attr = 0;
-long long g_fail_alloc = -1;
+long long g_fail_alloc = -1, g_byte_limit = -1;
 long long g_bad = 0, g_launches = 0, g_graph_launches = 0, g_graphs = 0;
 size_t g_bytes = 0, g_peak = 0;
 bool g_capturing = false;
@@ -77,7 +77,7 @@ extern "C" {
 
 void fake_reset() {
   g_device = g_fail_attr = 0;
-  g_fail_alloc = -1;
+  g_fail_alloc = g_byte_limit = -1;
   g_bad = g_launches = g_graph_launches = g_graphs = 0;
   g_peak = g_bytes;
   g_limit.clear();
@@ -85,6 +85,7 @@ void fake_reset() {
 }
 void fake_set_device(int d) { g_device = d; }
 void fake_fail_alloc(long long after) { g_fail_alloc = after; }
+void fake_limit(long long bytes) { g_byte_limit = bytes; }
 void fake_fail_attr(int on) { g_fail_attr = on; }
 void fake_watch(const char* name, int arg) { g_watch.emplace_back(name, arg); }
 long long fake_bad() { return g_bad; }
@@ -159,6 +160,7 @@ const char* cudaGetErrorString(cudaError_t e) { return e == cudaSuccess ? "no er
 // ---- memory ----
 cudaError_t cudaMalloc(void** p, size_t bytes) {
   if (g_fail_alloc >= 0 && g_fail_alloc-- == 0) return note(cudaErrorMemoryAllocation);
+  if (g_byte_limit >= 0 && g_bytes + bytes > (size_t)g_byte_limit) return note(cudaErrorMemoryAllocation);
   *p = std::calloc(1, bytes);
   g_live[(char*)*p] = bytes;
   g_bytes += bytes;

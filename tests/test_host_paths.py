@@ -30,7 +30,7 @@ def fake(tmp_path_factory):
     lib.lamp_apply_map.argtypes = [vp, vp, i64, vp, ctypes.c_int]
     lib.lamp_last_error.argtypes, lib.lamp_last_error.restype = [vp], ctypes.c_char_p
     lib.lamp_destroy.argtypes, lib.lamp_destroy.restype = [vp], None
-    lib.fake_fail_alloc.argtypes = [ctypes.c_longlong]
+    lib.fake_fail_alloc.argtypes = lib.fake_limit.argtypes = [ctypes.c_longlong]
     for f in ("bad", "launches", "graph_launches", "graphs", "bytes", "peak"):
         getattr(lib, "fake_" + f).restype = ctypes.c_longlong
     lib.L = L
@@ -124,3 +124,20 @@ def test_context_survives_a_failed_allocation(fake, make, kind, d, prec, call, w
     assert fake.lamp_iterate(h, 2) == 0 and fake.fake_bad() == 0
     assert run() == 0 and fake.lamp_iterate(h, 2) == 0, fake.lamp_last_error(h)
     assert fake.fake_bad() == 0 and fake.fake_bytes() >= before
+
+
+@pytest.mark.parametrize("n,m,d", [(1 << 18, 1 << 18, 64), (40001, 1 << 18, 33), (1 << 18, 100, 9), (3000, 3001, 64)])
+@pytest.mark.parametrize("room", [256, 33])
+def test_gradient_partials_are_bounded(fake, make, n, m, d, room):
+    """The float32 gradient's partial sums stay within 256 MiB, whatever the number of points, and
+    within 32 MiB where there is no more memory; they are allocated once, and every launch gets its
+    part of them."""
+    code, h = make(fake.L.COST_SQEUCLID, n, m, d)
+    assert code == 0
+    fake.fake_watch(b"k_dot_grad_fin", 0)
+    before = fake.fake_bytes()
+    fake.fake_limit(before + (room << 20))
+    for _ in range(2):
+        assert fake.lamp_grad(h, BUF, BUF) == 0, fake.lamp_last_error(h)
+    assert 0 < fake.fake_bytes() - before <= room << 20
+    assert fake.fake_bad() == 0
