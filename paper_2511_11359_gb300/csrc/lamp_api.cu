@@ -1190,15 +1190,14 @@ extern "C" int lamp_step_host(lamp_ctx* ctx, const float* C_or_x, const float* y
   }
   int rc = lamp_iterate(ctx, iters);
   if (rc) return rc;
-  CK(cudaMemcpyAsync(&ctx->host_dev->res, &ctx->w.dev->res, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
+  // the control block in one copy: the residual, and the buffer parity, which is only known on the
+  // device (its host copy is pageable memory, where each copy waits for the stream)
+  if ((rc = poll(ctx))) return rc;
   if (nu_out) {
-    // the buffer parity is only known on the device; copy both halves' candidate after reading cur
-    CK(cudaMemcpyAsync(&ctx->host_dev->cur, &ctx->w.dev->cur, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
-    CK(cudaStreamSynchronize(ctx->stream));
     CK(cudaMemcpyAsync(nu_out, ctx->w.nu[ctx->host_dev->cur], k.m * sizeof(double), cudaMemcpyDeviceToHost,
                        ctx->stream));
+    CK(cudaStreamSynchronize(ctx->stream));
   }
-  CK(cudaStreamSynchronize(ctx->stream));
   if (infeas_out) *infeas_out = ctx->host_dev->res;
   return LAMP_OK;
 }

@@ -28,7 +28,7 @@ struct Config {
 
 int g_device = 0, g_fail_attr = 0;
 long long g_fail_alloc = -1, g_byte_limit = -1;
-long long g_bad = 0, g_launches = 0, g_graph_launches = 0, g_graphs = 0;
+long long g_bad = 0, g_reads = 0, g_launches = 0, g_graph_launches = 0, g_graphs = 0;
 size_t g_bytes = 0, g_peak = 0;
 bool g_capturing = false;
 std::map<const void*, std::string> g_names;
@@ -78,7 +78,7 @@ extern "C" {
 void fake_reset() {
   g_device = g_fail_attr = 0;
   g_fail_alloc = g_byte_limit = -1;
-  g_bad = g_launches = g_graph_launches = g_graphs = 0;
+  g_bad = g_reads = g_launches = g_graph_launches = g_graphs = 0;
   g_peak = g_bytes;
   g_limit.clear();
   g_watch.clear();
@@ -92,6 +92,8 @@ long long fake_bad() { return g_bad; }
 long long fake_launches() { return g_launches; }
 long long fake_graph_launches() { return g_graph_launches; }
 long long fake_graphs() { return g_graphs; }
+// copies from device to host memory
+long long fake_reads() { return g_reads; }
 long long fake_bytes() { return (long long)g_bytes; }
 long long fake_peak() { return (long long)g_peak; }
 
@@ -180,7 +182,8 @@ cudaError_t cudaHostAlloc(void** p, size_t bytes, unsigned) { return *p = std::c
 cudaError_t cudaMallocHost(void** p, size_t bytes) { return *p = std::calloc(1, bytes), cudaSuccess; }
 cudaError_t cudaFreeHost(void* p) { return std::free(p), cudaSuccess; }
 cudaError_t cudaMemcpy(void* d, const void* s, size_t n, cudaMemcpyKind) { return std::memcpy(d, s, n), cudaSuccess; }
-cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind, cudaStream_t) {
+cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind kind, cudaStream_t) {
+  g_reads += kind == cudaMemcpyDeviceToHost;
   return std::memcpy(d, s, n), cudaSuccess;
 }
 cudaError_t cudaMemcpy2DAsync(void* d, size_t dp, const void* s, size_t sp, size_t w, size_t h, cudaMemcpyKind,

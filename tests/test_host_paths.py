@@ -25,13 +25,15 @@ def fake(tmp_path_factory):
     lib = ctypes.CDLL(str(so))
     vp, i64 = ctypes.c_void_p, ctypes.c_int64
     lib.lamp_create.argtypes = [ctypes.POINTER(vp), vp, vp, vp]
+    lib.lamp_create_owned.argtypes = lib.lamp_create.argtypes
+    lib.lamp_step_host.argtypes = [vp, vp, vp, vp, vp, i64, ctypes.POINTER(ctypes.c_double), vp]
     lib.lamp_iterate.argtypes = [vp, i64]
     lib.lamp_grad.argtypes = [vp, vp, vp]
     lib.lamp_apply_map.argtypes = [vp, vp, i64, vp, ctypes.c_int]
     lib.lamp_last_error.argtypes, lib.lamp_last_error.restype = [vp], ctypes.c_char_p
     lib.lamp_destroy.argtypes, lib.lamp_destroy.restype = [vp], None
     lib.fake_fail_alloc.argtypes = lib.fake_limit.argtypes = [ctypes.c_longlong]
-    for f in ("bad", "launches", "graph_launches", "graphs", "bytes", "peak"):
+    for f in ("bad", "reads", "launches", "graph_launches", "graphs", "bytes", "peak"):
         getattr(lib, "fake_" + f).restype = ctypes.c_longlong
     lib.L = L
     lib.fake_reset()
@@ -141,3 +143,21 @@ def test_gradient_partials_are_bounded(fake, make, n, m, d, room):
         assert fake.lamp_grad(h, BUF, BUF) == 0, fake.lamp_last_error(h)
     assert 0 < fake.fake_bytes() - before <= room << 20
     assert fake.fake_bad() == 0
+
+
+@pytest.mark.parametrize("d,prec", [(2, 0), (64, 0), (64, 1)])
+def test_a_host_step_reads_the_control_block_once(fake, d, prec):
+    """lamp_step_host reads back the control block, in one copy, and nu."""
+    L, n, m = fake.L, 300, 200
+    r, c, x, y, nu = (np.zeros(k) for k in (n, m, n * d, m * d, m))
+    p = L._Problem()
+    p.n, p.m, p.d, p.kind, p.cost_scale = n, m, d, L.COST_SQEUCLID, 1.0
+    p.x, p.y, p.r, p.c = (a.ctypes.data for a in (x, y, r, c))
+    h, inf = ctypes.c_void_p(), ctypes.c_double()
+    fake.fake_reset()
+    assert fake.lamp_create_owned(ctypes.byref(h), ctypes.byref(p), ctypes.byref(L.default_params(prec=prec, K=1.0)), None) == 0
+    for out in (nu.ctypes.data, 0):
+        before = fake.fake_reads()
+        assert fake.lamp_step_host(h, p.x, p.y, p.r, p.c, 1, ctypes.byref(inf), out) == 0
+        assert fake.fake_reads() - before == (2 if out else 1)
+    fake.lamp_destroy(h)
