@@ -1,7 +1,8 @@
 """Build the in-tree CUDA library liblamp.so for sm_103a with nvcc.
 
 Usage: python -m paper_2511_11359_gb300.build   (or build() from Python).
-Translation units are compiled in parallel into _build/, then linked into
+Translation units are compiled in parallel into _build/ (with the registers and spills of
+every kernel, as ptxas reports them, in _build/<unit>.log), then linked into
 paper_2511_11359_gb300/liblamp.so.  Rebuilds only when a source or header is
 newer than the library.
 """
@@ -24,7 +25,7 @@ SOURCES = ["lamp_kernels.cu", "lamp_fin.cu", "lamp_api.cu", "lamp_noalloc.cu", "
            "lamp_eval.cu", "lamp_direct.cu", "lamp_direct_small.cu", "lamp_cluster.cu", "lamp_dot.cu", "lamp_wsum.cu", "lamp_dense.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden",
-         "--expt-relaxed-constexpr"]
+         "--expt-relaxed-constexpr", "-Xptxas", "-v"]
 
 
 def nvcc_path() -> str:
@@ -62,9 +63,10 @@ def build(force: bool = False, verbose: bool = False) -> Path:
     failed = []
     for src, p in procs:
         out, _ = p.communicate()
+        (BUILD / (Path(src).stem + ".log")).write_text(out)
         if p.returncode != 0:
             failed.append((src, out))
-        elif verbose and out.strip():
+        elif verbose and "warning" in out:
             print(out)
     if failed:
         msg = "\n".join(f"--- {s}\n{o}" for s, o in failed)

@@ -114,9 +114,13 @@ k_pts_direct(const float* __restrict__ P_out, const float* __restrict__ P_in, in
     const float* rec = srec[buf];
 #pragma unroll 1
     for (int p0 = 0; p0 < kDPairs; p0 += kDFold) {
-      // unrolled by 8: the FMA pipe waited on the record loads (2^17 points, d = 3: 7.58 / 7.88 ->
-      // 7.31 / 7.50 ms per sweep against 2)
-#pragma unroll 8
+      // unrolled, because the FMA pipe waited on the record loads: by 8, or by 4 where 8 made the
+      // kernel spill (d <= 2) or lengthened it (d = 5).  2^17 points, rows / columns, ms, unrolled by
+      // 2, 4, 8: d = 1 5.64 / 6.07, 5.46 / 5.68, 5.51 / 5.73; d = 3 7.58 / 7.88, 7.36 / 7.58, 7.31 /
+      // 7.50; d = 5 9.39 / 10.14, 9.32 / 9.54, 9.44 / 9.67; d = 8 12.01 / 12.37, 11.83 / 11.99,
+      // 11.81 / 12.12; l1 and l-inf alike
+      constexpr int U = D <= 2 || D == 5 ? 4 : 8;
+#pragma unroll U
       for (int p = p0; p < p0 + kDFold; ++p) {
         DirectPair<D> t;
         t.load(rec + p * REC);
