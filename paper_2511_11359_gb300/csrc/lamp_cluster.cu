@@ -235,7 +235,7 @@ k_cluster_iterate(const Inputs in, const Work w, const Shape s, int64_t passes, 
       if (role == 2) {
         rnext = -(float)quantize_add((double)(-roff[p]) + log2_table(S, stab), sp[1].g);
       } else {
-        const float q = (float)div_seeded(ri, S);
+        const float q = (float)(ri / S);
         if (role == 0) {
           fr[0] = roff[p];
           fr[2] = q;
@@ -261,12 +261,12 @@ k_cluster_iterate(const Inputs in, const Work w, const Shape s, int64_t passes, 
           const double A = __dmul_rn((double)cw[p], a);  // rounded, as the column sum that k_col_fin stores
           srp[p] = fabs(A - cj);
           const double tA = tanh(gj * (A - cj));
-          const double thbar = div_seeded(tA + thj, fma(tA, thj, 1.0));
+          const double thbar = (tA + thj) / fma(tA, thj, 1.0);
           nun = nuj + sp[0].wB * (thbar - nuj);
           snu[p] = nun;
         } else {
           const double tB = tanh(gj * (a - cj));
-          const double thhat = div_seeded(tB + thj, fma(tB, thj, 1.0));
+          const double thhat = (tB + thj) / fma(tB, thj, 1.0);
           thn = fmin(fmax(thhat, -k.clipb), k.clipb);
         }
       } else if (tid == 3 * 32) {

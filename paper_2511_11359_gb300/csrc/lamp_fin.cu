@@ -12,11 +12,12 @@
 // float64 instructions of the longest warp, plus the latency of its loads and of the last
 // block's tail.  Hence: the two streams of a point are worked by two warps on different
 // schedulers, what only an evaluation pass reports is computed there alone, the mirror step's
-// gain is kept per column, divisions start from a float32 reciprocal, the row shift's log2
-// comes from a table, and the parameters of the next iteration are prepared by a block of RF
-// instead of by CF's last thread.  RF + CF together, against one thread per point doing all of
-// it in blocks of 128: 22.9 -> 12.0 us at 4096 points (16 splits), 37.5 -> 23.1 us at 2^15 (19
-// splits).
+// gain is kept per column, the row shift's log2 comes from a table, and the parameters of the
+// next iteration are prepared by a block of RF instead of by CF's last thread.  RF + CF together,
+// against one thread per point doing all of it in blocks of 128: 22.9 -> 12.0 us at 4096 points
+// (16 splits), 37.5 -> 23.1 us at 2^15 (19 splits).  Divisions stay the correctly rounded ones: a
+// quotient from a float32 seed and one Newton step takes 4 operations less, 0.1 to 0.2 us an
+// iteration, but rounds the other way next to a tie.
 #include <cmath>
 
 #include "lamp_fin.cuh"
@@ -81,7 +82,7 @@ k_row_fin(const Work w, int splits, const double* __restrict__ r, int rowblocks,
     // by ~1e-6 instead of ~1e-8, and log Z, which amplifies nu by 2 K kappa, by ~1e-4
     if (role == 0) {
       // the row weight q = r / S, a float32 factor of the column sweep
-      const float q = (float)div_seeded(ri, S);
+      const float q = (float)(ri / S);
       reinterpret_cast<float2*>(w.g2row + i)[0] = make_float2(rq.x, q);
       if (w.g2row2) {
         store_pair_field(w.g2row2, i, 0, -rq.x);
@@ -95,7 +96,7 @@ k_row_fin(const Work w, int splits, const double* __restrict__ r, int rowblocks,
       w.logZ[i] = lz;
       contrib = ri * lz;
     } else {
-      const float q = (float)div_seeded(ri, S);
+      const float q = (float)(ri / S);
       reinterpret_cast<float2*>(w.g2row + i)[1] = make_float2(rq.y, q);
       if (w.g2row2) {
         store_pair_field(w.g2row2, i, 2, k.shared_shift ? 0.f : -rq.y);
@@ -181,7 +182,7 @@ k_col_fin(const Work w, int splits, const double* __restrict__ cvec, int rowbloc
         // (1 + theta tanh u): one tanh per stream and no atanh (|theta^t| <= tanh(beta/2) < 1,
         // so the denominator is at least 1 - tanh(beta/2))
         const double tA = tanh(gj * (A - cj));
-        const double thbar = div_seeded(tA + thj, fma(tA, thj, 1.0));  // M_{tau2}(theta^t; p^{eta_t}(nu^t))
+        const double thbar = (tA + thj) / fma(tA, thj, 1.0);  // M_{tau2}(theta^t; p^{eta_t}(nu^t))
         nun = nuj + sp.wB * (thbar - nuj);                             // nu^{t+1}
         snu[p] = nun;
         w.nu[cur ^ 1][j] = nun;
@@ -191,7 +192,7 @@ k_col_fin(const Work w, int splits, const double* __restrict__ cvec, int rowbloc
       // already inside the sweep's exponents
       const double B = k.shared_shift ? a : (double)cq.w * a;
       const double tB = tanh(gj * (B - cj));
-      const double thhat = div_seeded(tB + thj, fma(tB, thj, 1.0));  // M_{tau2}(theta^t; p^{eta_{t+1}}(nubar^{t+1}))
+      const double thhat = (tB + thj) / fma(tB, thj, 1.0);  // M_{tau2}(theta^t; p^{eta_{t+1}}(nubar^{t+1}))
       thn = fmin(fmax(thhat, -k.clipb), k.clipb);                    // tclip
       w.theta[cur ^ 1][j] = thn;
     }

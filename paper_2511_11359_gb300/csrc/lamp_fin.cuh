@@ -14,19 +14,6 @@ __device__ __forceinline__ double warp_sum_d(double v) {
   return v;
 }
 
-// a / b, b within float32's normal range: a float32 reciprocal, one Newton step (2^-46), and
-// the quotient corrected by its exact remainder: 5 float64 operations instead of the 9 of a
-// division.  The error before the last rounding is ~2^-93 of the quotient, so the result is
-// the correctly rounded one except where the quotient lies that close to a rounding boundary.
-__device__ __forceinline__ double div_seeded(double a, double b) {
-  float yf;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(yf) : "f"((float)b));
-  const double y0 = (double)yf;
-  const double y = fma(y0, fma(-b, y0, 1.0), y0);
-  const double q = a * y;
-  return fma(fma(-q, b, a), y, q);
-}
-
 // nearest multiple of the power of two g, ties to even: adding and subtracting 1.5 2^52 g
 // rounds |x| < 2^51 g there (two operations; the explicit roundings keep x's product unfused)
 __device__ __forceinline__ double quantize_add(double x, double g) {
