@@ -273,7 +273,7 @@ static int prime(lamp_ctx* ctx, double kappa, int cur) {
   if (ctx->k.shared_shift && kappa == 0.0) {
     // the start of Alg. 2 (eta_0 = infinity): stream A's exponents -kappa (C_ij + 2K nu_j) are all
     // zero, so every row maximum is, and stream B takes stream A's shift: no pass over the entries
-    // (2^18 points: 31.4 ms, 2^15 on tensor cores: 0.18 ms)
+    // (2^18 points: 15.2 ms, 2^15 on tensor cores: 0.18 ms)
     CK(cudaMemsetAsync(ctx->w.rowshift[cur], 0, ctx->k.n * sizeof(float2), ctx->stream));
     return LAMP_OK;
   }
@@ -655,11 +655,13 @@ extern "C" int lamp_create_owned(lamp_ctx** out, const lamp_problem* prob, const
   return create_impl(out, prob, params, stream, true);
 }
 
-// `passes` iterations' kernels on the context's stream, as graphs of kUnitPasses iterations:
-// launched one by one the kernels of a small problem wait for the host (2.5 us between kernels
-// against 0.7 us in a graph; 1024 points: 35 us per iteration of which 25 us are work).  Longer
-// graphs gain nothing (1500 points, 3000 iterations: 66.0 ms with graphs of 100, 65.9 ms with
-// these) and take 5 us per iteration to make and release.
+// `passes` iterations' kernels on the context's stream: graphs of kUnitPasses iterations, and what is
+// left of them (so all of a shorter run) launched one by one.  In longer runs the kernels of a small
+// problem launched one by one wait for the host (2.5 us between kernels against 0.7 us in a graph; 1024
+// points: 32 us per iteration of which 22 us are work); a single iteration takes as long as a graph of
+// one did with its launch (1500 points: 31 us against 55 us with the kernels of that time).  Longer
+// graphs gain nothing (1500 points, 3000 iterations: 66.0 ms with graphs of 100, 65.9 ms with these)
+// and take 5 us per iteration to make and release.
 constexpr int64_t kUnitPasses = 10;
 static int run_passes(lamp_ctx* ctx, int64_t passes) {
   if (ctx->on_chip && passes > 0) {

@@ -352,9 +352,10 @@ k_pts_sweep(const float* __restrict__ P_out, const float* __restrict__ P_in, int
 // takes columns t + 256 q); column sweep: a CTA of 128 threads owns 256 columns (two per thread)
 // and walks a split's rows in groups of 16.  These serve stored costs whose rows are not a
 // multiple of 16 bytes apart (lamp_dense.cu streams the others).  Bound by the latency of the
-// loads at the sizes that fit the L2 and by HBM above: the next chunk's (group's) entries are
-// loaded while the current one is evaluated, and the grid is fine enough to fill the SMs.  3001 x 2777: 19.9 -> 12.3 us (rows; 8 rows per CTA, no load
-// ahead, a butterfly of five steps per sum), 20.4 -> 13.9 us (columns; 1024 columns per CTA).
+// loads at the sizes that fit the L2 and by HBM above: the row sweep loads the next chunk's entries
+// while the current one is evaluated, the column sweep the 32 entries of a thread's group at once, and
+// the grid is fine enough to fill the SMs.  3001 x 2777: 19.9 -> 12.3 us (rows; 8 rows per CTA, no
+// load ahead, a butterfly of five steps per sum), 20.4 -> 13.9 us (columns; 1024 columns per CTA).
 constexpr int kDR = 4;          // rows per CTA in the row sweep
 constexpr int kDSplitRows = 8;  // rows per tile in the choice of its splits
 constexpr int kDChunk = 1024;   // columns per CTA step (4 per thread, stride 256)
@@ -812,7 +813,8 @@ cudaError_t launch_kmax(const Inputs& in, const Consts& k, const Work& w, const 
     return dot_launch(kDotKmax, w2, k, g, st);
   }
   if (k.shared_shift) return direct_max(kDirectKmax, in, w, k, g.rows_split, st);
-  // rowmax[split][0][n] = max_j D_ij, rowmax[split][1][n] = max_j -D_ij, D = |x|^2 + |y|^2 - 2 x.y
+  // l1 and l-inf with d > 8: rowmax[split][0][n] = max_j D_ij, rowmax[split][1][n] = max_j -D_ij, D the
+  // unscaled cost
   return launch_pts<M_KMAX, 0>(in.x, in.y, k.n, k.m, k.d, io_same(w.rowshift[1], nullptr, w.colq[1]), nullptr,
                                w.rowmax, g.rows_split, w.dev, k, st);
 }
