@@ -59,13 +59,13 @@ NCU_TRAFFIC = {
     ("highdim", "bf16_tc", 32768, 64): {
         "sources": ["paper_2511_11359_gb300/csrc/lamp_tc.cu", "paper_2511_11359_gb300/csrc/lamp_tc.cuh",
                     "paper_2511_11359_gb300/csrc/lamp_async.cuh", "paper_2511_11359_gb300/csrc/lamp_common.cuh"],
-        "sha256": "92caa86dd35da0e2d36fd75273dd237ead316436807c81fe48e7d6238dcd74ba",
+        "sha256": "4363a92d91c0a0d912257da72ba69f851c8a29e0a01754db073937db1f583498",
         "row_sweep": 9203712, "col_sweep": 9990400},
     ("image_grid", "fp32", 4096, 0): {
         "sources": ["paper_2511_11359_gb300/csrc/lamp_dense.cu", "paper_2511_11359_gb300/csrc/lamp_async.cuh",
                     "paper_2511_11359_gb300/csrc/lamp_common.cuh"],
-        "sha256": "71a85ed497bf04eabc18e41ca97860370dae675b4a09e98565429335bee8906b",
-        "row_sweep": 67231488 + 82688, "col_sweep": 67252736 + 100864},
+        "sha256": "10b53f21df2ee2a5177b1049edb8737a48411aebef67a56c6f784a4a3876faf1",
+        "row_sweep": 67230464 + 186368, "col_sweep": 67253248 + 217856},
 }
 
 
